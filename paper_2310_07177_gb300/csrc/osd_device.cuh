@@ -32,6 +32,7 @@ template <> struct Elem<float> {
         r.w = __float_as_uint(fmaxf(__uint_as_float(r.w), -1e30f));
     }
     __device__ static float clamp1(float x) { return fmaxf(x, -1e30f); }
+    __device__ static void minus(const uint4& r, float m, float2* d);  // x - m of the chunk, in pairs
     __device__ static float min_raw(const uint4& r) {
         return fminf(fminf(__uint_as_float(r.x), __uint_as_float(r.y)),
                      fminf(__uint_as_float(r.z), __uint_as_float(r.w)));
@@ -49,6 +50,7 @@ template <> struct Elem<__nv_bfloat16> {
     static constexpr uint32_t kClampBits = 0xF149F149u;  // bf16 pair of -1.0e30
     __device__ static float max_raw(const uint4& r);
     __device__ static float min_raw(const uint4& r);
+    __device__ static void minus(const uint4& r, float m, float2* d);
     __device__ static void clamp_raw(uint4& r);
     __device__ static float clamp1(float x) { return fmaxf(x, __uint_as_float(0xF1490000u)); }
     __device__ static float load(const __nv_bfloat16* p) {
@@ -77,6 +79,46 @@ __device__ __forceinline__ uint4 ldg_stream(const void* p) {
     asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
     return r;
+}
+// The same through L1 (data that a neighbouring lane reads too).
+__device__ __forceinline__ uint4 ldg_nc(const void* p) {
+    uint4 r;
+    asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    return r;
+}
+// Bytes [bytes, bytes + 16) of the 32 in lo, hi (bytes < 16, uniform over a row).
+__device__ __forceinline__ uint4 shift_words(const uint4& lo, const uint4& hi, uint32_t bytes) {
+    uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    if (bytes & 8u) {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
+    }
+    if (bytes & 4u) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) w[i] = w[i + 1];
+    }
+    const uint32_t sh = 8u * (bytes & 3u);
+    return make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh),
+                      __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh));
+}
+// The 16 bytes at an address of any element alignment, as two aligned loads and
+// a funnel shift (one load where the address is aligned).  Both aligned vectors
+// have to lie within the row (shifted_inside).
+__device__ __forceinline__ uint4 ldg_shifted(const void* p) {
+    const uintptr_t addr = reinterpret_cast<uintptr_t>(p);
+    const uint32_t off = static_cast<uint32_t>(addr & 15u);
+    const uint4* base = reinterpret_cast<const uint4*>(addr - off);
+    const uint4 lo = ldg_nc(base);
+    if (off == 0) return lo;
+    return shift_words(lo, ldg_nc(base + 1), off);
+}
+// Whether the aligned vectors around entries [j, j + 16 bytes) of a row of V
+// entries lie within the row.
+template <typename In>
+__device__ __forceinline__ bool shifted_inside(const In* row, int j, int V) {
+    constexpr int kVec = 16 / sizeof(In);
+    const int off = static_cast<int>((reinterpret_cast<uintptr_t>(row + j) & 15u) / sizeof(In));
+    return off == 0 ? j + kVec <= V : (j >= off && j - off + 2 * kVec <= V);
 }
 __device__ __forceinline__ uint4 lds_v4(const void* p) {
     return *reinterpret_cast<const uint4*>(p);
@@ -148,6 +190,21 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) {
     return upk2(d);
 }
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ void Elem<float>::minus(const uint4& r, float m, float2* d) {
+    d[0] = sub2(make_float2(__uint_as_float(r.x), __uint_as_float(r.y)), f2(m));
+    d[1] = sub2(make_float2(__uint_as_float(r.z), __uint_as_float(r.w)), f2(m));
+}
+__device__ __forceinline__ void Elem<__nv_bfloat16>::minus(const uint4& r, float m, float2* d) {
+    d[0] = bf16x2_minus(r.x, m);
+    d[1] = bf16x2_minus(r.y, m);
+    d[2] = bf16x2_minus(r.z, m);
+    d[3] = bf16x2_minus(r.w, m);
+}
+// 2^(d c) of a pair of differences, c = c_hi + c_lo carried as a float pair
+__device__ __forceinline__ float2 exp2_pair(float2 d, float c_hi, float c_lo) {
+    const float2 g = fma2(d, f2(c_hi), mul2(d, f2(c_lo)));
+    return make_float2(ex2(g.x), ex2(g.y));
+}
 
 // ---------------------------------------------------------------- packed bf16 pairs
 __device__ __forceinline__ uint32_t bmax2(uint32_t a, uint32_t b) {
@@ -292,6 +349,10 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
         :: "r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
+}
+// Start `bytes` bytes at src (both multiples of 16) on their way to L2.
+__device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(src), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;

@@ -1,34 +1,32 @@
 // osd_verify.cu -- speculative-sampling verification (Section 3 and
 // Appendix A.1 of the paper; the verify step of Algorithm 1) on sm_103a.
 //
-// Two launches on the caller's stream:
+// T > 0: one launch, a thread-block cluster per sequence, each CTA owning a span of
+// the vocabulary.  The tests u_i < p_i(y_i)/q_i(y_i) run in order and the first failure
+// ends them, so the rows past it decide nothing:
 //
-//   row_stats_kernel    one CTA per (row, vocabulary slice) over all B*k draft
-//                       rows and B*(k+1) target rows: a single streaming pass of
-//                       16-byte loads computing the online max and sum of
-//                       exp((x - max)/T) of the slice (or the argmax for T = 0).
-//                       This pass reads every logit once and carries almost all
-//                       of the operation's HBM traffic.
-//   verify_finalize     (T > 0) one thread-block cluster per sequence: merges the slice
-//                       statistics, runs the k accept tests u_i < p_i(y_i)/q_i(y_i),
-//                       all at once (a is the first failure), then draws the extra token from
-//                       norm(max(0, p_a - q_a)) (or p_k when all k pass) by inverse
-//                       CDF.  Each CTA of the cluster sums the residual weights of
-//                       its part of the vocabulary per tile; the partial sums meet
-//                       through distributed shared memory as exact 64-bit fixed
-//                       point, and the CTA whose part holds u*W rescans that one
-//                       tile with an exact warp scan.
+//   verify_lazy_kernel   rounds of positions: the round's rows are streamed once, the
+//                        span statistics (max and sum of exp((x - max)/T)) meet over the
+//                        cluster by st.async, every CTA runs the round's tests, and
+//                        only a round without a failure asks for the next one's rows.
+//   verify_fused_kernel  small batches, where latency costs more than bytes: all 2k + 1
+//                        rows staged in shared memory, one round.
 //
-//   verify_greedy       (T = 0) one warp per sequence: the argmax of every target
-//                       row from its slices, the matches in order, the target
-//                       argmax at the first mismatch.
+// The extra token is then drawn from norm(max(0, p_a - q_a)) (or p_k when all k
+// pass) by inverse CDF: each CTA sums the residual weights of its span per
+// sub-tile, the span totals meet as exact 64-bit fixed point, and the CTA whose
+// span holds u*W rescans that one sub-tile exactly.
+//
+// T = 0: two launches, row_stats_kernel (the argmax of every target row's slices) and
+// verify_greedy_kernel, one warp per sequence: the matches in order, the target
+// argmax at the first mismatch.
 //
 // The log-ratio of the accept test is formed from differences of raw logits and
 // maxima, (t_y - m_t) - (z_y - m_z), and the ratio of the two sums, so no
 // log-sum-exp is rounded on its own.
 #include <cuda.h>
 
-#include <atomic>
+#include <algorithm>
 #include <climits>
 #include <cstdint>
 #include <mutex>
@@ -41,13 +39,14 @@
 
 namespace osd {
 
-constexpr int kFinThreads = 128;
 constexpr int kFinMaxCluster = 8;
-constexpr uint64_t kDrawWaitNs = 3000000000ull;  // bound on the wait for the pushed span totals
-constexpr int kFinMaxSub = 8192;  // sub-tiles of one CTA's vocabulary span (>= span / 32)
+constexpr uint64_t kStageWaitNs = 1000000000ull;  // bound on the wait for staged rows ...
+constexpr uint64_t kPeerWaitNs = 3000000000ull;   // ... and for the peers' statistics and totals
 constexpr int kFinUnroll = 4;     // sub-tiles of loads in flight per warp
+// Where the draw reads the rows from: shared memory, 16-byte-aligned rows in global
+// memory, or rows of any alignment there.
+constexpr int kRowsStaged = 0, kRowsAligned = 1, kRowsAny = 2;
 
-// ------------------------------------------------------------------ pass 2
 struct FinParams {
     const void* draft;
     const void* target;
@@ -57,7 +56,6 @@ struct FinParams {
     float T, c_hi, c_lo;
     const RowStat* stats;
     int n_slices;
-    long long n_draft_rows;  // B*k when draft rows have statistics, 0 for greedy
     int32_t* accepted;
     int32_t* out_tokens;
     uint8_t* mask;
@@ -141,70 +139,7 @@ struct SeqSmem {
     float zy[OSD_VERIFY_MAX_K], ty[OSD_VERIFY_MAX_K];
     int y[OSD_VERIFY_MAX_K];
     float u[OSD_VERIFY_MAX_K + 1];
-    int a;
 };
-
-// Prologue of sequence b's decision, run by every thread of a CTA of kThreads:
-// every independent global load goes out in one round (the last warp fetches
-// the draft tokens and gathers the two logits each accept test needs, the warp
-// before it the uniforms); then, once the row statistics are complete, the
-// warps merge each row's slice statistics, loading up to four rows per lane
-// before reducing.  Returns non-zero, for every thread, when a draft token
-// lies outside [0, V).
-template <typename In, int kThreads>
-__device__ __forceinline__ int seq_prologue(const FinParams& p, int b, SeqSmem& sh) {
-    using E = Elem<In>;
-    constexpr int kWarps = kThreads / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int k = p.k, V = p.V;
-    const int32_t* y = p.tokens + size_t(b) * k;
-    const In* draft = static_cast<const In*>(p.draft);
-    const In* target = static_cast<const In*>(p.target);
-    int bad = 0;
-    if (warp == kWarps - 1) {
-        for (int i = lane; i < k; i += 32) {
-            const int t = y[i];
-            sh.y[i] = t;
-            if (t < 0 || t >= V) {
-                bad = 1;
-            } else {
-                sh.zy[i] = E::load(draft + (size_t(b) * k + i) * V + t);
-                sh.ty[i] = E::load(target + (size_t(b) * (k + 1) + i) * V + t);
-            }
-        }
-    }
-    if (warp == kWarps - 2)
-        for (int i = lane; i <= k; i += 32) sh.u[i] = p.uniforms[size_t(b) * (k + 1) + i];
-    grid_dependency_wait();  // the row statistics are complete from here on
-    const int nrows = 2 * k + 1;
-    const float ch0 = p.c_hi, cl0 = p.c_lo;
-    auto srow_of = [&](int r) -> long long {
-        return (r <= k) ? (p.n_draft_rows + (long long)b * (k + 1) + r) : ((long long)b * k + (r - k - 1));
-    };
-    for (int r0 = warp; r0 < nrows; r0 += 4 * kWarps) {
-        RowStat part[4][1];
-        bool have[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int r = r0 + q * kWarps;
-            have[q] = r < nrows && lane < p.n_slices;
-            if (have[q]) part[q][0] = p.stats[srow_of(r) * p.n_slices + lane];
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int r = r0 + q * kWarps;
-            if (r >= nrows) break;  // uniform across the warp
-            const RowStat* st = p.stats + srow_of(r) * p.n_slices;
-            auto merge = [ch0, cl0](MaxSum x, MaxSum z) { return merge_ms(x, z, ch0, cl0); };
-            MaxSum acc{kNegInf, 0.f};
-            if (have[q]) acc = MaxSum{part[q][0].m, part[q][0].s};
-            for (int sl = lane + 32; sl < p.n_slices; sl += 32) acc = merge(acc, MaxSum{st[sl].m, st[sl].s});
-            acc = warp_reduce(acc, merge);
-            if (lane == 0) { sh.m[r] = acc.m; sh.s[r] = acc.s; }
-        }
-    }
-    return __syncthreads_or(bad);
-}
 
 // Outputs of a sequence with a bad draft token (one CTA of kThreads writes them).
 template <int kThreads>
@@ -219,40 +154,84 @@ __device__ __forceinline__ void seq_write_bad(const FinParams& p, int b) {
     }
 }
 
-// The k accept tests: warp 0 runs them all at once, one position per lane, and
-// the first failing position is a (the tests after it are not decided).  Sets
-// sh.a, writes the margins of the decided positions when `margins` is set, and
-// ends on a block barrier.
-__device__ __forceinline__ void seq_accept(const FinParams& p, int b, SeqSmem& sh, bool margins) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = p.k;
-    if (warp == 0) {
-        int a = k;
-        float r_all[(OSD_VERIFY_MAX_K + 31) / 32];
+// One row's statistics from `count` <= 8 partials at x[0], x[stride], ..., merged in
+// that order: the maximum first, then the sums brought to it (all loads in flight together).
+__device__ __forceinline__ MaxSum merge_slots(const MaxSum* x, int stride, int count, float ch, float cl) {
+    MaxSum o[kFinMaxCluster];
+    float m = kNegInf, s = 0.f;
 #pragma unroll
-        for (int c = 0; c < (OSD_VERIFY_MAX_K + 31) / 32; ++c) {
-            const int i = c * 32 + lane;
-            bool fail = false;
-            r_all[c] = 0.f;
-            if (i < k) {
-                const float mt = sh.m[i], st = sh.s[i];
-                const float mz = sh.m[k + 1 + i], sz = sh.s[k + 1 + i];
-                const float D = (sh.ty[i] - mt) - (sh.zy[i] - mz);
-                r_all[c] = expf(__fdiv_rn(D, p.T)) * __fdiv_rn(sz, st);
-                fail = !(sh.u[i] < r_all[c]);
-            }
-            const unsigned f = __ballot_sync(0xffffffffu, fail);
-            if (f && a == k) a = c * 32 + __ffs(f) - 1;
-        }
-        if (margins) {
-#pragma unroll
-            for (int c = 0; c < (OSD_VERIFY_MAX_K + 31) / 32; ++c) {
-                const int i = c * 32 + lane;
-                if (i < k && i <= a) p.diag_margin[size_t(b) * k + i] = fabsf(sh.u[i] - r_all[c]);
-            }
-        }
-        if (lane == 0) sh.a = a;
+    for (int i = 0; i < kFinMaxCluster; ++i) {
+        o[i] = (i < count) ? x[i * stride] : MaxSum{kNegInf, 0.f};
+        m = fmaxf(m, o[i].m);
     }
-    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kFinMaxCluster; ++i)
+        if (o[i].m != kNegInf) s += o[i].s * ex2(mul_c(o[i].m - m, ch, cl));
+    return MaxSum{m, s};
+}
+
+// One round of accept tests, run by warp 0 of every CTA of the cluster alike:
+// positions i0 .. i0 + w - 1, a lane each, the first failing one is a.  Returns
+// a, k when the bonus position is reached without a failure, or -1 when the
+// round ends undecided; writes the margins of the decided positions when `margins`.
+__device__ __forceinline__ int seq_test(const FinParams& p, int b, const SeqSmem& sh, int i0, int w, bool margins) {
+    const int lane = threadIdx.x & 31, k = p.k;
+    for (int c = 0; c < w; c += 32) {
+        const int i = i0 + c + lane;
+        const bool test = c + lane < w && i < k;
+        float ratio = 0.f;
+        bool fail = false;
+        if (test) {
+            const float D = (sh.ty[i] - sh.m[i]) - (sh.zy[i] - sh.m[k + 1 + i]);
+            ratio = expf(__fdiv_rn(D, p.T)) * __fdiv_rn(sh.s[k + 1 + i], sh.s[i]);
+            fail = !(sh.u[i] < ratio);
+        }
+        const unsigned f = __ballot_sync(0xffffffffu, fail);
+        const int a = f ? i0 + c + __ffs(f) - 1 : k;
+        if (margins && test && i <= a) p.diag_margin[size_t(b) * k + i] = fabsf(sh.u[i] - ratio);
+        if (f) return a;
+    }
+    return i0 + w == k + 1 ? k : -1;
+}
+
+// Warp 0, after a round's span statistics (nr rows, `parts` partials each): merge
+// them, push the span's to every CTA of the cluster (slot [rank][row] of recv,
+// completing on bar), merge the cluster's and run the tests.  Every CTA merges the
+// same slots in the same order, so all decide alike.  Returns seq_test's answer,
+// or -2 when a CTA's copies (`stuck`, sent as a negative sum) or the wait gave up.
+__device__ __forceinline__ int seq_round(const FinParams& p, int b, SeqSmem& sh, const MaxSum* part, int parts,
+                                         MaxSum* recv, int stride, uint64_t* bar, uint32_t parity, int rank, int i0,
+                                         int w, int nr, bool stuck) {
+    const int lane = threadIdx.x & 31, csize = p.csize, k = p.k;
+    const float ch = p.c_hi, cl = p.c_lo;
+    for (int r = lane; r < nr; r += 32) {
+        MaxSum acc = merge_slots(part + r * parts, 1, parts, ch, cl);
+        if (stuck) acc.s = -1.f;
+        if (csize > 1) {
+            for (int d = 0; d < csize; ++d)
+                st_async_v2(map_rank(&recv[rank * stride + r], static_cast<uint32_t>(d)), make_float2(acc.m, acc.s),
+                            map_rank(bar, static_cast<uint32_t>(d)));
+        } else {
+            recv[r] = acc;
+        }
+    }
+    bool gone = false;
+    if (csize > 1) {
+        if (lane == 0) mbar_arrive_expect_tx(bar, static_cast<uint32_t>(csize * nr) * 8u);
+        gone = !mbar_wait_cluster_bounded(bar, parity, kPeerWaitNs);
+    }
+    __syncwarp();
+    if (!gone) {
+        for (int r = lane; r < nr; r += 32) {
+            for (int c = 0; c < csize; ++c) gone |= recv[c * stride + r].s < 0.f;
+            const MaxSum o = merge_slots(recv + r, stride, csize, ch, cl);
+            const int at = (r < w) ? i0 + r : k + 1 + i0 + r - w;
+            sh.m[at] = o.m;
+            sh.s[at] = o.s;
+        }
+    }
+    if (__any_sync(0xffffffffu, gone)) return -2;
+    return seq_test(p, b, sh, i0, w, rank == 0 && p.diag_margin);
 }
 
 // accepted, the accepted tokens and the -1 padding after a, the mask, and the
@@ -271,13 +250,12 @@ __device__ __forceinline__ void seq_write_outputs(const FinParams& p, int b, con
     }
 }
 
-// Shared memory of the extra token's draw (span_total is read by the other CTAs
-// of the cluster).
+// Shared memory of the extra token's draw.
 struct DrawSmem {
     unsigned long long span_total;
     unsigned long long tau, W, base;
     int owner, mode, tile;
-    // pushed span totals (the one-launch kernel): slot r from CTA r, completing on tbar
+    // pushed span totals: slot r from CTA r, completing on tbar
     unsigned long long totals[kFinMaxCluster];
     uint64_t tbar;
 };
@@ -289,41 +267,43 @@ struct DrawSmem {
 // sub-tile (fp32 in a warp, exact 64-bit fixed point beyond), the CTAs' span
 // totals meet through distributed shared memory, and the CTA whose span holds
 // tau = floor(u W) rescans that one sub-tile exactly.  Entry j of the target and
-// draft rows at position a is trow[j - off], zrow[j - off], in shared memory when
-// kSmem (a staged span) and global memory otherwise; trow_g is the whole target
-// row in global memory, for the case W = 0 (argmax of p_a).  s_sub holds at least
-// n / (32 kW) floats.  Every thread calls it.  Without kPush the totals are read
-// from the peers' shared memory after a cluster barrier, and the draw ends
-// having arrived (relaxed) at the cluster barrier, where the caller waits before
-// it exits.  With kPush (ds.tbar initialised with count 1 and visible to the
-// cluster) each CTA pushes its total by st.async into slot `rank` of every CTA's
-// ds.totals and waits on its own ds.tbar: no cluster barrier, nothing read from
-// a peer.  Returns false if that wait gave up (the draw is then not made).
-template <typename In, bool kVecPath, int kThreads, bool kSmem, bool kPush = false>
+// draft rows at position a is trow[j - off], zrow[j - off]; kMode says in which
+// memory and how aligned.  trow_g is the whole target row in global memory, for the
+// case W = 0 (argmax of p_a).  s_sub holds at least n / (32 kVec) floats.  Every thread
+// calls it.  Each CTA pushes its total by st.async into slot `rank` of every
+// CTA's ds.totals and waits on its own ds.tbar (initialised with count 1 and visible
+// to the cluster): no cluster barrier, nothing read from a peer.  Returns false if
+// that wait gave up (the draw is then not made).
+template <typename In, int kMode, int kThreads>
 __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, const SeqSmem& sh, int rank,
                                               int e0, int n, const In* trow, const In* zrow, int off,
                                               const In* trow_g, float* s_sub, DrawSmem& ds) {
     using E = Elem<In>;
-    constexpr int kW = kVecPath ? E::kVec : 1;  // entries per lane per sub-tile
+    constexpr int kW = E::kVec;  // entries per lane per sub-tile
     constexpr int kSub = 32 * kW;
     constexpr int kWarps = kThreads / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k = p.k, V = p.V;
     const bool bonus = (a == k);
     int32_t* out = p.out_tokens + size_t(b) * (k + 1);
-    // entry j of the two rows: trow[j - off], zrow[j - off], from shared memory when kSmem
-    auto ldv = [&](const In* q) { return kSmem ? lds_v4(q) : ldg_stream(q); };
-    auto ld1 = [&](const In* q) { return kSmem ? E::lds(q) : E::load(q); };
+    // kW entries from entry j of a row, and one entry; `whole`: all kW belong to this span
+    auto ldv = [&](const In* row, int j) {
+        if constexpr (kMode == kRowsStaged) return lds_v4(row + (j - off));
+        else if constexpr (kMode == kRowsAligned) return ldg_stream(row + (j - off));
+        else return ldg_shifted(row + (j - off));
+    };
+    auto ld1 = [&](const In* row, int j) {
+        return kMode == kRowsStaged ? E::lds(row + (j - off)) : E::load(row + (j - off));
+    };
+    // unaligned rows: the aligned vectors around the entries have to lie within the row
+    auto inside = [&](const In* row, int j) {
+        if constexpr (kMode != kRowsAny) return true;
+        else return shifted_inside(row, j, V);
+    };
     const float mt = sh.m[a], inv_st = 1.0f / sh.s[a];
     const float mz = bonus ? 0.f : sh.m[k + 1 + a];
     const float inv_sz = bonus ? 0.f : 1.0f / sh.s[k + 1 + a];
     const float ch = p.c_hi, cl = p.c_lo;
-    auto weight = [&](float t, float z) -> float {
-        const float pj = ex2(mul_c(t - mt, ch, cl)) * inv_st;
-        if (bonus) return pj;
-        const float qj = ex2(mul_c(z - mz, ch, cl)) * inv_sz;
-        return fmaxf(pj - qj, 0.f);
-    };
     const int nsub = (n + kSub - 1) / kSub;  // sub-tiles: one warp step of 32 x kW entries
     // raw entries of this lane in sub-tile s (slots past the span read as -inf: weight 0)
     struct Raw {
@@ -332,68 +312,73 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
     auto load_sub = [&](int s, Raw& r) {
         const int j0 = e0 + s * kSub + lane * kW;
         const int cnt = min(kW, e0 + n - j0);
-        if (kVecPath && cnt == kW) {
-            r.t = ldv(trow + (j0 - off));
-            r.z = bonus ? r.t : ldv(zrow + (j0 - off));
+        if (cnt == kW && inside(trow, j0) && (bonus || inside(zrow, j0))) {
+            r.t = ldv(trow, j0);
+            r.z = bonus ? r.t : ldv(zrow, j0);
         } else {
             float tv[kW], zv[kW];
 #pragma unroll
             for (int e = 0; e < kW; ++e) {
-                tv[e] = (e < cnt) ? ld1(trow + (j0 - off) + e) : kNegInf;
-                zv[e] = (e < cnt && !bonus) ? ld1(zrow + (j0 - off) + e) : kNegInf;
+                tv[e] = (e < cnt) ? ld1(trow, j0 + e) : kNegInf;
+                zv[e] = (e < cnt && !bonus) ? ld1(zrow, j0 + e) : kNegInf;
             }
             r.t = pack_raw<In, kW>(tv);
             r.z = pack_raw<In, kW>(zv);
         }
     };
-    // residual weights of one sub-tile slot, two entries per packed f32x2 step
-    // (the same operations as `weight`, so both passes round identically)
-    auto sub_weights = [&](const Raw& r, float* w) {
-        float tv[kW], zv[kW];
-        unpack_raw<In, kW>(r.t, tv);
-        unpack_raw<In, kW>(r.z, zv);
-        if constexpr (kW == 1) {
-            w[0] = weight(tv[0], zv[0]);
-        } else {
+    // residual weights of one sub-tile slot, in pairs (both passes take them here, so
+    // they round identically)
+    auto sub_weights = [&](const Raw& r, float2* w) {
+        float2 d[kW / 2];
+        E::minus(r.t, mt, d);
 #pragma unroll
-            for (int e = 0; e < kW; e += 2) {
-                const float2 dt = sub2(make_float2(tv[e], tv[e + 1]), f2(mt));
-                const float2 at = fma2(dt, f2(ch), mul2(dt, f2(cl)));
-                const float2 pj = mul2(make_float2(ex2(at.x), ex2(at.y)), f2(inv_st));
-                if (bonus) {
-                    w[e] = pj.x;
-                    w[e + 1] = pj.y;
-                } else {
-                    const float2 dz = sub2(make_float2(zv[e], zv[e + 1]), f2(mz));
-                    const float2 az = fma2(dz, f2(ch), mul2(dz, f2(cl)));
-                    const float2 qj = mul2(make_float2(ex2(az.x), ex2(az.y)), f2(inv_sz));
-                    const float2 df = sub2(pj, qj);
-                    w[e] = fmaxf(df.x, 0.f);
-                    w[e + 1] = fmaxf(df.y, 0.f);
-                }
+        for (int e = 0; e < kW / 2; ++e) w[e] = exp2_pair(d[e], ch, cl);
+        if (bonus) {
+#pragma unroll
+            for (int e = 0; e < kW / 2; ++e) w[e] = mul2(w[e], f2(inv_st));
+        } else {
+            E::minus(r.z, mz, d);
+#pragma unroll
+            for (int e = 0; e < kW / 2; ++e) {
+                const float2 q = mul2(exp2_pair(d[e], ch, cl), f2(-inv_sz));
+                const float2 df = fma2(w[e], f2(inv_st), q);
+                w[e] = make_float2(fmaxf(df.x, 0.f), fmaxf(df.y, 0.f));
             }
         }
     };
 
-    // pass 1: one fp32 sum per sub-tile, reduced inside the warp, no block barrier
+    // pass 1: one fp32 sum per sub-tile, no block barrier.  The kFinUnroll sums of a
+    // step are reduced over the lanes together: each exchange halves the number of
+    // sums a lane carries, 6 shuffles instead of 20, and lane l ends with the sum of
+    // sub-tile l / 8
+    static_assert(kFinUnroll == 4, "the reduction below carries four sums");
     for (int s0 = warp; s0 < nsub; s0 += kWarps * kFinUnroll) {
         Raw r[kFinUnroll];
 #pragma unroll
         for (int u = 0; u < kFinUnroll; ++u)
             if (s0 + u * kWarps < nsub) load_sub(s0 + u * kWarps, r[u]);
+        float sum[kFinUnroll];
 #pragma unroll
         for (int u = 0; u < kFinUnroll; ++u) {
-            const int s = s0 + u * kWarps;
-            if (s < nsub) {
-                float w[kW];
+            sum[u] = 0.f;
+            if (s0 + u * kWarps < nsub) {
+                float2 w[kW / 2];
                 sub_weights(r[u], w);
-                float sum = 0.f;
+                float2 s2 = w[0];
 #pragma unroll
-                for (int e = 0; e < kW; ++e) sum += w[e];
-                for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-                if (lane == 0) s_sub[s] = sum;
+                for (int e = 1; e < kW / 2; ++e) s2 = add2(s2, w[e]);
+                sum[u] = s2.x + s2.y;
             }
         }
+        const bool hi = lane & 16, mid = lane & 8;
+        float s01 = hi ? sum[2] : sum[0], s23 = hi ? sum[3] : sum[1];
+        s01 += __shfl_xor_sync(0xffffffffu, hi ? sum[0] : sum[2], 16);
+        s23 += __shfl_xor_sync(0xffffffffu, hi ? sum[1] : sum[3], 16);
+        float tot = mid ? s23 : s01;
+        tot += __shfl_xor_sync(0xffffffffu, mid ? s01 : s23, 8);
+        for (int o = 4; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        const int s = s0 + (lane >> 3) * kWarps;
+        if ((lane & 7) == 0 && s < nsub) s_sub[s] = tot;
     }
     __syncthreads();
     // span total, exact, reduced across warp 0
@@ -403,25 +388,22 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
         for (int s2 = lane; s2 < nsub; s2 += 32) part += fix_of(s_sub[s2]);
         part = warp_sum_u64(part);
         if (lane == 0) ds.span_total = part;
-        if (kPush && p.csize > 1) {
+        if (p.csize > 1) {
             if (lane < p.csize)
                 st_async_u64(map_rank(&ds.totals[rank], static_cast<uint32_t>(lane)), part,
                              map_rank(&ds.tbar, static_cast<uint32_t>(lane)));
             if (lane == 0) mbar_arrive_expect_tx(&ds.tbar, static_cast<uint32_t>(p.csize) * 8u);
-            got = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&ds.tbar, 0, kDrawWaitNs));
+            got = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&ds.tbar, 0, kPeerWaitNs));
         }
     }
-    if (!kPush && p.csize > 1) cluster_sync_publish(tid == 0); else __syncthreads();
+    __syncthreads();
 
     // warp 0 of every CTA derives W, tau = floor(u W) and the owning CTA identically:
     // lane r holds CTA r's total, a warp scan gives the prefix in rank order
     if (warp == 0 && got) {
         const float u = sh.u[k];
         unsigned long long tot = 0ull;
-        if (lane < p.csize) {
-            if (kPush) tot = (p.csize > 1) ? ds.totals[lane] : ds.span_total;
-            else tot = (lane == rank) ? ds.span_total : ld_dsmem_u64(map_rank(&ds.span_total, lane));
-        }
+        if (lane < p.csize) tot = (p.csize > 1) ? ds.totals[lane] : ds.span_total;
         const unsigned long long incl = warp_incl_scan_u64(tot);
         const unsigned long long W = __shfl_sync(0xffffffffu, incl, 31);
         const unsigned long long tau = fix_scale(u, W);
@@ -480,7 +462,6 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
     }
     if (warp == 0 && lane == 0 && !got) ds.owner = -1;
     __syncthreads();
-    if (!kPush && p.csize > 1) cluster_arrive_relaxed();  // done reading the other CTAs' shared memory
     if (ds.owner < 0) return false;
 
     if (rank == ds.owner && warp == 0) {
@@ -492,7 +473,13 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
                 Raw r;
                 if (s >= 0) load_sub(s, r);
                 else { r.t = ninf_raw<In>(); r.z = r.t; }
-                sub_weights(r, w);
+                float2 w2[kW / 2];
+                sub_weights(r, w2);
+#pragma unroll
+                for (int e = 0; e < kW / 2; ++e) {
+                    w[2 * e] = w2[e].x;
+                    w[2 * e + 1] = w2[e].y;
+                }
             }
             const int j0 = e0 + max(s, 0) * kSub + lane * kW;
             bool done = false;
@@ -554,75 +541,292 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
     return true;
 }
 
-template <typename In, bool kVecPath>
-__global__ void __launch_bounds__(kFinThreads) verify_finalize_kernel(FinParams p) {
+// ------------------------------------------------------------------ rows on demand (T > 0)
+// The tests run in order and nothing past the first failure is decided, so the
+// rows past it are never needed.  One thread-block cluster per sequence walks the
+// positions in rounds: its CTAs, each owning a span of the vocabulary, stream the
+// round's rows once (warps shared out over the rows), exchange the span statistics
+// by st.async, and every CTA merges the same slots in rank order and runs the
+// round's accept tests, so all decide alike without a further exchange.  An
+// accepted round doubles the next one's positions.  At the first failure (or after
+// the bonus row) the cluster draws the extra token from rows that L2 mostly still
+// holds.
+//
+// What bounds it: with a poor draft at B = 256, k = 8, V = 128256 (0.13 accepted) the two
+// rows a sequence needs are 148 MB, 22 us at the copy bandwidth, of which it takes
+// 76 us (all rows in two launches: 211 us), 50 % issue activity, the rest waits of the
+// dependent phases (statistics, exchange, draw); the same batch with 2.8 accepted takes
+// 153 us (211), with 6.8, where nearly every row is read, 218 us (208).  64 registers and four
+// CTAs an SM with groups of 4 vectors in flight measured best (groups of 2 with five or six
+// CTAs: 84 us); staging the first position in shared memory at these sizes, three CTAs an
+// SM, gave 70 us with the poor draft and 257 us with the good one, whose rounds then wait
+// for their copies.
+constexpr int kLazyMaxWin = 4;               // positions per round ...
+constexpr int kLazyMaxRows = 2 * kLazyMaxWin;  // ... two rows each
+constexpr int kLazyUnroll = 4;               // 16-byte vectors per lane per group (one group in flight ahead)
+constexpr int kLazyThreads = 256;
+constexpr int kStagedThreads = 512;          // with a staged first round: one CTA an SM
+constexpr size_t kStageMaxSmem = 200 * 1024;  // dynamic shared memory per CTA of the staging kernels
+
+// Max and sum of 2^((x - max) c) of chunks [c0, c1) of a staged row, by one warp: the
+// maximum first, then the sum against it.
+template <typename In>
+__device__ __forceinline__ MaxSum staged_stats(const In* row, int c0, int c1, float ch, float cl) {
+    using E = Elem<In>;
+    constexpr int kVec = E::kVec;
+    const int lane = threadIdx.x & 31;
+    float m = kNegInf;
+    for (int c = c0 + lane; c < c1; c += 32) m = fmaxf(m, E::max_raw(lds_v4(row + c * kVec)));
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    float2 s2 = f2(0.f);
+    if (m != kNegInf) {
+        for (int c = c0 + lane; c < c1; c += 32) {
+            float2 d[kVec / 2];
+            E::minus(lds_v4(row + c * kVec), m, d);
+#pragma unroll
+            for (int e = 0; e < kVec / 2; ++e) s2 = add2(s2, exp2_pair(d[e], ch, cl));
+        }
+    }
+    float s = s2.x + s2.y;
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    return MaxSum{m, s};
+}
+
+// Max and sum of 2^((x - max) c) of the entries p[0, n), taken by `parts` warps:
+// this one, number `part`, takes every parts-th group of 32 vectors (part 0 also the
+// entries before the first 16-byte boundary, the last part those after the last).
+template <typename In>
+__device__ __forceinline__ MaxSum span_stats(const In* p, int n, int part, int parts, float c_hi, float c_lo) {
+    using E = Elem<In>;
+    constexpr int kVec = E::kVec;
+    const int lane = threadIdx.x & 31;
+    int head = static_cast<int>(((16u - (reinterpret_cast<uintptr_t>(p) & 15u)) & 15u) / sizeof(In));
+    if (head > n) head = n;
+    const int nvec = (n - head) / kVec;
+    const int tail0 = head + nvec * kVec;
+    const In* body = p + head;
+    float m = kNegInf;
+    float2 s2 = f2(0.f);
+    auto raise_max = [&](float cm) {
+        if (cm > m) {
+            s2 = (m == kNegInf) ? f2(0.f) : mul2(s2, f2(ex2(mul_c(m - cm, c_hi, c_lo))));
+            m = cm;
+        }
+    };
+    auto one = [&](float x) {
+        raise_max(x);
+        if (m != kNegInf) s2.x += ex2(mul_c(x - m, c_hi, c_lo));
+    };
+    const int step = 32 * parts;
+    auto load_group = [&](int v, uint4* r) {
+#pragma unroll
+        for (int u = 0; u < kLazyUnroll; ++u) {
+            const int vv = v + u * step;
+            r[u] = (vv < nvec) ? ldg_stream(body + size_t(vv) * kVec) : ninf_raw<In>();
+        }
+    };
+    auto absorb = [&](const uint4* r) {
+        float cm = E::max_raw(r[0]);
+#pragma unroll
+        for (int u = 1; u < kLazyUnroll; ++u) cm = fmaxf(cm, E::max_raw(r[u]));
+        raise_max(cm);
+        if (m != kNegInf) {
+#pragma unroll
+            for (int u = 0; u < kLazyUnroll; ++u) {
+                float2 d[kVec / 2];
+                E::minus(r[u], m, d);  // exact, as is c = c_hi + c_lo
+#pragma unroll
+                for (int e = 0; e < kVec / 2; ++e) s2 = add2(s2, exp2_pair(d[e], c_hi, c_lo));
+            }
+        }
+    };
+    // two groups in turn, the next one's loads out before this one's sums
+    uint4 ra[kLazyUnroll], rb[kLazyUnroll];
+    const int stride = kLazyUnroll * step;
+    int v = part * 32 + lane;
+    if (v < nvec) load_group(v, ra);
+    if (part == 0 && lane < head) one(E::load(p + lane));
+    if (part == parts - 1 && lane < n - tail0) one(E::load(p + tail0 + lane));
+    for (; v < nvec; v += 2 * stride) {
+        if (v + stride < nvec) load_group(v + stride, rb);
+        absorb(ra);
+        if (v + stride >= nvec) break;
+        if (v + 2 * stride < nvec) load_group(v + 2 * stride, ra);
+        absorb(rb);
+    }
+    // warp merge: the maximum first, then one rescale per lane and a plain sum
+    float wm = m;
+    for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
+    float s = (m == kNegInf) ? 0.f : (s2.x + s2.y) * ex2(mul_c(m - wm, c_hi, c_lo));
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return MaxSum{wm, s};
+}
+
+// Byte offset of the sub-tile sums in the kernel's dynamic shared memory: after the
+// staged rows of the first round (none when kStaged is off).
+__host__ __device__ inline size_t lazy_sub_offset(int nslots, int span, size_t es) {
+    return (size_t(nslots) * span * es + 15) / 16 * 16;
+}
+
+// kStaged (16-byte-aligned rows): the first round's rows are bulk-copied to shared memory,
+// and a draw at one of its positions, the usual one with a draft that is often wrong,
+// reads them there.
+template <typename In, bool kStaged, bool kAligned>
+__global__ void __launch_bounds__(kStaged ? kStagedThreads : kLazyThreads, kStaged ? 1 : 4)
+verify_lazy_kernel(FinParams p, int win, int ahead) {
+    static_assert(kAligned || !kStaged, "bulk copies want 16-byte-aligned rows");
+    using E = Elem<In>;
+    constexpr int kVec = E::kVec;
+    constexpr int kThreads = kStaged ? kStagedThreads : kLazyThreads, kWarps = kThreads / 32;
     __shared__ SeqSmem sh;
-    extern __shared__ float s_sub[];  // one residual sum per sub-tile of this CTA's span
-    // residual masses in exact 64-bit fixed point (fix_of): a dependent fp64 add is slow here
     __shared__ DrawSmem ds;
+    __shared__ MaxSum s_part[kWarps];
+    __shared__ __align__(8) MaxSum s_recv[2][kFinMaxCluster * kLazyMaxRows];  // [CTA][row], two rounds
+    __shared__ __align__(8) uint64_t s_bar[2];
+    __shared__ __align__(8) uint64_t s_rbar[kLazyMaxRows];  // staged rows
+    __shared__ int s_dec;  // first failing position, k after the bonus row, -1 undecided, -2 a wait gave up
+    extern __shared__ __align__(128) unsigned char lsm[];
 
-    const int rank = (p.csize > 1) ? static_cast<int>(cluster_rank()) : 0;
-    const int b = blockIdx.x / p.csize;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int csize = p.csize;
+    const int rank = (csize > 1) ? static_cast<int>(cluster_rank()) : 0;
+    const int b = blockIdx.x / csize;
     const int k = p.k, V = p.V;
-    const In* draft = static_cast<const In*>(p.draft);
-    const In* target = static_cast<const In*>(p.target);
+    const int e0 = rank * p.span;
+    const int n = min(p.span, V - e0);
+    const In* draft = static_cast<const In*>(p.draft) + size_t(b) * k * V;
+    const In* target = static_cast<const In*>(p.target) + size_t(b) * (k + 1) * V;
+    const float ch = p.c_hi, cl = p.c_lo;
+    In* staged = reinterpret_cast<In*>(lsm);
+    float* s_sub = reinterpret_cast<float*>(lsm + (kStaged ? lazy_sub_offset(2 * win, p.span, sizeof(In)) : 0));
+    const int w0 = min(win, k + 1);  // positions of the first round
+    // row q of the round of w positions from i0: the target rows first, then the draft rows
+    // (the bonus position k has none)
+    auto row_of = [&](int i0, int w, int q) {
+        return ((q < w) ? target + size_t(i0 + q) * V : draft + size_t(i0 + q - w) * V) + e0;
+    };
+    auto rows_of = [&](int i0, int w) { return 2 * w - (i0 + w == k + 1 ? 1 : 0); };
 
-    const int bad = seq_prologue<In, kFinThreads>(p, b, sh);
-    if (bad) {  // uniform over the cluster, before any distributed shared memory access
-        if (rank == 0) seq_write_bad<kFinThreads>(p, b);
+    if (tid == 0) {
+        mbar_init_only(&s_bar[0], 1);
+        mbar_init_only(&s_bar[1], 1);
+        mbar_init_only(&ds.tbar, 1);
+        if constexpr (kStaged)
+            for (int q = 0; q < kLazyMaxRows; ++q) mbar_init_only(&s_rbar[q], 1);
+        fence_mbarrier_init();
+        if constexpr (kStaged) {
+            const uint32_t bytes = static_cast<uint32_t>(n * sizeof(In));  // a multiple of 16 on this path
+            for (int q = 0; q < rows_of(0, w0); ++q) {
+                mbar_arrive_expect_tx(&s_rbar[q], bytes);
+                bulk_g2s(staged + size_t(q) * p.span, row_of(0, w0, q), bytes, &s_rbar[q]);
+            }
+            if (ahead && w0 <= k) {  // the second round's rows start on their way to L2
+                const int w1 = min(min(2 * w0, kLazyMaxWin), k + 1 - w0);
+                for (int q = 0; q < rows_of(w0, w1); ++q) bulk_prefetch_l2(row_of(w0, w1, q), bytes);
+            }
+        }
+    }
+    // the draft tokens, the two logits each accept test needs, and the uniforms
+    int bad = 0;
+    if (warp == kWarps - 1) {
+        const int32_t* y = p.tokens + size_t(b) * k;
+        for (int i = lane; i < k; i += 32) {
+            const int t = y[i];
+            sh.y[i] = t;
+            if (t < 0 || t >= V) {
+                bad = 1;
+            } else {
+                sh.zy[i] = E::load(draft + size_t(i) * V + t);
+                sh.ty[i] = E::load(target + size_t(i) * V + t);
+            }
+        }
+    }
+    if (warp == kWarps - 2)
+        for (int i = lane; i <= k; i += 32) sh.u[i] = p.uniforms[size_t(b) * (k + 1) + i];
+    __syncthreads();  // the barriers are initialised before anyone waits on them
+    // ... and before any peer pushes to them: arrive now, wait before the first push
+    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+
+    int a = -1, i0 = 0, w = w0;
+    unsigned round = 0;
+    bool stuck = false;  // a staging copy gave up in this CTA
+    for (;;) {
+        const int nr = rows_of(i0, w);
+        const int parts = max(1, kWarps / nr);  // warps per row
+        int timed_out = 0;
+        for (int it = warp; it < nr * parts; it += kWarps) {
+            const int q = it / parts, part = it - q * parts;
+            MaxSum mine;
+            if (kStaged && round == 0) {
+                if (!mbar_wait_bounded(&s_rbar[q], 0, kStageWaitNs)) timed_out = 1;
+                const int nch = n / kVec;
+                mine = staged_stats<In>(staged + size_t(q) * p.span, nch * part / parts, nch * (part + 1) / parts, ch, cl);
+            } else {
+                mine = span_stats<In>(row_of(i0, w, q), n, part, parts, ch, cl);
+            }
+            if (lane == 0) s_part[it] = mine;
+        }
+        if (round == 0) {
+            if (__syncthreads_or(timed_out | bad)) {
+                if constexpr (kStaged)  // every copy lands, or gets a last chance to, before this CTA goes on or leaves
+                    for (int q = 0; q < nr; ++q) mbar_wait_bounded(&s_rbar[q], 0, kStageWaitNs);
+                if (__syncthreads_or(bad)) {  // uniform over the cluster, before any push to a peer
+                    if (rank == 0) seq_write_bad<kThreads>(p, b);
+                    return;
+                }
+                stuck = true;
+            }
+            if (csize > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        } else {
+            __syncthreads();
+        }
+        if (warp == 0) {
+            const int dec = seq_round(p, b, sh, s_part, parts, s_recv[round & 1u], kLazyMaxRows, &s_bar[round & 1u],
+                                      (round >> 1) & 1u, rank, i0, w, nr, stuck);
+            if (lane == 0) s_dec = dec;
+        }
+        __syncthreads();
+        a = s_dec;
+        if (a != -1) break;
+        // an accepted round makes a longer one likely to pass: twice the positions
+        i0 += w;
+        w = min(min(2 * w, kLazyMaxWin), k + 1 - i0);
+        ++round;
+    }
+    if (a < 0) {  // a row or the peers' statistics did not arrive in time: the sequence is reported as bad
+        if (csize > 1 && tid == 0) mbar_wait_cluster_bounded(&s_bar[round & 1u], (round >> 1) & 1u, kPeerWaitNs);
+        if (rank == 0) seq_write_bad<kThreads>(p, b);
         return;
     }
-    seq_accept(p, b, sh, rank == 0 && p.diag_margin);
-    const int a = sh.a;
-    if (rank == 0) seq_write_outputs<kFinThreads>(p, b, sh, a);
-
-    // ---- extra token: inverse CDF of w = max(0, p_a - q_a) (a < k) or p_k (a == k)
-    {
-        const bool bonus = (a == k);
-        const In* trow = target + (size_t(b) * (k + 1) + a) * V;
-        const In* zrow = draft + (size_t(b) * k + (bonus ? 0 : a)) * V;
-        const int e0 = rank * p.span;
-        const int n = max(0, min(p.span, V - e0));
-        residual_draw<In, kVecPath, kFinThreads, false>(p, b, a, sh, rank, e0, n, trow, zrow, 0, trow, s_sub, ds);
-    }
-    if (p.csize > 1) cluster_wait();  // keep this CTA's shared memory alive for its peers
+    if (rank == 0) seq_write_outputs<kThreads>(p, b, sh, a);
+    const In* trow = target + size_t(a) * V;
+    const In* zrow = draft + size_t(a == k ? 0 : a) * V;
+    bool drawn;
+    if (kStaged && a < w0)
+        drawn = residual_draw<In, kRowsStaged, kThreads>(p, b, a, sh, rank, e0, n, staged + size_t(a) * p.span,
+                                                         staged + size_t(a == k ? a : w0 + a) * p.span, e0, trow, s_sub, ds);
+    else
+        drawn = residual_draw<In, kAligned ? kRowsAligned : kRowsAny, kThreads>(p, b, a, sh, rank, e0, n, trow, zrow, 0,
+                                                                                trow, s_sub, ds);
+    if (!drawn) seq_write_bad<kThreads>(p, b);
 }
 
-// ------------------------------------------------------------------ one launch for small batches
-// At serving batch sizes the two launches above cost more in latency than in
-// bytes.  One thread-block cluster per sequence does both passes (T > 0): each
-// CTA bulk-copies its vocabulary span of all 2k+1 rows into shared memory,
-// computes the span's statistics of every row from there, merges them across
-// the cluster, runs the accept tests, and draws the extra token from the staged
-// rows (residual_draw) without reading them again.  The CTAs exchange the span
-// statistics and the residual totals by pushing them with st.async into every
-// peer's shared memory, each CTA waiting on its own barrier: no cluster barrier
-// after the start, no fence, and nothing read from a peer.  It runs only when
-// its grid fits in one wave (fused_shape).  At B = 32, k = 5, V = 32000 it measured 23.9 us
-// in the bench step against 27.1 us for the two launches (512 threads; 256 threads
-// 26.7 us; 16-CTA clusters 38 us).  The greedy pass (T = 0) keeps its two
-// launches: one launch over the k+1 target rows measured 11.2 against 10.3 us.
+// ------------------------------------------------------------------ every row staged (T > 0)
+// At serving batch sizes one round of latency costs more than the bytes of rows that
+// turn out not to be needed: each CTA of the sequence's cluster bulk-copies its
+// vocabulary span of all 2k + 1 rows (all the copies in flight at once, a barrier
+// per row, so that a row's statistics start as soon as it has landed), and one
+// exchange decides all the positions.  It runs only when its grid fits in one wave.
+// At B = 32, k = 5, V = 32000 it measured 23.9 us in the bench step with 512 threads
+// (256 threads 26.7 us; 16-CTA clusters 38 us).
 constexpr int kFuseThreads = 512;
-constexpr int kFuseCluster = 8;          // CTAs per sequence (above 8 needs the non-portable opt-in)
 constexpr int kFuseParts = 4;           // warp items per row for the span statistics
 constexpr int kFuseMaxB = 64;           // at most this many sequences, and the grid in one wave
-constexpr size_t kFuseMaxSmem = 200 * 1024;  // staged rows + sub-tile sums per CTA
-constexpr uint64_t kFuseWaitNs = 1000000000ull;  // bound on the wait for the staged rows
 
-// Byte offset of the one-launch kernel's receive slots in its dynamic shared
-// memory: after the staged rows and the sub-tile sums, 16-byte aligned.
+// Byte offset of the receive slots in the dynamic shared memory: after the staged
+// rows and the sub-tile sums, 16-byte aligned.
 __host__ __device__ inline size_t fused_recv_offset(int nrows, int span, size_t es) {
     return (size_t(nrows) * span * es + size_t(span / 128 + 1) * sizeof(float) + 15) / 16 * 16;
-}
-
-// Rows of sequence b staged by this CTA: local row r <= k is target row r, r > k
-// draft row r-k-1; each holds entries [e0, e0 + n) at r * span.
-template <typename In>
-__device__ __forceinline__ const In* fused_src(const FinParams& p, int b, int r, int e0) {
-    const In* draft = static_cast<const In*>(p.draft);
-    const In* target = static_cast<const In*>(p.target);
-    return (r <= p.k) ? target + (size_t(b) * (p.k + 1) + r) * p.V + e0
-                      : draft + (size_t(b) * p.k + (r - p.k - 1)) * p.V + e0;
 }
 
 template <typename In>
@@ -635,9 +839,9 @@ __global__ void __launch_bounds__(kFuseThreads) verify_fused_kernel(FinParams p)
     __shared__ __align__(8) uint64_t rbar[kMaxRows];  // one staging barrier per row
     __shared__ SeqSmem sh;
     __shared__ DrawSmem ds;
-    __shared__ MaxSum part_ms[kMaxRows * kFuseParts];
-    __shared__ __align__(8) uint64_t sbar;  // the cluster's span statistics have arrived
-    __shared__ int s_any_tmo;  // a staging copy (or a wait for the peers) gave up in the cluster
+    __shared__ MaxSum s_part[kMaxRows * kFuseParts];
+    __shared__ __align__(8) uint64_t s_bar;  // the cluster's span statistics have arrived
+    __shared__ int s_dec;  // as in verify_lazy_kernel
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int csize = p.csize;
@@ -647,36 +851,37 @@ __global__ void __launch_bounds__(kFuseThreads) verify_fused_kernel(FinParams p)
     const int nrows = 2 * k + 1;
     const int e0 = rank * p.span;
     const int n = min(p.span, V - e0);
-    In* rows = reinterpret_cast<In*>(fsm);
+    const In* draft = static_cast<const In*>(p.draft) + size_t(b) * k * V;
+    const In* target = static_cast<const In*>(p.target) + size_t(b) * (k + 1) * V;
+    In* rows = reinterpret_cast<In*>(fsm);  // row q <= k is target row q, q > k draft row q - k - 1
     float* s_sub = reinterpret_cast<float*>(fsm + size_t(nrows) * p.span * sizeof(In));
     // [csize][nrows]: CTA c's span statistics of every row, pushed by CTA c
-    MaxSum* recv_ms = reinterpret_cast<MaxSum*>(fsm + fused_recv_offset(nrows, p.span, sizeof(In)));
+    MaxSum* recv = reinterpret_cast<MaxSum*>(fsm + fused_recv_offset(nrows, p.span, sizeof(In)));
     const uint32_t bytes = static_cast<uint32_t>(n * sizeof(In));  // a multiple of 16 on this path
 
-    // ---- stage every row's span (all the copies in flight at once, a barrier per row,
-    // so that a row's statistics start as soon as it has landed)
     if (tid == 0) {
-        for (int r = 0; r < nrows; ++r) mbar_init_only(&rbar[r], 1);
-        mbar_init_only(&sbar, 1);
+        for (int q = 0; q < nrows; ++q) mbar_init_only(&rbar[q], 1);
+        mbar_init_only(&s_bar, 1);
         mbar_init_only(&ds.tbar, 1);
         fence_mbarrier_init();
-        for (int r = 0; r < nrows; ++r) {
-            mbar_arrive_expect_tx(&rbar[r], bytes);
-            bulk_g2s(rows + size_t(r) * p.span, fused_src<In>(p, b, r, e0), bytes, &rbar[r]);
+        for (int q = 0; q < nrows; ++q) {
+            mbar_arrive_expect_tx(&rbar[q], bytes);
+            bulk_g2s(rows + size_t(q) * p.span,
+                     ((q <= k) ? target + size_t(q) * V : draft + size_t(q - k - 1) * V) + e0, bytes, &rbar[q]);
         }
     }
     // meanwhile the draft tokens, the two logits each accept test needs, and the uniforms
     int bad = 0;
-    const int32_t* y = p.tokens + size_t(b) * k;
     if (warp == kWarps - 1) {
+        const int32_t* y = p.tokens + size_t(b) * k;
         for (int i = lane; i < k; i += 32) {
             const int t = y[i];
             sh.y[i] = t;
             if (t < 0 || t >= V) {
                 bad = 1;
             } else {
-                sh.zy[i] = E::load(static_cast<const In*>(p.draft) + (size_t(b) * k + i) * V + t);
-                sh.ty[i] = E::load(static_cast<const In*>(p.target) + (size_t(b) * (k + 1) + i) * V + t);
+                sh.zy[i] = E::load(draft + size_t(i) * V + t);
+                sh.ty[i] = E::load(target + size_t(i) * V + t);
             }
         }
     }
@@ -684,101 +889,47 @@ __global__ void __launch_bounds__(kFuseThreads) verify_fused_kernel(FinParams p)
         for (int i = lane; i <= k; i += 32) sh.u[i] = p.uniforms[size_t(b) * (k + 1) + i];
     __syncthreads();  // the barriers are initialised before anyone waits on them
     // ... and before any peer pushes to them: arrive now, wait before the first push
-    if (csize > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-    bad = __syncthreads_or(bad);
-    // every row's copy has landed (or its wait gave up) before this CTA leaves
-    auto wait_all = [&]() {
-        int t = 0;
-        for (int r = 0; r < nrows; ++r) t |= mbar_wait_bounded(&rbar[r], 0, kFuseWaitNs) ? 0 : 1;
-        return t;
-    };
-    if (bad) {  // uniform over the cluster, before any push to a peer
-        wait_all();
-        if (rank == 0) seq_write_bad<kFuseThreads>(p, b);
-        return;
-    }
+    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 
-    // ---- span statistics of every row: warp items (row, part), each its row's
-    // maximum first, then the sum of 2^((x - m) c) against it; then per row over the parts
+    // span statistics of every row: warp items (row, part)
     const int nch = n / kVec;
-    const float ch = p.c_hi, cl = p.c_lo;
     int timed_out = 0;
     for (int it = warp; it < nrows * kFuseParts; it += kWarps) {
-        const int r = it / kFuseParts, part = it - r * kFuseParts;
-        if (!mbar_wait_bounded(&rbar[r], 0, kFuseWaitNs)) timed_out = 1;
-        const In* row = rows + size_t(r) * p.span;
-        const int c0 = nch * part / kFuseParts, c1 = nch * (part + 1) / kFuseParts;
-        float m = kNegInf;
-        for (int c = c0 + lane; c < c1; c += 32) m = fmaxf(m, E::max_raw(lds_v4(row + c * kVec)));
-        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-        float2 s2 = f2(0.f);
-        if (m != kNegInf) {
-            for (int c = c0 + lane; c < c1; c += 32) {
-                float x[kVec];
-                E::unpack(lds_v4(row + c * kVec), x);
-#pragma unroll
-                for (int e = 0; e < kVec; e += 2) {
-                    const float2 d = sub2(make_float2(x[e], x[e + 1]), f2(m));
-                    const float2 g = fma2(d, f2(ch), mul2(d, f2(cl)));
-                    s2 = add2(s2, make_float2(ex2(g.x), ex2(g.y)));
-                }
-            }
+        const int q = it / kFuseParts, part = it - q * kFuseParts;
+        if (!mbar_wait_bounded(&rbar[q], 0, kStageWaitNs)) timed_out = 1;
+        const MaxSum mine = staged_stats<In>(rows + size_t(q) * p.span, nch * part / kFuseParts,
+                                             nch * (part + 1) / kFuseParts, p.c_hi, p.c_lo);
+        if (lane == 0) s_part[it] = mine;
+    }
+    bool stuck = false;
+    if (__syncthreads_or(timed_out | bad)) {
+        // every copy lands, or gets a last chance to, before this CTA goes on or leaves
+        for (int q = 0; q < nrows; ++q) mbar_wait_bounded(&rbar[q], 0, kStageWaitNs);
+        if (__syncthreads_or(bad)) {  // uniform over the cluster, before any push to a peer
+            if (rank == 0) seq_write_bad<kFuseThreads>(p, b);
+            return;
         }
-        float s = s2.x + s2.y;
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (lane == 0) part_ms[it] = MaxSum{m, s};
+        stuck = true;
     }
-    const int tmo = __syncthreads_or(timed_out);
-    if (tmo) wait_all();  // a copy that gave up gets a last chance to land
-    // ---- the cluster's spans: thread r < nrows merges its row's parts and pushes the
-    // result (a negative sum flags a copy that gave up) into slot `rank` of every CTA;
-    // every CTA then merges the csize slots of each row in rank order (lane c <- CTA c)
-    if (tid < nrows) {
-        MaxSum acc = part_ms[tid * kFuseParts];
-        for (int q = 1; q < kFuseParts; ++q) acc = merge_ms(acc, part_ms[tid * kFuseParts + q], ch, cl);
-        if (tmo) acc.s = -1.f;
-        if (csize > 1) {
-            asm volatile("barrier.cluster.wait.acquire;" ::: "memory");  // the peers' barriers are ready
-            for (int d = 0; d < csize; ++d)
-                st_async_v2(map_rank(&recv_ms[rank * nrows + tid], static_cast<uint32_t>(d)), make_float2(acc.m, acc.s),
-                            map_rank(&sbar, static_cast<uint32_t>(d)));
-        } else {
-            recv_ms[tid] = acc;
-        }
+    if (csize > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (warp == 0) {
+        const int dec = seq_round(p, b, sh, s_part, kFuseParts, recv, nrows, &s_bar, 0, rank, 0, k + 1, nrows, stuck);
+        if (lane == 0) s_dec = dec;
     }
-    if (csize > 1) {
-        if (tid >= nrows) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-        if (tid == 0) mbar_arrive_expect_tx(&sbar, static_cast<uint32_t>(csize * nrows) * 8u);
-    }
-    bool got = true;
-    if (csize > 1) got = mbar_wait_cluster_bounded(&sbar, 0, kFuseWaitNs); else __syncthreads();
-    got = __syncthreads_and(got);
-    int any_tmo = got ? 0 : 1;
-    for (int r = warp; r < nrows; r += kWarps) {
-        MaxSum o{kNegInf, 0.f};
-        if (lane < csize && got) o = recv_ms[lane * nrows + r];
-        if (__any_sync(0xffffffffu, o.s < 0.f)) any_tmo = 1;
-        o.s = fmaxf(o.s, 0.f);
-        o = warp_reduce(o, [ch, cl](MaxSum x, MaxSum z) { return merge_ms(x, z, ch, cl); });
-        if (lane == 0) { sh.m[r] = o.m; sh.s[r] = o.s; }
-    }
-    any_tmo = __syncthreads_or(any_tmo);
-    if (any_tmo) {  // the GPU did not deliver a row in time: the sequence is reported as bad
+    __syncthreads();
+    const int a = s_dec;
+    if (a < 0) {  // the GPU did not deliver a row in time: the sequence is reported as bad
+        if (csize > 1 && tid == 0) mbar_wait_cluster_bounded(&s_bar, 0, kPeerWaitNs);
         if (rank == 0) seq_write_bad<kFuseThreads>(p, b);
         return;
     }
-
-    seq_accept(p, b, sh, rank == 0 && p.diag_margin);
-    const int a = sh.a;
     if (rank == 0) seq_write_outputs<kFuseThreads>(p, b, sh, a);
     // ---- extra token from the staged rows at position a
-    const bool bonus = (a == k);
     const In* trow_s = rows + size_t(a) * p.span;
-    const In* zrow_s = bonus ? trow_s : rows + size_t(k + 1 + a) * p.span;
-    const In* trow_g = static_cast<const In*>(p.target) + (size_t(b) * (k + 1) + a) * V;
+    const In* zrow_s = (a == k) ? trow_s : rows + size_t(k + 1 + a) * p.span;
     // (a peer whose pushed total did not arrive in time reports the sequence as bad)
-    if (!residual_draw<In, true, kFuseThreads, true, true>(p, b, a, sh, rank, e0, n, trow_s, zrow_s, e0, trow_g,
-                                                        s_sub, ds))
+    if (!residual_draw<In, kRowsStaged, kFuseThreads>(p, b, a, sh, rank, e0, n, trow_s, zrow_s, e0,
+                                                      target + size_t(a) * V, s_sub, ds))
         seq_write_bad<kFuseThreads>(p, b);
 }
 
@@ -792,31 +943,11 @@ static int verify_slices(int B, int k, int V) {
 
 static size_t round256(size_t x) { return (x + 255) / 256 * 256; }
 
-// CTAs per sequence: up to 8 for few sequences (short spans, low latency); 4 past
-// 128 sequences, where 8 would leave more clusters than fit on the GPU at once and
-// the second wave would wait out the first one's latency phases.  A span must fit
-// in kFinMaxSub sub-tiles of `sub` entries: the element-wise path (32-entry
-// sub-tiles) takes 8 CTAs at any B once V passes 4 * 8192 * 32 = 2^20.
-static void finalize_shape(int B, int V, int sub, int* csize, int* span) {
-    int cmax = (B > 128) ? kFinMaxCluster / 2 : kFinMaxCluster;
-    const long long per_cta = (long long)kFinMaxSub * sub;
-    if ((long long)cmax * per_cta < V) cmax = kFinMaxCluster;
-    int c = (V + 4095) / 4096;
-    c = c < 1 ? 1 : (c > cmax ? cmax : c);
-    int s = (V + c - 1) / c;
-    s = (s + 63) / 64 * 64;
-    c = (V + s - 1) / s;
-    *csize = c;
-    *span = s;
-}
-
-// Resident CTAs an SM of the one-launch kernel with `smem` bytes of dynamic shared
-// memory, or 0 when a query fails.  The opt-in for that much shared memory is set
-// here first; both are kept per device for the last size asked, so repeated calls
-// (and calls under stream capture) make no runtime query.
-template <typename In>
-static int fused_ctas_per_sm(size_t smem) {
-    auto kern = verify_fused_kernel<In>;
+// Opt in for `smem` bytes of dynamic shared memory and ask how many CTAs an SM then
+// holds (0 when a query fails).  Kept per device for the last size asked, so repeated
+// calls (and calls under stream capture) make no runtime query.
+template <auto kern, int kThreads>
+static int ctas_per_sm(size_t smem) {
     static std::mutex mu;
     static size_t allowed[64] = {};
     static size_t last_smem[64] = {};
@@ -832,53 +963,73 @@ static int fused_ctas_per_sm(size_t smem) {
         allowed[dev] = smem;
     }
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kFuseThreads, smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, smem) != cudaSuccess) return 0;
     last_smem[dev] = smem;
     last_occ[dev] = occ;
     return occ;
 }
 
-// One launch for small batches: the cluster shape and shared memory, or false
-// when the rows are not 16-byte aligned, the staged rows do not fit, or the
-// grid would not fit in one wave (the two-launch path then runs).
-template <typename In>
-static bool fused_shape(int B, int k, int V, bool greedy, const void* draft, const void* target, int* csize,
-                        int* span, size_t* smem) {
-    if (greedy || B > kFuseMaxB) return false;
-    if (!aligned_to(target, 16) || !aligned_to(draft, 16) || ((size_t)V * sizeof(In)) % 16 != 0) return false;
-    int c = kFuseCluster;
+// Split V over at most c CTAs in spans of a multiple of 64 entries.
+static void split_vocab(int V, int c, FinParams* fp) {
     int s = (V + c - 1) / c;
     s = (s + 63) / 64 * 64;
-    c = (V + s - 1) / s;
-    const int nrows = 2 * k + 1;
-    const size_t bytes = fused_recv_offset(nrows, s, sizeof(In)) + size_t(c) * nrows * sizeof(MaxSum);
-    if (bytes > kFuseMaxSmem) return false;
-    // only in one wave: at B = 32, k = 5, V = 32000 (two CTAs an SM) one launch took
-    // 22.2 us against 23.2 us for two; from B = 48 on, past one wave, 34 against 26 us
-    const long long ctas = (long long)B * c;
-    if (ctas > (long long)device_sms() * fused_ctas_per_sm<In>(bytes)) return false;
-    *csize = c;
-    *span = s;
-    *smem = bytes;
-    return true;
+    fp->span = s;
+    fp->csize = (V + s - 1) / s;
 }
-// The one-launch kernel (fused_shape has set its shared-memory opt-in).
+
+// T > 0: which kernel, CTAs per sequence and positions per round.
 template <typename In>
-static cudaError_t launch_fused(const FinParams& fp, size_t smem, cudaStream_t stream) {
-    auto kern = verify_fused_kernel<In>;
-    if (kFuseCluster > 8) {
-        static std::atomic<int> nonportable[64];
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64) return cudaErrorInvalidValue;
-        if (!nonportable[dev].load(std::memory_order_relaxed)) {
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-            if (e != cudaSuccess) return e;
-            nonportable[dev].store(1, std::memory_order_relaxed);
+static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
+    const int B = fp.B, k = fp.k, V = fp.V;
+    constexpr size_t es = sizeof(In);
+    const bool aligned = aligned_to(fp.target, 16) && aligned_to(fp.draft, 16) && ((size_t)V * es) % 16 == 0;
+    if (aligned && B <= kFuseMaxB) {
+        // every row staged, only in one wave: at B = 32, k = 5, V = 32000 (two CTAs an SM) 12.8 us
+        // against 14.7 us on demand; at B = 48, past one wave, it took 34 us (17.8 on demand)
+        split_vocab(V, kFinMaxCluster, &fp);
+        const size_t smem = fused_recv_offset(2 * k + 1, fp.span, es) + size_t(fp.csize) * (2 * k + 1) * sizeof(MaxSum);
+        if (smem <= kStageMaxSmem &&
+            (long long)B * fp.csize <= (long long)device_sms() * ctas_per_sm<verify_fused_kernel<In>, kFuseThreads>(smem))
+            return from_cuda(launch(verify_fused_kernel<In>, dim3(unsigned(B) * unsigned(fp.csize)), dim3(kFuseThreads),
+                                    smem, stream, fp.csize, fp));
+    }
+    // Rows on demand.  A round costs about 2 us beside its bytes, and positions past the
+    // first failure are read for nothing: the first round takes as many positions as
+    // 200 MB hold, at most 4 (B = 256, V = 128256, 131 MB a position: 1, 76 us with a poor
+    // draft against 93 and 135 us with 2 and 4; B = 64, V = 32000, 8 MB: 4, 17.0 us against 18.0
+    // and 19.0 us with 2 and 1).
+    constexpr int sub = 32 * Elem<In>::kVec;
+    auto sub_bytes = [&]() { return size_t((fp.span + sub - 1) / sub) * sizeof(float); };
+    const double pos = double(B) * 2 * V * double(es);  // bytes of one position of the batch
+    int win = 1;
+    while (win < kLazyMaxWin && win <= k && pos * win < 100e6) win *= 2;
+    // the first round staged where the batch is at most one CTA an SM, with fewer positions
+    // where they do not fit (B = 16, k = 8, V = 128256, 2 positions: 27 us against 39 us streamed)
+    if (aligned) {
+        split_vocab(V, kFinMaxCluster, &fp);
+        for (int w = win; w >= 1 && (long long)B * fp.csize <= device_sms(); w /= 2) {
+            const size_t smem = lazy_sub_offset(2 * w, fp.span, es) + sub_bytes();
+            if (smem > kStageMaxSmem || ctas_per_sm<verify_lazy_kernel<In, true, true>, kStagedThreads>(smem) < 1) continue;
+            // so small a second round that its bytes cost nothing if the first one rejects
+            const int ahead = pos * std::min(2 * w, kLazyMaxWin) <= 9e6;
+            return from_cuda(launch(verify_lazy_kernel<In, true, true>, dim3(unsigned(B) * unsigned(fp.csize)),
+                                    dim3(kStagedThreads), smem, stream, fp.csize, fp, w, ahead));
         }
     }
-    return launch(kern, dim3(unsigned(fp.B) * unsigned(fp.csize)), dim3(kFuseThreads), smem, stream, fp.csize, fp);
+    // fewer, longer spans while three CTAs an SM remain and a position's span stays within
+    // 68 KB, so that the rows in flight stay in L2 for the draw (B = 256: V = 32000 2 CTAs a
+    // sequence, 37.9 us against 41.1 and 45.9 us with 4 and 8; V = 128256 8 CTAs, 76 us against
+    // 85 and 102 us with 4 and 2)
+    int c = kFinMaxCluster;
+    while (c > 1 && (V <= 2048 * c || ((long long)B * c / 2 >= 3LL * device_sms() && size_t(V / (c / 2)) * 2 * es <= 68 * 1024)))
+        c /= 2;
+    split_vocab(V, c, &fp);
+    if ((long long)B * fp.csize > INT_MAX) return OSD_ERR_UNSUPPORTED;
+    const dim3 grid(unsigned(B) * unsigned(fp.csize));
+    return from_cuda(aligned ? launch(verify_lazy_kernel<In, false, true>, grid, dim3(kLazyThreads), sub_bytes(), stream,
+                                      fp.csize, fp, win, 0)
+                             : launch(verify_lazy_kernel<In, false, false>, grid, dim3(kLazyThreads), sub_bytes(), stream,
+                                      fp.csize, fp, win, 0));
 }
 
 template <typename In>
@@ -888,67 +1039,29 @@ static osd_status launch_verify(const void* draft, const void* target, int B, in
                                 float* diag_margin, float* diag_gap, RowStat* stats,
                                 cudaStream_t stream) {
     const bool greedy = (T == 0.f);
-    {
-        int fc = 1, fspan = V;
-        size_t fsmem = 0;
-        if (fused_shape<In>(B, k, V, greedy, draft, target, &fc, &fspan, &fsmem)) {
-            FinParams fp = {};
-            fp.draft = draft; fp.target = target; fp.B = B; fp.k = k; fp.V = V;
-            fp.tokens = tokens; fp.uniforms = uniforms; fp.T = T;
-            split_scale(T, &fp.c_hi, &fp.c_lo);
-            fp.accepted = accepted; fp.out_tokens = out_tokens; fp.mask = mask;
-            fp.diag_margin = diag_margin; fp.diag_gap = diag_gap;
-            fp.csize = fc;
-            fp.span = fspan;
-            return from_cuda(launch_fused<In>(fp, fsmem, stream));
-        }
-    }
-    const int slice_len = verify_slice_len(B, k);
-    const int n_slices = verify_slices(B, k, V);
-    const long long n_draft_rows = greedy ? 0 : (long long)B * k;
-    const long long rows = n_draft_rows + (long long)B * (k + 1);
-    float c_hi = 0.f, c_lo = 0.f;
-    if (!greedy) split_scale(T, &c_hi, &c_lo);
-
-    const long long grid1 = rows * n_slices;
-    if (grid1 > INT_MAX) return OSD_ERR_UNSUPPORTED;
-    cudaError_t e;
-    if (greedy)
-        e = launch(row_stats_kernel<In, true>, dim3(unsigned(grid1)), dim3(kStatThreads), 0, stream, 1,
-                   static_cast<const In*>(draft), static_cast<const In*>(target), n_draft_rows, V,
-                   slice_len, n_slices, c_hi, c_lo, stats);
-    else
-        e = launch(row_stats_kernel<In, false>, dim3(unsigned(grid1)), dim3(kStatThreads), 0, stream, 1,
-                   static_cast<const In*>(draft), static_cast<const In*>(target), n_draft_rows, V,
-                   slice_len, n_slices, c_hi, c_lo, stats);
-    if (e != cudaSuccess) return OSD_ERR_CUDA;
-
-    FinParams fp;
+    FinParams fp = {};
     fp.draft = draft; fp.target = target; fp.B = B; fp.k = k; fp.V = V;
-    fp.tokens = tokens; fp.uniforms = uniforms; fp.T = T; fp.c_hi = c_hi; fp.c_lo = c_lo;
-    fp.stats = stats; fp.n_slices = n_slices; fp.n_draft_rows = n_draft_rows;
+    fp.tokens = tokens; fp.uniforms = uniforms; fp.T = T;
     fp.accepted = accepted; fp.out_tokens = out_tokens; fp.mask = mask;
     fp.diag_margin = diag_margin; fp.diag_gap = diag_gap;
     if (greedy) {
+        const int slice_len = verify_slice_len(B, k);
+        fp.n_slices = verify_slices(B, k, V);
+        fp.stats = stats;
+        const long long grid1 = (long long)B * (k + 1) * fp.n_slices;
+        if (grid1 > INT_MAX) return OSD_ERR_UNSUPPORTED;
+        const cudaError_t e =
+            launch(row_stats_kernel<In, true>, dim3(unsigned(grid1)), dim3(kStatThreads), 0, stream, 1,
+                   static_cast<const In*>(draft), static_cast<const In*>(target), 0LL, V, slice_len, fp.n_slices,
+                   0.f, 0.f, stats);
+        if (e != cudaSuccess) return OSD_ERR_CUDA;
         fp.csize = 1;
         fp.span = V;
         const dim3 grid_g(unsigned((B + kGreedyWarps - 1) / kGreedyWarps));
         return from_cuda(launch_ex(true, verify_greedy_kernel, grid_g, dim3(kGreedyWarps * 32), 0, stream, 1, fp));
     }
-    const bool vec = aligned_to(draft, 16) && aligned_to(target, 16) && ((size_t)V * sizeof(In)) % 16 == 0;
-    const int sub = 32 * (vec ? Elem<In>::kVec : 1);
-    int csize = 1, span = V;
-    finalize_shape(B, V, sub, &csize, &span);
-    fp.csize = csize;
-    fp.span = span;
-    const dim3 grid2(unsigned(B) * unsigned(csize));
-    const size_t smem2 = size_t((span + sub - 1) / sub) * sizeof(float);
-    if (smem2 > size_t(kFinMaxSub) * sizeof(float)) return OSD_ERR_UNSUPPORTED;
-    if (vec)
-        e = launch_ex(true, verify_finalize_kernel<In, true>, grid2, dim3(kFinThreads), smem2, stream, csize, fp);
-    else
-        e = launch_ex(true, verify_finalize_kernel<In, false>, grid2, dim3(kFinThreads), smem2, stream, csize, fp);
-    return from_cuda(e);
+    split_scale(T, &fp.c_hi, &fp.c_lo);
+    return launch_sampling<In>(fp, stream);
 }
 
 }  // namespace osd

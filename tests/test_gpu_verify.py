@@ -81,6 +81,36 @@ def test_verify_matches_oracle(osd, B, k, V, dtype, T):
     print(f"B={B} k={k} V={V} {dtype} T={T}: {rep}")
 
 
+# Rounds of positions read on demand: drafts near the target, so that sequences end in
+# every round, by shape of the first round, alignment and CTAs per sequence.
+ROUND_CASES = [  # (B, k, V, dtype, T, noise)
+    (64, 9, 32000, torch.bfloat16, 1.0, 0.2),    # past one wave: rounds of 4, 4 and 2 positions
+    (3, 12, 32001, torch.float32, 0.7, 0.1),     # the same on unaligned rows, a last round of the bonus row alone
+    (40, 5, 33003, torch.bfloat16, 1.0, 0.3),    # every phase of a 16-byte vector
+    (2, 9, 128256, torch.bfloat16, 1.0, 0.1),    # two positions staged, then streamed
+    (19, 3, 131072, torch.float32, 1.0, 0.2),    # one position staged, one CTA on every SM ...
+    (20, 3, 131072, torch.float32, 1.0, 0.2),    # ... and one sequence more
+    (64, 2, 400000, torch.bfloat16, 1.0, 0.2),   # one position in the first round
+    (256, 3, 4104, torch.bfloat16, 1.3, 0.3),    # two CTAs a sequence
+    (300, 2, 63, torch.bfloat16, 1.0, 0.3),      # one, and no whole warp step
+    (9, 1, 32008, torch.bfloat16, 1.0, 0.3),
+]
+
+
+@pytest.mark.parametrize("B,k,V,dtype,T,noise", ROUND_CASES)
+def test_rounds_match_oracle(osd, B, k, V, dtype, T, noise):
+    spec = W.VerifySpec(B, k, V, dtype, 2.0, 1.0, noise, T)
+    inp = W.verify_inputs(spec, seed=77 + V + k)
+    if B > 3:  # a draft token outside [0, V) marks its own sequence only
+        inp["tokens"][1, k - 1] = V
+        inp["tokens"][2, 0] = -1
+    res, ref = _run(osd, inp, T)
+    check_verify(res, ref, k, V)
+    check_margins(res, ref)
+    bad = ref["accepted"] < 0
+    np.testing.assert_array_equal(res.accepted.cpu().numpy() < 0, bad)
+
+
 GREEDY_CASES = [
     (16, 3, 1, torch.float32), (32, 4, 1001, torch.bfloat16), (9, 2, 40000, torch.float32),
     (12, 5, 32000, torch.bfloat16), (38, 7, 32768, torch.bfloat16), (7, 3, 4096, torch.bfloat16),
