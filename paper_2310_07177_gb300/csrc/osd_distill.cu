@@ -45,6 +45,7 @@ constexpr int kDistMaxClusterWide = 16;       // ... and up to 16 (non-portable 
 constexpr int kDistSpanBytes = 32768;         // target bytes of both rows per CTA
 constexpr int kDistSpanBytesJsd = 49152;      // JSD, with the most work per entry, does best with fewer, longer spans
 constexpr int kDistMaxSmem = 192 * 1024;      // largest staging buffer per CTA
+constexpr int kSpanPad = 16;                   // staged entries past a span: a head and a tail (< 12)
 constexpr float kMinNormal = 1.17549435e-38f;  // smallest normal fp32
 
 struct DistParams {
@@ -69,7 +70,8 @@ struct DistParams {
     int32_t* seq_of_row;  // nullable: seq_of_row[r] = b
     int32_t* count;       // nullable: number of active sequences
     int csize;  // CTAs per row (cluster size)
-    int span;   // vocabulary entries per CTA (multiple of 64)
+    int span;   // vocabulary entries per CTA (a multiple of 64, or of a 16-byte chunk)
+    int same_phase;  // rows off the 16-byte grid, but draft, target and gradient alike
 };
 
 // Pass-1 partial of a span: maxima, sums of 2^((x-m) log2 e) and one loss moment.
@@ -176,8 +178,8 @@ __device__ __forceinline__ float load_q(const In* zs, const In* ts, int j) {
 // q < p: both products of positive sums, so nothing cancels when one side
 // holds almost all the mass.
 template <typename In, bool kAligned, int kT>
-__device__ __forceinline__ void tvd_gradient(const In* zs, const In* ts, int n, float gpos, float gneg,
-                                             float* orow) {
+__device__ __forceinline__ void tvd_gradient(const In* zs, const In* ts, int n, const SpanMap& sm, float gpos,
+                                             float gneg, float* orow) {
     const int tid = threadIdx.x;
     auto g_of = [gpos, gneg](float q) { return q * (__float_as_int(q) < 0 ? gneg : gpos); };
     // the factor of q': gpos, or gneg where the sign bit is set (one shift and one
@@ -187,9 +189,9 @@ __device__ __forceinline__ void tvd_gradient(const In* zs, const In* ts, int n, 
         const uint32_t neg = static_cast<uint32_t>(__float_as_int(q) >> 31);
         return __uint_as_float(fpos ^ (neg & fdiff));
     };
-    if constexpr (kAligned) {
+    {
         constexpr int kVec = Elem<In>::kVec;
-        const int nv = n / kVec;
+        const int nv = kAligned ? n / kVec : sm.nv;
         for (int v = tid; v < nv; v += kT) {
             float q[kVec];
             if constexpr (sizeof(In) == 4) {
@@ -215,9 +217,11 @@ __device__ __forceinline__ void tvd_gradient(const In* zs, const In* ts, int n, 
             for (int e = 0; e < kVec; e += 4) stg_v4(orow + v * kVec + e, g[e], g[e + 1], g[e + 2], g[e + 3]);
         }
         const int r0 = nv * kVec;
-        if (tid < n - r0) orow[r0 + tid] = g_of(load_q(zs, ts, r0 + tid));
-    } else {
-        for (int e = tid; e < n; e += kT) orow[e] = g_of(load_q(zs, ts, e));
+        if constexpr (kAligned) {
+            if (tid < n - r0) orow[r0 + tid] = g_of(load_q(zs, ts, r0 + tid));
+        } else {
+            if (tid < sm.rag) orow[span_entry<In>(sm, r0 + tid) - sm.jb] = g_of(load_q(zs, ts, r0 + tid));
+        }
     }
 }
 
@@ -260,15 +264,15 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
     const int e0 = rank * p.span;
     const int n = min(p.span, V - e0);
     In* zs = reinterpret_cast<In*>(dsm);
-    In* ts = zs + p.span;
+    In* ts = zs + p.span + (kAligned ? 0 : kSpanPad);
     bool issued = false;  // accepted mode: the span's copies went out before the slot count
     if (p.accepted) {
         // sequence b = row keeps position a = accepted[b] when a < k (the first rejected
         // draft token); the output slot counts the active sequences before it
         const int b = static_cast<int>(row), a = p.accepted[b];
         const bool active = a >= 0 && a < p.k;
-        if (active) {  // the copies first: the count below runs while they are in flight
-            stage_span_issue<In, kAligned>(zs, ts, static_cast<const In*>(p.draft) + b * p.dsg + a * p.dsp + e0,
+        if (kAligned && active) {  // the copies first: the count below runs while they are in flight
+            stage_span_issue<In>(zs, ts, static_cast<const In*>(p.draft) + b * p.dsg + a * p.dsp + e0,
                                            static_cast<const In*>(p.target) + b * p.tsg + a * p.tsp + e0, n,
                                            &bar, &s_err);
             issued = true;
@@ -306,18 +310,38 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
     const In* trow = static_cast<const In*>(p.target) + g * p.tsg + pp * p.tsp;
 
     // ---- stage the span of both rows in shared memory
-    const int err_local = issued ? stage_span_land<In, kAligned, kT>(zs, ts, zrow + e0, trow + e0, n, &bar, &s_err)
-                                 : stage_span<In, kAligned, kT>(zs, ts, zrow + e0, trow + e0, n, &bar, &s_err);
+    int err_local = 0;
+    SpanMap sm{};  // rows off the 16-byte grid: this CTA's part, by the phase of the gradient's row ...
+    if constexpr (kAligned) {
+        err_local = issued ? stage_span_land<In, kT>(zs, ts, zrow + e0, trow + e0, n, &bar, &s_err)
+                           : stage_span<In, kT>(zs, ts, zrow + e0, trow + e0, n, &bar, &s_err);
+    } else if (p.same_phase) {  // ... which the logits' rows share: chunks go by bulk copy
+        sm = span_map<In, Elem<In>::kVec>(
+            rank, p.span, V, static_cast<int>((reinterpret_cast<uintptr_t>(zrow) & 15u) / sizeof(In)));
+        err_local = stage_phased<In>(zs, ts, zrow, trow, sm, &bar, &s_err);
+    } else {
+        sm = span_map<In, 4>(rank, p.span, V,
+                             static_cast<int>((reinterpret_cast<uintptr_t>(p.dlogits + row * V) >> 2) & 3u));
+        stage_shifted<In, kT>(zs, ts, zrow, trow, V, sm);
+    }
+    const int jb = kAligned ? e0 : sm.jb;  // the first chunk's entry
+    // a staged slot's entry, counted from jb
+    auto entry = [&](int i) {
+        return kAligned || i < sm.nv * Elem<In>::kVec ? i : span_entry<In>(sm, i) - sm.jb;
+    };
 
     // ---- pass 0: this thread's maxima, and the chunk where each first appears
     float mz = kNegInf, mt = kNegInf;
     int jz = -1, jt = -1;
     if (!err_local) {
-        sweep<In, kAligned, kClampZ, kClampT, true, false, kUn0, kT>(zs, ts, n, [&](const float* z, const float* t, auto tag,
+        sweep<In, kAligned, kClampZ, kClampT, true, false, kUn0, kT>(zs, ts, n, sm, [&](const float* z, const float* t, auto tag,
                                                                    int j0, float cz, float ct, bool,
                                                                    const uint4& zr, const uint4& tr) {
             if (cz > mz) { mz = cz; jz = j0; }
-            if (ct > mt) { mt = ct; jt = j0; }
+            // (CE's label is the lowest index: a head entry comes before the chunks, though visited after)
+            const bool head = kKind == OSD_CE && !kAligned && decltype(tag)::value == 1 &&
+                              j0 >= sm.nv * Elem<In>::kVec + sm.tail;
+            if (ct > mt || (head && ct == mt)) { mt = ct; jt = j0; }
             if constexpr (kClamp) {  // clamp the staged logits once, for every later pass
                 if constexpr (decltype(tag)::value > 1) {
                     *reinterpret_cast<uint4*>(zs + j0) = zr;
@@ -330,9 +354,9 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
         });
     }
     // the entry that holds a maximum: RKL's pivot target logit, CE's label
-    auto chunk_len = [n](int j0) {
+    auto chunk_len = [&](int j0) {
         constexpr int kVec = Elem<In>::kVec;
-        return (kAligned && j0 < (n / kVec) * kVec) ? kVec : 1;
+        return j0 < (kAligned ? n / kVec : sm.nv) * kVec ? kVec : 1;
     };
     float tp = 0.f;                      // RKL: target logit at this thread's draft maximum
     Label lab{kNegInf, INT_MAX, 0.f};    // CE: this thread's first target maximum
@@ -351,7 +375,7 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
 #pragma unroll
         for (int e = Elem<In>::kVec - 1; e >= 0; --e)
             if (e < cnt && Elem<In>::lds(ts + jt + e) == mt) ei = e;
-        lab = Label{mt, e0 + jt + ei, Elem<In>::lds(zs + jt + ei)};
+        lab = Label{mt, jb + entry(jt + ei), Elem<In>::lds(zs + jt + ei)};
     }
     // block maxima: every thread's sums of pass 1 then share one reference
     float gzb, gtb, tpv = 0.f;
@@ -391,7 +415,7 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
     if (!err_local) {
         const float2 gz2 = f2(gzb), gt2 = f2(gtb), tp2 = f2(tpv);
         const float2 nMz2 = f2(-Mz), nMt2 = f2(-Mt);
-        sweep<In, kAligned, false, false, false, kMoment, kUn, kT>(zs, ts, n, [&](const float* z, const float* t,
+        sweep<In, kAligned, false, false, false, kMoment, kUn, kT>(zs, ts, n, sm, [&](const float* z, const float* t,
                                                                              auto tag, int, float, float,
                                                                              bool ninf, const uint4&, const uint4&) {
             constexpr int kCnt = decltype(tag)::value;
@@ -551,7 +575,7 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
         // ---- pass 2: divergence terms with the global normalisers
         float2 A2 = f2(0.f), B2 = f2(0.f), C2 = f2(0.f);
         if (!row_err && !jsd_trivial) {
-            sweep<In, kAligned, false, false, false, false, kUn, kT>(zs, ts, n, [&](const float* z, const float* t,
+            sweep<In, kAligned, false, false, false, false, kUn, kT>(zs, ts, n, sm, [&](const float* z, const float* t,
                                                                                auto tag, int j0, float, float, bool,
                                                                                const uint4& zr, const uint4& tr) {
                 constexpr int kCnt = decltype(tag)::value;
@@ -650,15 +674,15 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
     // ---- pass 3: d loss / d draft logits of the span
     if (kKind == OSD_TVD && !row_err) {
         // from the stored q' = q sign(q - p): q' Q- / tau, or q' Q+ / tau where q' < 0
-        tvd_gradient<In, kAligned, kT>(zs, ts, n, s2.c * inv_tau, s2.b * inv_tau, p.dlogits + row * V + e0);
+        tvd_gradient<In, kAligned, kT>(zs, ts, n, sm, s2.c * inv_tau, s2.b * inv_tau, p.dlogits + row * V + jb);
     } else if (kKind != OSD_TVD && !row_err) {
-        float* orow = p.dlogits + row * V + e0;
+        float* orow = p.dlogits + row * V + jb;
         const float K = s_K, tpg = s_tp;
         // q and p of this pass come out multiplied by the gradient's constant factor
         const float2 cvs = f2(cv + p.lg_scale), cus = f2(cu + p.lg_scale);
         const int label = st.idx;
         bool own_label = false;  // CE: this thread's stores hold the label's entry
-        sweep<In, kAligned, false, false, false, false, kUn3, kT>(zs, ts, n, [&](const float* z, const float* t,
+        sweep<In, kAligned, false, false, false, false, kUn3, kT>(zs, ts, n, sm, [&](const float* z, const float* t,
                                                                             auto tag, int j0, float, float, bool,
                                                                             const uint4& zr, const uint4& tr) {
             constexpr int kCnt = decltype(tag)::value;
@@ -676,6 +700,7 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
                 if constexpr (kRaw) return bf16x2_minus(tw[e / 2], m);
                 else return sub2(make_float2(t[e], (e + 1 < kCnt) ? t[e + 1] : t[e]), f2(m));
             };
+            const int jr = kCnt > 1 ? j0 : entry(j0);
             float gr[kCnt];
 #pragma unroll
             for (int e = 0; e < kCnt; e += 2) {
@@ -688,7 +713,7 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
                     const float2 u = fma2(tdiff(e, st.mt), f2(c), cus);
                     gg = sub2(qj, make_float2(ex2(u.x), ex2(u.y)));
                 } else if (kKind == OSD_CE) {  // (q - onehot(y*)) / tau
-                    const int j = e0 + j0 + e;
+                    const int j = jb + jr + e;
                     const bool lx = (j == label), ly = (j + 1 == label);
                     own_label |= lx || (two && ly);
                     gg = sub2(qj, make_float2(lx ? inv_tau : 0.f, ly ? inv_tau : 0.f));
@@ -715,19 +740,19 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
                 gr[e] = gg.x;
                 if (two) gr[e + 1] = gg.y;
             }
-            if constexpr (kAligned && kCnt >= 4) {
+            if constexpr (kCnt >= 4) {
 #pragma unroll
-                for (int e = 0; e < kCnt; e += 4) stg_v4(orow + j0 + e, gr[e], gr[e + 1], gr[e + 2], gr[e + 3]);
+                for (int e = 0; e < kCnt; e += 4) stg_v4(orow + jr + e, gr[e], gr[e + 1], gr[e + 2], gr[e + 3]);
             } else {
 #pragma unroll
-                for (int e = 0; e < kCnt; ++e) orow[j0 + e] = gr[e];
+                for (int e = 0; e < kCnt; ++e) orow[jr + e] = gr[e];
             }
         });
         // CE: at the label q / tau - 1 / tau keeps only the resolution of 1 / tau (an ulp
         // of 1.43 at tau = 0.7, where q is near 1); the thread that stored the entry writes
         // it again as (q - 1) / tau, with q - 1 exact (a CTA barrier before a write by one
         // fixed thread cost CE 6 %)
-        if (kKind == OSD_CE && own_label) orow[label - e0] = (ex2(fmaf(st.zy - st.mz, c, cv)) - 1.f) * inv_tau;
+        if (kKind == OSD_CE && own_label) orow[label - jb] = (ex2(fmaf(st.zy - st.mz, c, cv)) - 1.f) * inv_tau;
     }
     if (csize > 1) cluster_wait();  // keep this CTA's statistics readable until every peer is done
 }
@@ -769,12 +794,13 @@ struct TmShape {
 
 // This thread's chunks of a span held in tensor memory: slot s is chunk
 // v = tid + kTmThreads s (entries v kVec ..), its draft words in columns
-// 4s .. 4s+3 and its target words in t_off + 4s ..; then the ragged tail of
-// fewer than kVec entries, one per thread tid < tail, kept in that thread's
-// registers (tz, tt).  f is `sweep`'s callback, with the chunk's packed words by
+// 4s .. 4s+3 and its target words in t_off + 4s ..; then the single entries, one per
+// thread tid < tail, kept in that thread's registers (tz, tt); rj(): that entry,
+// counted from the first chunk's.  f is `sweep`'s callback, with the chunk's packed words by
 // reference: kStore writes them back.
-template <typename In, bool kClampZ, bool kClampT, bool kMax, bool kMin, bool kStore, int kG = kTmG, typename F>
-__device__ __forceinline__ void sweep_tm(uint32_t tw, const TmShape& sh, int nv, int tail, float& tz, float& tt,
+template <typename In, bool kClampZ, bool kClampT, bool kMax, bool kMin, bool kStore, int kG = kTmG, typename R,
+          typename F>
+__device__ __forceinline__ void sweep_tm(uint32_t tw, const TmShape& sh, int nv, int tail, R&& rj, float& tz, float& tt,
                                          F&& f) {
     static_assert(kG == 1 || kG == kTmG, "one or kTmG chunk slots per round");
     using E = Elem<In>;
@@ -818,7 +844,7 @@ __device__ __forceinline__ void sweep_tm(uint32_t tw, const TmShape& sh, int nv,
         if (kClampZ) z = E::clamp1(z);
         if (kClampT) t = E::clamp1(t);
         uint4 dz{}, dt{};
-        f(&z, &t, std::integral_constant<int, 1>{}, nv * kVec + tid, z, t, fminf(z, t) == kNegInf, dz, dt);
+        f(&z, &t, std::integral_constant<int, 1>{}, rj(), z, t, fminf(z, t) == kNegInf, dz, dt);
         if constexpr (kStore) { tz = z; tt = t; }
     }
 }
@@ -914,7 +940,7 @@ __device__ __forceinline__ void named_sync(int id) {
 constexpr int kTmNinf = 1;    // some logit is -inf
 constexpr int kTmRklInf = 2;  // a finite draft logit meets a -inf target logit: the loss is +inf
 
-template <typename In, int kKind>
+template <typename In, int kKind, bool kAnyPhase>
 __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p, TmShape tsh) {
     static_assert(kKind == OSD_TVD || kKind == OSD_JSD || kKind == OSD_RKL || kKind == OSD_FKL,
                   "the TMEM-staged runs serve TVD, JSD, RKL and FKL");
@@ -949,10 +975,17 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
     const int cid = blockIdx.x / csize;
     const long long rows = static_cast<long long>(p.G) * p.P;
     const int V = p.V;
-    const int e0 = rank * p.span;
-    const int n = min(p.span, V - e0);
-    const int nv = n / kVec, tail0 = nv * kVec, tail = n - tail0;
+    // this CTA's part of a row, `e0` its first chunk's entry and `tail` its single entries:
+    // of every row alike on 16-byte-aligned rows; with kAnyPhase by the row's phase (its
+    // first entry's place in a 16-byte vector), head entries among the single ones
+    int e0 = rank * p.span;
+    const int n = kAnyPhase ? 0 : min(p.span, V - e0);
+    int nv = n / kVec, tail = n - nv * kVec;
+    const int tail0 = nv * kVec;
     const uint32_t bytes = static_cast<uint32_t>(tail0 * sizeof(In));
+    [[maybe_unused]] SpanMap sm{};     // kAnyPhase: of the row being processed ...
+    [[maybe_unused]] int nphase = 0;  // ... and the phase of the row in flight
+    auto rj = [&]() { return kAnyPhase ? span_entry<In>(sm, nv * kVec + threadIdx.x) - sm.jb : nv * kVec + int(threadIdx.x); };
     In* zs = reinterpret_cast<In*>(dsm);
     In* ts = zs + p.span;
     float4* recv1 = reinterpret_cast<float4*>(ts + p.span);  // [csize] CTA partials of the first exchange
@@ -1026,6 +1059,26 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
     // the bulk copies of a row's span (tid 0, when `copy`) and its tail entries
     auto issue = [&](long long row, bool copy) {
         const long long g = row / p.P, pp = row - g * p.P;
+        if constexpr (kAnyPhase) {
+            const In* zrow = static_cast<const In*>(p.draft) + g * p.dsg + pp * p.dsp;
+            const In* trow = static_cast<const In*>(p.target) + g * p.tsg + pp * p.tsp;
+            nphase = static_cast<int>((reinterpret_cast<uintptr_t>(zrow) & 15u) / sizeof(In));
+            const SpanMap m = span_map<In, kVec>(rank, p.span, V, nphase);
+            if (tid == 0 && copy) {  // (a part without chunks still completes its phase)
+                fence_proxy_async_smem();  // this CTA's reads of the staging buffer come first
+                mbar_arrive_expect_tx(&bar, static_cast<uint32_t>(m.nv) * 32u);
+                if (m.nv) {
+                    bulk_g2s(zs, zrow + m.jb, static_cast<uint32_t>(m.nv) * 16u, &bar);
+                    bulk_g2s(ts, trow + m.jb, static_cast<uint32_t>(m.nv) * 16u, &bar);
+                }
+            }
+            if (tid < m.rag) {
+                const int j = span_entry<In>(m, m.nv * kVec + tid);
+                nz = Elem<In>::load(zrow + j);
+                nt = Elem<In>::load(trow + j);
+            }
+            return;
+        }
         const In* zsrc = static_cast<const In*>(p.draft) + g * p.dsg + pp * p.dsp + e0;
         const In* tsrc = static_cast<const In*>(p.target) + g * p.tsg + pp * p.tsp + e0;
         if (tid == 0 && bytes && copy) {
@@ -1085,7 +1138,13 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
         // pass 0 on the way (this thread's maxima), TVD and JSD the maxima of this
         // thread's first chunk (JSD clamps the logits first, and tensor memory keeps the
         // clamped words)
-        const bool landed = !bytes || mbar_wait_bounded(&bar, phase, kStageWaitNs);
+        if constexpr (kAnyPhase) {
+            sm = span_map<In, kVec>(rank, p.span, V, nphase);
+            e0 = sm.jb;
+            nv = sm.nv;
+            tail = sm.rag;
+        }
+        const bool landed = (!kAnyPhase && !bytes) || mbar_wait_bounded(&bar, phase, kStageWaitNs);
         if (tid == 0 && landed) pending = false;
         float mz = kNegInf, mt = kNegInf, tp = kNegInf;
         [[maybe_unused]] uint4 pz = make_uint4(0u, 0u, 0u, 0u), pt = pz;
@@ -1136,7 +1195,7 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
             // ---- pass 0 (RKL): this warp's maxima; the raw words of the chunk that first
             // raised this thread's draft maximum, or the tail entry's target logit, are
             // kept and scanned for the pivot once the pass is done
-            sweep_tm<In, false, false, true, false, false>(tw, tsh, nv, tail, tz, tt,
+            sweep_tm<In, false, false, true, false, false>(tw, tsh, nv, tail, rj, tz, tt,
                 [&](const float*, const float* t, auto tag, int, float cz, float ct, bool, uint4& zr, uint4& tr) {
                     constexpr int kCnt = decltype(tag)::value;
                     if (cz > mz) {
@@ -1185,7 +1244,7 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                 Ez2 = f2(0.f);
                 Et2 = f2(0.f);
                 const float Mz = mz == kNegInf ? 0.f : __fmul_rn(mz, c), Mt = mt == kNegInf ? 0.f : __fmul_rn(mt, c);
-                sweep_tm<In, false, false, false, false, false>(tw, tsh, nv, tail, tz, tt,
+                sweep_tm<In, false, false, false, false, false>(tw, tsh, nv, tail, rj, tz, tt,
                     [&](const float* z, const float* t, auto tag, int, float, float, bool, uint4& zr, uint4& tr) {
                         constexpr int kCnt = decltype(tag)::value;
                         // JSD's bf16 chunks take x - m straight from the packed words (the
@@ -1223,7 +1282,7 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                                             (mt == kNegInf && st != 0.f))) {
                 mz = kNegInf;
                 mt = kNegInf;
-                sweep_tm<In, false, false, true, false, false>(tw, tsh, nv, tail, tz, tt,
+                sweep_tm<In, false, false, true, false, false>(tw, tsh, nv, tail, rj, tz, tt,
                     [&](const float*, const float*, auto, int, float cz, float ct, bool, uint4&, uint4&) {
                         mz = fmaxf(mz, cz);
                         mt = fmaxf(mt, ct);
@@ -1268,7 +1327,7 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                 // place of the chunk's logits) and Q = sum q; JSD: KL(p||m) and KL(q||m) in bits
                 float2 A2 = f2(0.f), B2 = f2(0.f), C2 = f2(0.f);
                 if (!jsd_trivial) {
-                    sweep_tm<In, false, false, false, false, kTvd, kJsd ? kTmJsdG : kTmG>(tw, tsh, nv, tail, tz, tt,
+                    sweep_tm<In, false, false, false, false, kTvd, kJsd ? kTmJsdG : kTmG>(tw, tsh, nv, tail, rj, tz, tt,
                         [&](const float* z, const float* t, auto tag, int, float, float, bool, uint4& zr, uint4& tr) {
                             constexpr int kCnt = decltype(tag)::value;
                             constexpr bool kRaw = sizeof(In) == 2 && kCnt == 8;
@@ -1366,7 +1425,7 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                 bool ninf = false, rinf = false;
                 const float Mz = gz == kNegInf ? 0.f : __fmul_rn(gz, c), Mt = gt == kNegInf ? 0.f : __fmul_rn(gt, c);
                 const float2 gz2 = f2(gz), tp2 = f2(tp);
-                sweep_tm<In, false, false, false, true, false, kTmMomG>(tw, tsh, nv, tail, tz, tt,
+                sweep_tm<In, false, false, false, true, false, kTmMomG>(tw, tsh, nv, tail, rj, tz, tt,
                     [&](const float* z, const float* t, auto tag, int, float, float, bool cninf, uint4&, uint4&) {
                         constexpr int kCnt = decltype(tag)::value;
                         if (kCnt == 1 || cninf) {  // element-wise, with the guards a -inf needs
@@ -1446,7 +1505,7 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
             // and Q = sum q (1 up to rounding; summed, it cancels S exactly where
             // every s is the same): k1 q' + k2 |q'| with k1 = Q / (2 tau), k2 = -S / (2 tau)
             const float k1 = sa, k2 = sb;
-            sweep_tm<In, false, false, false, false, false>(tw, tsh, nv, 0, tz, tt,
+            sweep_tm<In, false, false, false, false, false>(tw, tsh, nv, 0, rj, tz, tt,
                 [&](const float*, const float*, auto tag, int j0, float, float, bool, uint4& zr, uint4& tr) {
                     constexpr int kCnt = decltype(tag)::value;
                     if constexpr (kCnt == kVec) {
@@ -1458,7 +1517,7 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                         for (int e = 0; e < kVec; e += 4) stg_v4(orow + j0 + e, gr[e], gr[e + 1], gr[e + 2], gr[e + 3]);
                     }
                 });
-            if (tid < tail) orow[tail0 + tid] = fmaf(k2, fabsf(tq), k1 * tq);
+            if (tid < tail) orow[kAnyPhase ? rj() : tail0 + tid] = fmaf(k2, fabsf(tq), k1 * tq);
         } else {
             // JSD: q (log2(q/m) - S), every probability carrying the gradient's factor,
             // which cancels in log2(q/m); RKL: q ((z - gz) - (t - tp) - X / E) / tau^2,
@@ -1466,7 +1525,7 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
             // q - p, both carrying 1 / tau
             const float2 cvs = f2(cv + p.lg_scale), cus = f2(cu + p.lg_scale);
             const bool has_ninf = (flags & kTmNinf) != 0;
-            sweep_tm<In, false, false, false, false, false, kJsd ? kTmJsdG : kTmG>(tw, tsh, nv, tail, tz, tt,
+            sweep_tm<In, false, false, false, false, false, kJsd ? kTmJsdG : kTmG>(tw, tsh, nv, tail, rj, tz, tt,
                 [&](const float* z, const float* t, auto tag, int j0, float, float, bool, uint4& zr, uint4& tr) {
                     constexpr int kCnt = decltype(tag)::value;
                     // RKL's bf16 chunks take x - m from the packed words (mixed-precision subtracts)
@@ -1519,7 +1578,7 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                 });
         }
     }
-    if (tid == 0 && pending && bytes) mbar_wait_bounded(&bar, pend_phase, kStageWaitNs);  // a copy still in flight lands first
+    if (tid == 0 && pending && (kAnyPhase || bytes)) mbar_wait_bounded(&bar, pend_phase, kStageWaitNs);  // a copy still in flight lands first
     if (csize > 1) {
         // every peer has made all its pushes (in the normal course this CTA has
         // received them all); after a wait that gave up, the partial it waited
@@ -1584,22 +1643,18 @@ static cudaError_t launch_distill_kind(const DistParams& dp, long long rows, siz
                   dp.csize, dp);
 }
 
-// Wide CTAs only on the 16-byte path (TVD, whose extra cluster exchange costs
-// more with them, always takes kDistThreads).
+// (TVD, whose extra cluster exchange costs more with wide CTAs, always takes kDistThreads.)
 template <typename In, bool kAligned>
 static cudaError_t launch_distill_dtype(osd_loss kind, const DistParams& dp, long long rows, size_t smem,
                                         cudaStream_t s) {
-    constexpr int kN = kDistThreads;
-    if constexpr (kAligned) {
-        constexpr int kWd = kDistThreadsWide;
-        if (dp.span >= kDistWideSpan) {
-            switch (kind) {
-                case OSD_FKL: return launch_distill_kind<In, OSD_FKL, true, kWd>(dp, rows, smem, s);
-                case OSD_RKL: return launch_distill_kind<In, OSD_RKL, true, kWd>(dp, rows, smem, s);
-                case OSD_JSD: return launch_distill_kind<In, OSD_JSD, true, kWd>(dp, rows, smem, s);
-                case OSD_CE: return launch_distill_kind<In, OSD_CE, true, kWd>(dp, rows, smem, s);
-                default: break;
-            }
+    constexpr int kN = kDistThreads, kWd = kDistThreadsWide;
+    if (dp.span >= kDistWideSpan) {
+        switch (kind) {
+            case OSD_FKL: return launch_distill_kind<In, OSD_FKL, kAligned, kWd>(dp, rows, smem, s);
+            case OSD_RKL: return launch_distill_kind<In, OSD_RKL, kAligned, kWd>(dp, rows, smem, s);
+            case OSD_JSD: return launch_distill_kind<In, OSD_JSD, kAligned, kWd>(dp, rows, smem, s);
+            case OSD_CE: return launch_distill_kind<In, OSD_CE, kAligned, kWd>(dp, rows, smem, s);
+            default: break;
         }
     }
     switch (kind) {
@@ -1625,7 +1680,7 @@ struct TmLaunch {
 // processing clusters hold at once for a given shared-memory request, which the
 // query cannot do on the TMEM kernel itself.  It is never launched.
 __global__ void __launch_bounds__(kTmThreads, 7) tm_cluster_probe() {}
-template <typename In, int kKind>
+template <typename In, int kKind, bool kAnyPhase>
 static cudaError_t tm_launch_shape(int span, int csize, TmLaunch* out) {
     constexpr int kVec = Elem<In>::kVec;
     const int nv = span / kVec;
@@ -1634,7 +1689,7 @@ static cudaError_t tm_launch_shape(int span, int csize, TmLaunch* out) {
     uint32_t ncols = 32;
     while (ncols < static_cast<uint32_t>(2 * t_off)) ncols <<= 1;
     if (ncols > 512) return cudaErrorInvalidValue;
-    auto kern = distill_tm_kernel<In, kKind>;
+    auto kern = distill_tm_kernel<In, kKind, kAnyPhase>;
     struct Entry {
         int dev, span, csize;
         size_t smem;
@@ -1745,14 +1800,14 @@ static cudaError_t tm_launch_shape(int span, int csize, TmLaunch* out) {
     out->clusters = clusters;
     return cudaSuccess;
 }
-template <typename In, int kKind>
+template <typename In, int kKind, bool kAnyPhase>
 static cudaError_t launch_distill_tm(const DistParams& dp, long long rows, cudaStream_t s) {
     if (dp.csize > 8) {
-        const cudaError_t e = allow_wide_clusters<distill_tm_kernel<In, kKind>>();
+        const cudaError_t e = allow_wide_clusters<distill_tm_kernel<In, kKind, kAnyPhase>>();
         if (e != cudaSuccess) return e;
     }
     TmLaunch tl;
-    const cudaError_t e = tm_launch_shape<In, kKind>(dp.span, dp.csize, &tl);
+    const cudaError_t e = tm_launch_shape<In, kKind, kAnyPhase>(dp.span, dp.csize, &tl);
     if (e != cudaSuccess) return e;
     // Longest runs first: the hardware hands out clusters in about index order, so
     // the last rows, in runs of 2 and then of 1, even out the clusters' finishing
@@ -1783,16 +1838,16 @@ static cudaError_t launch_distill_tm(const DistParams& dp, long long rows, cudaS
     sh.n2 = static_cast<int>((twos + sh.piece2 - 1) / sh.piece2);
     const long long n1 = (ones + sh.piece1 - 1) / sh.piece1;
     const long long runs = sh.n8 + sh.n2 + n1;
-    return launch(distill_tm_kernel<In, kKind>, dim3(static_cast<unsigned>(runs * dp.csize)),
+    return launch(distill_tm_kernel<In, kKind, kAnyPhase>, dim3(static_cast<unsigned>(runs * dp.csize)),
                   dim3(kTmThreads), tl.smem, s, dp.csize, dp, sh);
 }
-template <typename In>
+template <typename In, bool kAnyPhase>
 static cudaError_t launch_distill_tm_kind(osd_loss kind, const DistParams& dp, long long rows, cudaStream_t s) {
     switch (kind) {
-        case OSD_FKL: return launch_distill_tm<In, OSD_FKL>(dp, rows, s);
-        case OSD_JSD: return launch_distill_tm<In, OSD_JSD>(dp, rows, s);
-        case OSD_RKL: return launch_distill_tm<In, OSD_RKL>(dp, rows, s);
-        default: return launch_distill_tm<In, OSD_TVD>(dp, rows, s);
+        case OSD_FKL: return launch_distill_tm<In, OSD_FKL, kAnyPhase>(dp, rows, s);
+        case OSD_JSD: return launch_distill_tm<In, OSD_JSD, kAnyPhase>(dp, rows, s);
+        case OSD_RKL: return launch_distill_tm<In, OSD_RKL, kAnyPhase>(dp, rows, s);
+        default: return launch_distill_tm<In, OSD_TVD, kAnyPhase>(dp, rows, s);
     }
 }
 
@@ -1822,28 +1877,58 @@ static osd_status distill_run(const void* draft_logits, const void* target_logit
     // copy bandwidth (65536 x 32000 bf16); CE stays at 96.3 % on the per-row kernel.
     // Rows chosen by verification stay on the per-row kernel: on the runs, 32 rows
     // of 32000 took 12.8 against 10.4 us, and 256 of 128256 no less time
-    const bool tm_path = aligned && !accepted &&
-                         (kind == OSD_TVD || kind == OSD_JSD || kind == OSD_RKL || kind == OSD_FKL);
+    const bool tm_kind = !accepted && (kind == OSD_TVD || kind == OSD_JSD || kind == OSD_RKL || kind == OSD_FKL);
+    // Rows off the 16-byte grid take the runs too where every row's draft, target and gradient
+    // share one phase in it, as those of contiguous tensors do (V = 32001): the same
+    // bulk copies from the row's first boundary, its head and tail entry by entry (4096 x 32001
+    // bf16: TVD 192 us, FKL 182, JSD 218, CE, on the per-row kernel with the same copies, 181; with
+    // 2-byte loads and 4-byte stores on the per-row kernel they took 455, 512, 775 and 488 us).
+    // Where the phases differ (a view of [B, k + 1, V], rows chosen by verification) the per-row
+    // kernel shifts the rows into place as it loads them (1024 x 32003 bf16 RKL against such a
+    // view: 100 us, 152 element by element).
+    const int vec = static_cast<int>(16 / es);
+    auto phase = [&](const void* ptr, size_t size, int m) {
+        return static_cast<int>((reinterpret_cast<uintptr_t>(ptr) / size) % static_cast<unsigned>(m));
+    };
+    const bool same_phase =
+        !aligned && !accepted && phase(draft_logits, es, vec) == phase(target_logits, es, vec) &&
+        phase(draft_logits, es, 4) == phase(dlogits, 4, 4) &&
+        (G <= 1 || ((d_stride_g - t_stride_g) % vec == 0 && (d_stride_g - int64_t(P) * V) % 4 == 0)) &&
+        (P <= 1 || ((d_stride_p - t_stride_p) % vec == 0 && (d_stride_p - V) % 4 == 0));
+    bool any_phase = same_phase && tm_kind;
+    const bool tm_path = aligned && tm_kind;
     int csize = 1, span = V;
     // JSD, with the most work per entry, stages best in longer spans on the per-row
     // kernel; the TMEM-staged runs take the 32 KB spans for every kind.  (At
     // V = 32000 a span of 8000 bf16 entries leaves room for seven CTAs an SM; spans
     // cut in 16-byte steps to seven CTAs at V = 32128, five CTAs a row instead of
     // four, measured 8 % slower for JSD than four spans of 8064 at six CTAs.)
-    size_t span_bytes = (kind == OSD_JSD && !tm_path) ? kDistSpanBytesJsd : kDistSpanBytes;
+    size_t span_bytes = (kind == OSD_JSD && !tm_path && !any_phase) ? kDistSpanBytesJsd : kDistSpanBytes;
     // no more rows than SMs: half-length spans put twice the CTAs to work on them
     // (measured 6-12 % less latency at 4 and 128 rows of 32000)
-    if (static_cast<long long>(G) * P <= device_sms()) span_bytes /= 2;
-    if (!row_span_shape(V, es, span_bytes, kDistMaxCluster, kDistMaxSmem, &csize, &span))
-        return OSD_ERR_UNSUPPORTED;
+    const bool few = static_cast<long long>(G) * P <= device_sms();
+    if (few) span_bytes /= 2;
     // on the TMEM-staged runs, rows that need more than 8 spans of the target size
     // take up to 16 CTAs: spans that fit 64 columns of tensor memory and six CTAs
     // an SM instead of 128 columns and two (2048 x 128256 bf16: FKL 77.7 against
     // 75.6 %, RKL 71.5 against 67.9 %, TVD 71.8 against 65.0 %, JSD 55.3 against
     // 54.3 %); the per-row kernel keeps at most 8 (measured no faster)
-    if (tm_path && csize == kDistMaxCluster && size_t(span) * 2 * es > span_bytes &&
-        !row_span_shape(V, es, span_bytes, kDistMaxClusterWide, kDistMaxSmem, &csize, &span))
-        return OSD_ERR_UNSUPPORTED;
+    if (any_phase) {
+        // a row may start up to vec - 1 positions into the grid; spans in steps of one chunk
+        const int Vp = V + vec - 1;
+        any_phase = row_span_shape(Vp, es, span_bytes, kDistMaxClusterWide, kDistMaxSmem, vec, &csize, &span) &&
+                    span / vec <= kTmMaxChunks;
+        if (!any_phase && kind == OSD_JSD) span_bytes = kDistSpanBytesJsd / (few ? 2 : 1);
+    }
+    if (!any_phase) {
+        // (rows off the 16-byte grid start up to vec - 1 positions into it)
+        if (!row_span_shape(aligned ? V : V + vec - 1, es, span_bytes, kDistMaxCluster, kDistMaxSmem + (aligned ? 0 : 512), 64,
+                            &csize, &span))
+            return OSD_ERR_UNSUPPORTED;
+        if (tm_path && csize == kDistMaxCluster && size_t(span) * 2 * es > span_bytes &&
+            !row_span_shape(V, es, span_bytes, kDistMaxClusterWide, kDistMaxSmem, 64, &csize, &span))
+            return OSD_ERR_UNSUPPORTED;
+    }
     const long long rows = static_cast<long long>(G) * P;
     if (rows * csize > INT_MAX) return OSD_ERR_UNSUPPORTED;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -1877,14 +1962,18 @@ static osd_status distill_run(const void* draft_logits, const void* target_logit
         if (kind == OSD_JSD) scale *= (1.0 - static_cast<double>(beta)) * 0.69314718055994530942;
         dp.lg_scale = scale > 0.0 ? static_cast<float>(std::log2(scale)) : 0.f;  // beta = 1: gradient is 0
     }
-    dp.csize = csize; dp.span = span;
-    const size_t smem = 2 * size_t(span) * es;
+    dp.csize = csize; dp.span = span; dp.same_phase = same_phase;
+    const size_t smem = 2 * size_t(span + (aligned ? 0 : kSpanPad)) * es;
     cudaError_t e;
     // 16-byte rows and a span that fits tensor memory: the TMEM-staged runs
-    const bool tm = tm_path && span / static_cast<int>(16 / es) <= kTmMaxChunks;
-    if (tm) {
-        e = (dtype == OSD_BF16) ? launch_distill_tm_kind<__nv_bfloat16>(kind, dp, rows, s)
-                                : launch_distill_tm_kind<float>(kind, dp, rows, s);
+    if (any_phase) {
+        e = (dtype == OSD_BF16) ? launch_distill_tm_kind<__nv_bfloat16, true>(kind, dp, rows, s)
+                                : launch_distill_tm_kind<float, true>(kind, dp, rows, s);
+        return from_cuda(e);
+    }
+    if (tm_path && span / vec <= kTmMaxChunks) {
+        e = (dtype == OSD_BF16) ? launch_distill_tm_kind<__nv_bfloat16, false>(kind, dp, rows, s)
+                                : launch_distill_tm_kind<float, false>(kind, dp, rows, s);
         return from_cuda(e);
     }
     if (dtype == OSD_BF16)

@@ -379,3 +379,40 @@ def test_concurrent_flushes_on_two_streams(osd):
         torch.cuda.synchronize()
         for ref, out in ((ref_a, out_a), (ref_b, out_b)):
             assert torch.equal(ref[0], out[0]) and torch.equal(ref[1], out[1])
+
+
+# Rows off the 16-byte grid: chunks at the row's (or the gradient's) own phase, head and
+# tail entries single.  `shift` moves the target off the draft's phase (per-row kernel, through
+# registers); without it FKL, RKL, JSD and TVD take the runs and CE bulk copies at the shared phase.
+PHASE_CASES = [  # (N, V, dtype, shift)
+    (9, 9, torch.bfloat16, 0),          # every phase; some parts without a chunk
+    (9, 9, torch.bfloat16, 3),
+    (9, 3, torch.float32, 1),
+    (40, 4095, torch.bfloat16, 0),
+    (17, 8193, torch.float32, 0),       # a last part of one entry
+    (200, 16385, torch.bfloat16, 0),    # runs of several rows, the phase changing from row to row
+    (200, 16385, torch.bfloat16, 1),
+    (9, 32004, torch.bfloat16, 0),      # rows on 8-byte boundaries
+    (9, 128257, torch.bfloat16, 0),     # 16 CTAs a row
+    (3, 128257, torch.float32, 2),      # wide CTAs
+]
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("N,V,dtype,shift", PHASE_CASES)
+def test_rows_off_the_16_byte_grid(osd, kind, N, V, dtype, shift):
+    inp = W.distill_inputs(W.DistillSpec(N, V, dtype, 2.0, "draft+noise", 1.5, 1.0), seed=11 + V + N)
+    z, t = inp["draft"], inp["target"]
+    if kind == "ce":  # ties of the target maximum, so that the lowest index counts, head entries among them
+        t = (t.float() * 2).round().div(2).to(dtype)
+    store = torch.zeros(N * V + shift, dtype=dtype, device="cuda")
+    td = store[shift:].view(N, V)
+    td.copy_(t)
+    mask = torch.ones(N, dtype=torch.uint8)
+    mask[N // 2] = 0
+    dl = torch.full((N, V), float("nan"), device="cuda")
+    loss, g = osd.osd_distill(z.cuda(), td, mask.cuda(), kind, 0.3, dlogits=dl)
+    torch.cuda.synchronize()
+    lr, gr = _oracle(z, t, mask, kind, 0.3)
+    check_distill(loss.cpu().numpy(), g.cpu().numpy(), lr, gr, mask.numpy() == 1,
+                  _tvd_ambiguous(z, t) if kind == "tvd" else None)
