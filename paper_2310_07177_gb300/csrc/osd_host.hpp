@@ -7,6 +7,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstdint>
+#include <mutex>
 
 #include "osd.h"
 
@@ -43,6 +44,32 @@ inline int device_sms() {
     if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
         sms[dev].store(n, std::memory_order_relaxed);
     return n;
+}
+
+// Opt in for `smem` bytes of dynamic shared memory and ask how many CTAs an SM then
+// holds (0 when a query fails).  Kept per device for the last size asked, so repeated
+// calls (and calls under stream capture) make no runtime query.
+template <auto kern, int kThreads>
+static int ctas_per_sm(size_t smem) {
+    static std::mutex mu;
+    static size_t allowed[64] = {};
+    static size_t last_smem[64] = {};
+    static int last_occ[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    std::lock_guard<std::mutex> lock(mu);
+    if (last_smem[dev] == smem && last_occ[dev] > 0) return last_occ[dev];
+    if (allowed[dev] < smem) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
+            cudaSuccess)
+            return 0;
+        allowed[dev] = smem;
+    }
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, smem) != cudaSuccess) return 0;
+    last_smem[dev] = smem;
+    last_occ[dev] = occ;
+    return occ;
 }
 
 // Launch `kernel` with an optional thread-block cluster of `cluster` CTAs

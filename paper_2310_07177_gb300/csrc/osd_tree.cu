@@ -2,25 +2,19 @@
 // speculative decoding the paper runs OSD on with Medusa heads: several
 // candidates per position) on sm_103a.
 //
-// Two launches on the caller's stream:
+// T > 0: one launch, tree_walk_kernel, one thread-block cluster per sequence, which
+// walks the tree from the root.  At a node it tests the children in index order
+// with the accept rule of Appendix A.1 against the current residual.  After j
+// rejections the residual is norm(max(0, p - s_j q)) with s_0 = 0 and
+// s_{j+1} = s_j + N_j, N_j = sum max(0, p - s_j q), so child y passes iff
+// u < max(0, p(y)/q(y) - s_j) / N_j.  Every rejection costs one cluster-wide pass
+// that recomputes N_{j+1}; an acceptance moves the walk to the child.  When no child
+// passes, the extra token is drawn from max(0, p - s q) by inverse CDF from the
+// sub-tile sums of the last pass, as the verifier draws its residual token (masses
+// summed in exact 64-bit fixed point).  Only the rows the walk comes to are read.
 //
-//   row_stats_kernel   (osd_rowstats.cuh) the max and sum of 2^((x - max) c) of
-//                      every vocabulary slice of every node's draft and target
-//                      row (the argmax at T = 0): the one pass over all logits.
-//   tree_walk_kernel   one thread-block cluster per sequence walks the tree from
-//                      the root.  It merges every node's slice statistics up
-//                      front; at a node it tests the children in index order
-//                      with the accept rule of Appendix A.1 against the current
-//                      residual.  After j rejections the residual is
-//                      norm(max(0, p - s_j q)) with s_0 = 0 and s_{j+1} = s_j + N_j,
-//                      N_j = sum max(0, p - s_j q), so child y passes iff
-//                      u < max(0, p(y)/q(y) - s_j) / N_j.  Every rejection costs one
-//                      cluster-wide pass that recomputes N_{j+1}; an acceptance
-//                      moves the walk to the child.  When no child passes, the
-//                      extra token is drawn from max(0, p - s q) by inverse CDF
-//                      from the sub-tile sums of the last pass, as the verifier's
-//                      finalize kernel draws its residual token (masses summed in
-//                      exact 64-bit fixed point).
+// T = 0: two launches, row_argmax_kernel (osd_rowstats.cuh) over every target row's
+// slices and tree_greedy_kernel, which follows the matching children.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -33,11 +27,12 @@
 
 namespace osd {
 
-constexpr int kTreeThreads = 128;
+constexpr int kTreeThreads = 256;
 constexpr int kTreeWarps = kTreeThreads / 32;
-constexpr int kTreeMaxCluster = 8;
-constexpr int kTreeMaxSub = 8192;  // sub-tiles of one CTA's vocabulary span
-constexpr int kTreeUnroll = 4;     // sub-tiles of loads in flight per warp in a mass pass
+constexpr int kTreeMaxWin = 4;                  // nodes per round ...
+constexpr int kTreeMaxRows = 2 * kTreeMaxWin;   // ... and their rows
+constexpr int kTreeUnroll = 4;                  // sub-tiles of loads in flight per warp in a mass pass
+constexpr int kGreedyThreads = 128;
 
 // Children lists of the static tree: first child and next sibling, increasing
 // index; and each node's parent (-1 at the root).
@@ -54,9 +49,8 @@ struct TreeParams {
     const int32_t* tokens;
     const float* uniforms;
     float T, c_hi, c_lo;
-    const RowStat* stats;
+    const RowStat* stats;  // T = 0: the target rows' slice argmaxes
     int n_slices;
-    long long n_draft_rows;  // rows of draft statistics ahead of the target rows (0 at T = 0)
     int32_t* accepted;
     int32_t* path;
     int32_t* out_tokens;
@@ -67,114 +61,226 @@ struct TreeParams {
     TreeTopo topo;
 };
 
-template <typename In, bool kVecPath>
-__global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
-    using E = Elem<In>;
-    constexpr int kW = kVecPath ? E::kVec : 1;  // entries per lane per sub-tile
-    constexpr int kSub = 32 * kW;
-    extern __shared__ float s_sub[];           // mass of every sub-tile of this CTA's span (last pass)
-    // masses in exact 64-bit fixed point (fix_of): a dependent fp64 add is slow here
-    __shared__ unsigned long long s_span_total;            // read by the other CTAs of the cluster
-    __shared__ unsigned long long s_cta_incl[kTreeMaxCluster];  // inclusive prefix of the CTA masses, rank order
-    __shared__ unsigned long long s_W;
-    __shared__ int s_next, s_extra;
-    // per node: merged statistics of its target (0) and draft (1) rows, or the target argmax at T = 0
-    __shared__ float s_nm[2][OSD_TREE_MAX_NODES], s_ns[2][OSD_TREE_MAX_NODES];
+// T = 0: the walk follows the child whose token is the target argmax.  One CTA per sequence.
+__global__ void __launch_bounds__(kGreedyThreads) tree_greedy_kernel(TreeParams p) {
     __shared__ int s_nidx[OSD_TREE_MAX_NODES];
+    const int tid = threadIdx.x, b = blockIdx.x, n = p.n;
+    const int32_t* y = p.tokens + size_t(b) * n;
+    int32_t* pth = p.path + size_t(b) * n;
+    int32_t* out = p.out_tokens + size_t(b) * n;
+    int bad = 0;
+    for (int i = 1 + tid; i < n; i += kGreedyThreads) bad |= (y[i] < 0 || y[i] >= p.V) ? 1 : 0;
+    bad = __syncthreads_or(bad);
+    for (int i = tid; i < n; i += kGreedyThreads) {
+        pth[i] = -1;
+        out[i] = -1;
+        if (p.diag_margin) p.diag_margin[size_t(b) * n + i] = __int_as_float(0x7fc00000);
+    }
+    if (tid == 0) {
+        if (p.diag_gap) p.diag_gap[b] = __int_as_float(0x7fc00000);
+        if (bad) {
+            p.accepted[b] = -1;
+            p.last_node[b] = -1;
+        }
+    }
+    if (bad) return;
+    grid_dependency_wait();  // the row statistics are complete from here on
+    for (int nd = tid; nd < n; nd += kGreedyThreads) {
+        const RowStat* st = p.stats + (size_t(b) * n + nd) * p.n_slices;
+        MaxIdx acc{kNegInf, INT_MAX};
+#pragma unroll 4
+        for (int sl = 0; sl < p.n_slices; ++sl) acc = merge_mi(acc, MaxIdx{st[sl].m, st[sl].idx});
+        s_nidx[nd] = (acc.i == INT_MAX) ? 0 : acc.i;
+    }
+    __syncthreads();  // (the initialisation above lands before the walk writes its entries)
+    if (tid != 0) return;
+    int node = 0, depth = 0;
+    for (;;) {
+        const int best = s_nidx[node];
+        int next = -1;
+        for (int c = p.topo.first_child[node]; c >= 0; c = p.topo.next_sibling[c])
+            if (y[c] == best) { next = c; break; }
+        if (next < 0) {
+            out[depth] = best;
+            break;
+        }
+        pth[depth] = next;
+        out[depth++] = y[next];
+        node = next;
+    }
+    p.accepted[b] = depth;
+    p.last_node[b] = node;
+}
+
+// T > 0.  Each CTA owns a span of the vocabulary.  A round takes the rows of a node and of
+// the `win` - 1 next ones down its first children (the likeliest way on).  The span
+// statistics meet by st.async, every CTA merging the same slots in rank order, and
+// warp 0 of every CTA walks on alike: tests cost no exchange until a rejection needs
+// a mass pass, whose span totals meet the same way, or the walk leaves the round.
+//
+// What bounds it: the chain of dependent phases, about 3 us a round and 2 us a rejection.
+// B = 32, 27 nodes, V = 32000 (1.8 accepted): 24 us where the statistics of every node's rows
+// took 44; V = 128256: 50 us against 125; B = 64, V = 32001: 39 us against 107.  Two CTAs an SM
+// at 120 registers: with three or four the passes spill (33 and 35 us); rows staged in
+// shared memory first took 26 us, and at V = 128256, where they leave one CTA an SM, 79 us.
+template <typename In, bool kAligned>
+__global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p, int win) {
+    using E = Elem<In>;
+    constexpr int kW = E::kVec;  // entries per lane per sub-tile
+    constexpr int kSub = 32 * kW;
+    extern __shared__ float s_sub[];  // mass of every sub-tile of this CTA's span (last pass)
+    __shared__ MaxSum s_part[kTreeMaxRows > kTreeWarps ? kTreeMaxRows : kTreeWarps];
+    __shared__ __align__(8) MaxSum s_recv[2][kSeqMaxCluster * kTreeMaxRows];  // [CTA][row slot], two rounds
+    __shared__ __align__(8) unsigned long long s_totals[2][kSeqMaxCluster];   // span masses, two passes
+    __shared__ __align__(8) uint64_t s_bar[2], s_tbar[2];
+    // the round's statistics: row slot 2 q is node q's target row, 2 q + 1 its draft row
+    __shared__ float s_m[kTreeMaxRows], s_s[kTreeMaxRows];
+    __shared__ double s_ratio[kTreeMaxWin];  // E_z / E_t of each node with children
     // per child c: its token's logits in the draft and target rows of its parent, and its uniform
     __shared__ float s_zy[OSD_TREE_MAX_NODES], s_ty[OSD_TREE_MAX_NODES], s_u[OSD_TREE_MAX_NODES];
-    __shared__ double s_nratio[OSD_TREE_MAX_NODES];  // per node with children: E_z / E_t
+    __shared__ int s_y[OSD_TREE_MAX_NODES];
+    __shared__ int s_act, s_node, s_q, s_depth;  // what warp 0 decided
+    __shared__ float s_shift;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int csize = p.csize;
     const int rank = (csize > 1) ? static_cast<int>(cluster_rank()) : 0;
     const int b = blockIdx.x / csize;
     const int n = p.n, V = p.V;
-    const bool greedy = (p.T == 0.f);
-    const int32_t* y = p.tokens + size_t(b) * n;
-    const float* u = p.uniforms ? p.uniforms + size_t(b) * n : nullptr;
+    const int e0 = rank * p.span;
+    const int cnt = min(p.span, V - e0);
+    const int nsub = (cnt + kSub - 1) / kSub;
+    const In* draft = static_cast<const In*>(p.draft) + size_t(b) * n * V;
+    const In* target = static_cast<const In*>(p.target) + size_t(b) * n * V;
     int32_t* pth = p.path + size_t(b) * n;
     int32_t* out = p.out_tokens + size_t(b) * n;
     const float ch = p.c_hi, cl = p.c_lo;
 
-    // Prologue, before the statistics are ready: check the tokens and gather the two
-    // logits every child's accept test needs, all in one round of loads.
+    // nodes of the round that starts at `node`: down the first children; and their rows
+    // (a leaf, which only the last can be, has no use for its draft row)
+    auto round_nodes = [&](int node) {
+        int w = 1;
+        for (int nd = p.topo.first_child[node]; nd >= 0 && w < win; nd = p.topo.first_child[nd]) ++w;
+        return w;
+    };
+    auto node_at = [&](int node, int q) {
+        for (; q > 0; --q) node = p.topo.first_child[node];
+        return node;
+    };
+    auto row_of = [&](int node, int slot) {
+        const size_t nd = static_cast<size_t>(node_at(node, slot >> 1));
+        return ((slot & 1) ? draft : target) + nd * V + e0;
+    };
+    auto rows_of = [&](int node, int w) { return 2 * w - (p.topo.first_child[node_at(node, w - 1)] < 0 ? 1 : 0); };
+
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init_only(&s_bar[i], 1);
+            mbar_init_only(&s_tbar[i], 1);
+        }
+        fence_mbarrier_init();
+    }
+    // check the tokens and gather the two logits every child's accept test needs
     int bad = 0;
-    if (!greedy)
-        for (int i = tid; i < n; i += kTreeThreads) s_u[i] = u[i];
-    for (int i = 1 + tid; i < n; i += kTreeThreads) {
-        const int yi = y[i];
+    for (int i = tid; i < n; i += kTreeThreads) {
+        s_u[i] = p.uniforms[size_t(b) * n + i];
+        const int yi = p.tokens[size_t(b) * n + i];
+        s_y[i] = yi;
+        if (i == 0) continue;
         if (yi < 0 || yi >= V) {
             bad = 1;
-        } else if (!greedy) {
-            const size_t prow = size_t(b) * n + p.topo.parent[i];
-            s_zy[i] = E::load(static_cast<const In*>(p.draft) + prow * V + yi);
-            s_ty[i] = E::load(static_cast<const In*>(p.target) + prow * V + yi);
+        } else {
+            const size_t prow = static_cast<size_t>(p.topo.parent[i]) * V;
+            s_zy[i] = E::load(draft + prow + yi);
+            s_ty[i] = E::load(target + prow + yi);
         }
     }
-    bad = __syncthreads_or(bad);
-    if (rank == 0) {
-        for (int i = tid; i < n; i += kTreeThreads) {
-            pth[i] = -1;
-            out[i] = -1;
-            if (p.diag_margin) p.diag_margin[size_t(b) * n + i] = __int_as_float(0x7fc00000);
-        }
-        if (tid == 0 && p.diag_gap) p.diag_gap[b] = __int_as_float(0x7fc00000);
-        if (tid == 0 && bad) {
-            p.accepted[b] = -1;
-            p.last_node[b] = -1;
-        }
-    }
-    if (bad) return;  // uniform over the cluster, before any shared-memory exchange
-    __syncthreads();  // the initialisation above lands before the walk writes its entries
-    grid_dependency_wait();  // the row statistics are complete from here on
+    if (rank == 0 && p.diag_margin)
+        for (int i = tid; i < n; i += kTreeThreads) p.diag_margin[size_t(b) * n + i] = __int_as_float(0x7fc00000);
+    __syncthreads();  // the barriers are initialised before anyone waits on them
+    // ... and before any peer pushes to them: arrive now, wait before the first push
+    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 
-    // Every node's row statistics, merged from their slices up front (one thread per
-    // node and row, all loads in one round) instead of one dependent round per node
-    // on the walk.  Draft rows matter only where children are tested.
-    for (int t = tid; t < 2 * n; t += kTreeThreads) {
-        const int nd = t >> 1, which = t & 1;
-        if (greedy) {
-            if (which == 0) {
-                const RowStat* st = p.stats + (size_t(b) * n + nd) * p.n_slices;
-                MaxIdx acc{kNegInf, INT_MAX};
-#pragma unroll 4
-                for (int sl = 0; sl < p.n_slices; ++sl) acc = merge_mi(acc, MaxIdx{st[sl].m, st[sl].idx});
-                s_nidx[nd] = (acc.i == INT_MAX) ? 0 : acc.i;
+    constexpr int kRound = 0, kMass = 1, kDraw = 2, kGone = 3, kBad = 4;  // what comes next
+    int act = kRound, node = 0;  // node: the round's first
+    unsigned round = 0, pass = 0;
+
+    // warp 0's walk state (the same in every CTA): the current node, its place in the
+    // round, the child under test, the residual's shift and mass
+    int cur = 0, q = 0, child = p.topo.first_child[0], depth = 0;
+    float s = 0.f;
+    double N = 1.0;
+    unsigned long long Nfix = 0ull;
+    int rn_nodes = 1;
+    // Test children from `child` on until something else has to happen; every lane alike.
+    auto walk = [&]() {
+        for (;;) {
+            if (child < 0) {  // no child passed: draw, from p itself when none was rejected
+                act = (s > 0.f) ? kDraw : kMass;
+                return;
             }
-        } else if (which == 0 || p.topo.first_child[nd] >= 0) {
-            const RowStat* st = p.stats + ((which == 0 ? p.n_draft_rows : 0) + size_t(b) * n + nd) * p.n_slices;
-            MaxSum acc{kNegInf, 0.f};
-#pragma unroll 4
-            for (int sl = 0; sl < p.n_slices; ++sl) acc = merge_ms(acc, MaxSum{st[sl].m, st[sl].s}, ch, cl);
-            s_nm[which][nd] = acc.m;
-            s_ns[which][nd] = acc.s;
+            // p(y)/q(y) from the logit differences and the two sums, as the verifier
+            // forms it; the test u < max(0, p/q - s) / N is taken as u N < max(0, p/q - s)
+            const float zt = s_zy[child], tt = s_ty[child];
+            double rn;  // max(0, p(y)/q(y) - s_j)
+            if (zt == kNegInf) {
+                rn = (tt > kNegInf) ? INFINITY : 0.0;
+            } else {
+                const float D = (tt - s_m[2 * q]) - (zt - s_m[2 * q + 1]);
+                const double rho = double(ex2(mul_c(D, ch, cl))) * s_ratio[q];
+                rn = fmax(rho - double(s), 0.0);
+            }
+            const float uc = s_u[child];
+            if (rank == 0 && lane == 0 && p.diag_margin)  // |u - r|, a diagnostic: fp32 is enough
+                p.diag_margin[size_t(b) * n + child] = fabsf(uc - float(rn) / float(N));
+            if (!(double(uc) * N < rn)) {
+                s = static_cast<float>(double(s) + N);  // rejected: s_{j+1} = s_j + N_j
+                act = kMass;
+                return;
+            }
+            if (rank == 0 && lane == 0) {
+                pth[depth] = child;
+                out[depth] = s_y[child];
+            }
+            ++depth;
+            const bool next_in_round = q + 1 < rn_nodes && child == p.topo.first_child[cur];
+            cur = child;
+            child = p.topo.first_child[cur];
+            s = 0.f;
+            N = 1.0;
+            if (!next_in_round) {
+                act = kRound;
+                return;
+            }
+            ++q;
         }
-    }
-    __syncthreads();
-    // the sum ratio of each accept test's p/q, once per node (fp64 divisions are slow here)
-    if (!greedy) {
-        for (int nd = tid; nd < n; nd += kTreeThreads)
-            if (p.topo.first_child[nd] >= 0) s_nratio[nd] = double(s_ns[1][nd]) / double(s_ns[0][nd]);
-        __syncthreads();
-    }
-    float cur_mt = 0.f, cur_st = 1.f, cur_mz = 0.f, cur_sz = 1.f;  // the current node's statistics
-
-    const int e0 = rank * p.span;
-    const int cnt = max(0, min(p.span, V - e0));
-    const int nsub = (cnt + kSub - 1) / kSub;
-    bool pending = false;  // a cluster barrier phase is open: peers may still read s_span_total
-
-    // weights w = max(0, p - s q) of kW entries of one lane (q only when s > 0)
+    };
+    auto publish = [&]() {
+        if (lane == 0) {
+            s_act = act;
+            s_node = cur;
+            s_q = q;
+            s_shift = s;
+            s_depth = depth;
+        }
+    };
     struct Raw {
         uint4 t, z;
     };
     auto load_sub = [&](const In* trow, const In* zrow, bool use_q, int sb, Raw& r) {
-        const int j0 = e0 + sb * kSub + lane * kW;
-        const int m = min(kW, e0 + cnt - j0);
-        if (kVecPath && m == kW) {
-            r.t = ldg_stream(trow + j0);
-            r.z = use_q ? ldg_stream(zrow + j0) : r.t;
+        const int j0 = sb * kSub + lane * kW;  // in the span
+        const int m = min(kW, cnt - j0);
+        bool whole = m == kW;
+        if constexpr (!kAligned)
+            whole = whole && shifted_inside(trow - e0, e0 + j0, V) && (!use_q || shifted_inside(zrow - e0, e0 + j0, V));
+        if (whole) {
+            if constexpr (kAligned) {
+                r.t = ldg_stream(trow + j0);
+                r.z = use_q ? ldg_stream(zrow + j0) : r.t;
+            } else {
+                r.t = ldg_shifted(trow + j0);
+                r.z = use_q ? ldg_shifted(zrow + j0) : r.t;
+            }
         } else {
             float tv[kW], zv[kW];
 #pragma unroll
@@ -186,271 +292,305 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
             r.z = pack_raw<In, kW>(zv);
         }
     };
-    auto weights = [&](const Raw& r, bool use_q, float s, float* w) {
-        const float mt = cur_mt, inv_st = 1.0f / cur_st;
-        float tv[kW], zv[kW];
-        unpack_raw<In, kW>(r.t, tv);
-        unpack_raw<In, kW>(r.z, zv);
-        const float mz = cur_mz, inv_sz = use_q ? 1.0f / cur_sz : 0.f;
+    // w = max(0, p - s q) of kW entries of one lane (p itself when !use_q), in pairs
+    auto weights = [&](const Raw& r, bool use_q, float sh, float mt, float inv_st, float mz, float inv_sz, float2* w) {
+        float2 d[kW / 2];
+        E::minus(r.t, mt, d);
 #pragma unroll
-        for (int e = 0; e < kW; ++e) {
-            const float pj = ex2(mul_c(tv[e] - mt, ch, cl)) * inv_st;
-            if (use_q) {
-                const float qj = ex2(mul_c(zv[e] - mz, ch, cl)) * inv_sz;
-                w[e] = fmaxf(fmaf(-s, qj, pj), 0.f);
-            } else {
-                w[e] = pj;
+        for (int e = 0; e < kW / 2; ++e) w[e] = mul2(exp2_pair(d[e], ch, cl), f2(inv_st));
+        if (use_q) {
+            E::minus(r.z, mz, d);
+#pragma unroll
+            for (int e = 0; e < kW / 2; ++e) {
+                const float2 qj = mul2(exp2_pair(d[e], ch, cl), f2(inv_sz));
+                const float2 df = fma2(f2(-sh), qj, w[e]);
+                w[e] = make_float2(fmaxf(df.x, 0.f), fmaxf(df.y, 0.f));
             }
         }
-    };
-    // One cluster-wide pass: the mass of every sub-tile of w = max(0, p - s q) into s_sub,
-    // the CTA masses' inclusive prefix into s_cta_incl, and the row's mass W (returned,
-    // fixed point).
-    auto mass_pass = [&](const In* trow, const In* zrow, bool use_q, float s) -> unsigned long long {
-        if (pending) cluster_wait();  // every peer has read the previous pass's total
-        for (int sb0 = warp; sb0 < nsub; sb0 += kTreeWarps * kTreeUnroll) {
-            Raw r[kTreeUnroll];  // the loads of kTreeUnroll sub-tiles go out together
-#pragma unroll
-            for (int u2 = 0; u2 < kTreeUnroll; ++u2)
-                if (sb0 + u2 * kTreeWarps < nsub) load_sub(trow, zrow, use_q, sb0 + u2 * kTreeWarps, r[u2]);
-#pragma unroll
-            for (int u2 = 0; u2 < kTreeUnroll; ++u2) {
-                const int sb = sb0 + u2 * kTreeWarps;
-                if (sb < nsub) {
-                    float w[kW];
-                    weights(r[u2], use_q, s, w);
-                    float sum = 0.f;
-#pragma unroll
-                    for (int e = 0; e < kW; ++e) sum += w[e];
-                    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-                    if (lane == 0) s_sub[sb] = sum;
-                }
-            }
-        }
-        __syncthreads();
-        if (warp == 0) {
-            unsigned long long part = 0ull;
-            for (int sb = lane; sb < nsub; sb += 32) part += fix_of(s_sub[sb]);
-            part = warp_sum_u64(part);
-            if (lane == 0) s_span_total = part;
-        }
-        if (csize > 1) cluster_sync_publish(tid == 0); else __syncthreads();
-        if (warp == 0) {
-            unsigned long long tot = 0ull;
-            if (lane < csize) tot = (lane == rank) ? s_span_total : ld_dsmem_u64(map_rank(&s_span_total, lane));
-            const unsigned long long incl = warp_incl_scan_u64(tot);
-            if (lane < csize) s_cta_incl[lane] = incl;
-            if (lane == 31) s_W = incl;
-        }
-        __syncthreads();
-        if (csize > 1) {
-            cluster_arrive_relaxed();  // done reading the peers' totals
-            pending = true;
-        }
-        return s_W;
     };
 
-    int node = 0, depth = 0;
     for (;;) {
-        const In* trow = static_cast<const In*>(p.target) + (size_t(b) * n + node) * V;
-        const In* zrow = static_cast<const In*>(p.draft) + (size_t(b) * n + node) * V;
-        const bool has_child = p.topo.first_child[node] >= 0;
-        const bool need_q = !greedy && has_child;
-        cur_mt = s_nm[0][node];
-        cur_st = s_ns[0][node];
-        if (need_q) {
-            cur_mz = s_nm[1][node];
-            cur_sz = s_ns[1][node];
-        }
-
-        int next = -1;
-        if (greedy) {
-            const int best = s_nidx[node];
-            for (int c = p.topo.first_child[node]; c >= 0; c = p.topo.next_sibling[c])
-                if (y[c] == best) { next = c; break; }
-            if (next < 0) {
-                if (tid == 0) s_extra = best;
+        if (act == kRound) {
+            // ---- the round's rows: span statistics, exchanged and merged
+            const int w = round_nodes(node), nr = rows_of(node, w);
+            const int parts = max(1, kTreeWarps / nr);
+            for (int it = warp; it < nr * parts; it += kTreeWarps) {
+                const int r = it / parts;
+                const MaxSum mine = span_stats<In>(row_of(node, r), cnt, it - r * parts, parts, ch, cl);
+                if (lane == 0) s_part[it] = mine;
+            }
+            if (__syncthreads_or(bad)) {  // (only in the first round) uniform over the cluster, before any push to a peer
+                act = kBad;
                 break;
             }
+            if (round == 0 && csize > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+            if (warp == 0) {
+                const unsigned buf = round & 1u;
+                MaxSum* recv = s_recv[buf];
+                bool gone = false;
+                if (lane < nr) {
+                    const MaxSum acc = merge_slots(s_part + lane * parts, 1, parts, ch, cl);
+                    if (csize > 1) {
+                        for (int d = 0; d < csize; ++d)
+                            st_async_v2(map_rank(&recv[rank * kTreeMaxRows + lane], static_cast<uint32_t>(d)),
+                                        make_float2(acc.m, acc.s), map_rank(&s_bar[buf], static_cast<uint32_t>(d)));
+                    } else {
+                        recv[lane] = acc;
+                    }
+                }
+                if (csize > 1) {
+                    if (lane == 0) mbar_arrive_expect_tx(&s_bar[buf], static_cast<uint32_t>(csize * nr) * 8u);
+                    gone = !mbar_wait_cluster_bounded(&s_bar[buf], (round >> 1) & 1u, kPeerWaitNs);
+                }
+                __syncwarp();
+                if (!gone && lane < nr) {
+                    const MaxSum o = merge_slots(recv + lane, kTreeMaxRows, csize, ch, cl);
+                    s_m[lane] = o.m;
+                    s_s[lane] = o.s;
+                }
+                __syncwarp();
+                if (2 * lane + 1 < nr) s_ratio[lane] = double(s_s[2 * lane + 1]) / double(s_s[2 * lane]);
+                __syncwarp();
+                q = 0;
+                rn_nodes = w;
+                if (__any_sync(0xffffffffu, gone)) act = kGone;
+                else walk();
+                publish();
+            }
+            ++round;
         } else {
-            float s = 0.f;  // residual shift s_j
-            double N = 1.0;  // residual mass N_j (p itself has mass 1)
-            unsigned long long Nfix = 0ull;  // the same, in fixed point, after a mass pass
-            bool passed = false;  // a mass pass of the current residual has run
-            for (int c = p.topo.first_child[node]; c >= 0; c = p.topo.next_sibling[c]) {
-                if (tid == 0) {
-                    // p(y)/q(y) from the logit differences and the two sums, as the verifier
-                    // forms it; the test u < max(0, p/q - s) / N is taken as u N < max(0, p/q - s)
-                    const float zt = s_zy[c], tt = s_ty[c];
-                    double rn;  // max(0, p(y)/q(y) - s_j)
-                    if (zt == kNegInf) {
-                        rn = (tt > kNegInf) ? INFINITY : 0.0;
-                    } else {
-                        const float D = (tt - cur_mt) - (zt - cur_mz);
-                        const double rho = double(ex2(mul_c(D, ch, cl))) * s_nratio[node];
-                        rn = fmax(rho - double(s), 0.0);
+            // ---- one cluster-wide pass: the mass of every sub-tile of w = max(0, p - s q) (of p
+            // itself at a node without a rejection, to draw from) into s_sub, and the row's mass
+            const int nq = s_q;
+            const float sh = s_shift;
+            const bool use_q = sh > 0.f;
+            const int nd = s_node;
+            const In* trow = target + size_t(nd) * V + e0;
+            const In* zrow = draft + size_t(nd) * V + e0;
+            const float mt = s_m[2 * nq], inv_st = 1.0f / s_s[2 * nq];
+            const float mz = use_q ? s_m[2 * nq + 1] : 0.f, inv_sz = use_q ? 1.0f / s_s[2 * nq + 1] : 0.f;
+            for (int sb0 = warp; sb0 < nsub; sb0 += kTreeWarps * kTreeUnroll) {
+                Raw r[kTreeUnroll];  // the loads of kTreeUnroll sub-tiles go out together
+#pragma unroll
+                for (int u2 = 0; u2 < kTreeUnroll; ++u2)
+                    if (sb0 + u2 * kTreeWarps < nsub) load_sub(trow, zrow, use_q, sb0 + u2 * kTreeWarps, r[u2]);
+                float sum[kTreeUnroll];
+#pragma unroll
+                for (int u2 = 0; u2 < kTreeUnroll; ++u2) {
+                    sum[u2] = 0.f;
+                    if (sb0 + u2 * kTreeWarps < nsub) {
+                        float2 wv[kW / 2];
+                        weights(r[u2], use_q, sh, mt, inv_st, mz, inv_sz, wv);
+                        float2 s2 = wv[0];
+#pragma unroll
+                        for (int e = 1; e < kW / 2; ++e) s2 = add2(s2, wv[e]);
+                        sum[u2] = s2.x + s2.y;
                     }
-                    const float uc = s_u[c];
-                    if (rank == 0 && p.diag_margin)  // |u - r|, a diagnostic: fp32 is enough
-                        p.diag_margin[size_t(b) * n + c] = fabsf(uc - float(rn) / float(N));
-                    s_next = (double(uc) * N < rn) ? c : -1;
                 }
-                __syncthreads();
-                next = s_next;
-                __syncthreads();  // s_next is rewritten by the next test
-                if (next >= 0) break;
-                s = static_cast<float>(double(s) + N);  // rejected: s_{j+1} = s_j + N_j
-                Nfix = mass_pass(trow, zrow, true, s);
-                N = __ull2double_rn(Nfix) * (1.0 / static_cast<double>(1ull << kFixBits));
-                passed = true;
+                const float tot = warp_sum4(sum);
+                const int sb = sb0 + (lane >> 3) * kTreeWarps;
+                if ((lane & 7) == 0 && sb < nsub) s_sub[sb] = tot;
             }
-            if (next < 0) {
-                // ---- the extra token from w = max(0, p - s q) (p itself when nothing was rejected)
-                const bool use_q = passed;
-                const unsigned long long W = passed ? Nfix : mass_pass(trow, zrow, false, 0.f);
-                const unsigned long long tau = fix_scale(s_u[0], W);  // floor(u W)
-                int owner = -1, mode = 0;  // mode 0: inverse CDF, 1: largest positive entry, 2: argmax p
-                unsigned long long base = 0ull;
-                if (W > 0ull) {
-                    for (int r = 0; r < csize; ++r)
-                        if (s_cta_incl[r] > tau) { owner = r; break; }
-                    if (owner >= 0) {
-                        base = owner > 0 ? s_cta_incl[owner - 1] : 0ull;
-                    } else {
-                        mode = 1;
-                        for (int r = csize - 1; r >= 0 && owner < 0; --r)
-                            if (s_cta_incl[r] > (r > 0 ? s_cta_incl[r - 1] : 0ull)) owner = r;
-                        if (owner < 0) owner = csize - 1;
-                    }
+            __syncthreads();
+            if (warp == 0) {
+                unsigned long long part = 0ull;
+                for (int sb = lane; sb < nsub; sb += 32) part += fix_of(s_sub[sb]);
+                part = warp_sum_u64(part);
+                const unsigned buf = pass & 1u;
+                bool gone = false;
+                if (csize > 1) {
+                    if (lane < csize)
+                        st_async_u64(map_rank(&s_totals[buf][rank], static_cast<uint32_t>(lane)), part,
+                                     map_rank(&s_tbar[buf], static_cast<uint32_t>(lane)));
+                    if (lane == 0) mbar_arrive_expect_tx(&s_tbar[buf], static_cast<uint32_t>(csize) * 8u);
+                    gone = !mbar_wait_cluster_bounded(&s_tbar[buf], (pass >> 1) & 1u, kPeerWaitNs);
+                }
+                const unsigned long long tot = lane < csize ? (csize > 1 ? s_totals[buf][lane] : part) : 0ull;
+                Nfix = __shfl_sync(0xffffffffu, warp_incl_scan_u64(tot), 31);
+                if (__any_sync(0xffffffffu, gone)) {
+                    act = kGone;
+                } else if (!use_q) {  // a leaf, or a node whose draw is from p itself
+                    act = kDraw;
                 } else {
-                    mode = 2;
-                    owner = 0;
+                    N = __ull2double_rn(Nfix) * (1.0 / static_cast<double>(1ull << kFixBits));
+                    child = p.topo.next_sibling[child];
+                    walk();
                 }
-                if (rank == owner && warp == 0) {
-                    int pick = -1;
-                    float gap = __int_as_float(0x7fc00000);
-                    if (mode == 2) {  // no residual mass: argmax of p over the row, lowest index
-                        MaxIdx acc{kNegInf, INT_MAX};
-                        for (int j = lane; j < V; j += 32) {
-                            const float t = E::load(trow + j);
-                            if (t > acc.m) { acc.m = t; acc.i = j; }
-                        }
-                        acc = warp_reduce(acc, [](MaxIdx x, MaxIdx z) { return merge_mi(x, z); });
-                        pick = (acc.i == INT_MAX) ? 0 : acc.i;
-                    } else {
-                        // the sub-tile: lane l owns the run [s_lo, s_hi) of sub-tiles
-                        const int per = (nsub + 31) / 32;
-                        const int s_lo = min(nsub, lane * per), s_hi = min(nsub, s_lo + per);
-                        unsigned long long mine = 0ull;
-                        for (int sb = s_lo; sb < s_hi; ++sb) mine += fix_of(s_sub[sb]);
-                        const unsigned long long excl = base + warp_incl_scan_u64(mine) - mine;
-                        int tile = -1;
-                        unsigned long long tbase = 0ull;
-                        if (mode == 0) {
-                            const unsigned h = __ballot_sync(0xffffffffu, excl <= tau && excl + mine > tau);
-                            if (h) {
-                                const int l = __ffs(h) - 1;
-                                if (lane == l) {  // the sums are exact: the run holds tau in one sub-tile
-                                    unsigned long long c2 = excl;
-                                    for (int sb = s_lo; sb < s_hi; ++sb) {
-                                        const unsigned long long v = fix_of(s_sub[sb]);
-                                        if (c2 + v > tau) { tile = sb; break; }
-                                        c2 += v;
-                                    }
-                                    tbase = c2;
-                                }
-                                tile = __shfl_sync(0xffffffffu, tile, l);
-                                tbase = __shfl_sync(0xffffffffu, tbase, l);
-                            } else {
-                                mode = 1;
-                            }
-                        }
-                        if (mode == 1) {
-                            int last = -1;
-                            for (int sb = s_lo; sb < s_hi; ++sb)
-                                if (s_sub[sb] > 0.f) last = sb;
-                            for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
-                            tile = max(last, 0);
-                        }
-                        Raw r;
-                        load_sub(trow, zrow, use_q, tile, r);
-                        float w[kW];
-                        weights(r, use_q, s, w);
-                        const int j0 = e0 + tile * kSub + lane * kW;
-                        bool done = false;
-                        if (mode == 0) {
-                            unsigned long long wsum = 0ull;
-#pragma unroll
-                            for (int e = 0; e < kW; ++e) wsum += fix_of(w[e]);
-                            const unsigned long long wex = tbase + warp_incl_scan_u64(wsum) - wsum;
-                            const bool hit = wex <= tau && wex + wsum > tau;
-                            if (hit) {
-                                unsigned long long C = wex;
-                                for (int e = 0; e < kW; ++e) {
-                                    const unsigned long long Cprev = C;
-                                    C += fix_of(w[e]);
-                                    if (C > tau) {
-                                        pick = j0 + e;
-                                        gap = fminf(fix_to_float(C - tau), fix_to_float(tau - Cprev)) / fix_to_float(W);
-                                        break;
-                                    }
-                                }
-                            }
-                            done = __any_sync(0xffffffffu, hit);
-                        }
-                        if (!done) {  // the largest j of the sub-tile with w_j > 0 (rounding fallback)
-                            int best = -1;
-                            float wbest = 0.f;
-#pragma unroll
-                            for (int e = 0; e < kW; ++e)
-                                if (w[e] > 0.f) { best = j0 + e; wbest = w[e]; }
-                            int jb = best;
-                            for (int o = 16; o > 0; o >>= 1) jb = max(jb, __shfl_xor_sync(0xffffffffu, jb, o));
-                            pick = -1;
-                            if (jb >= 0 && best == jb) {
-                                pick = jb;
-                                const float Wf = fix_to_float(W), tf = fix_to_float(tau);
-                                gap = fminf(Wf - tf, tf - (Wf - wbest)) / Wf;
-                            } else if (jb < 0 && lane == 0) {
-                                pick = j0;  // no positive entry: cannot happen when W > 0
-                            }
-                        }
-                    }
-                    if (pick >= 0 && (mode != 2 || lane == 0)) {
-                        out[depth] = pick;
-                        if (p.diag_gap && mode != 2) p.diag_gap[b] = gap;
-                    }
-                }
-                if (tid == 0) s_extra = -1;  // written by the owner
-                break;
+                publish();
+            }
+            ++pass;
+        }
+        __syncthreads();
+        act = s_act;
+        node = s_node;
+        if (act == kDraw || act == kGone) break;
+    }
+    if (act != kDraw) {  // a bad token, or the GPU did not deliver in time: the sequence is reported as bad
+        if (act == kGone && csize > 1 && tid == 0) {
+            if (round > 0) mbar_wait_cluster_bounded(&s_bar[(round - 1) & 1u], ((round - 1) >> 1) & 1u, kPeerWaitNs);
+            if (pass > 0) mbar_wait_cluster_bounded(&s_tbar[(pass - 1) & 1u], ((pass - 1) >> 1) & 1u, kPeerWaitNs);
+        }
+        if (rank == 0) {
+            for (int i = tid; i < n; i += kTreeThreads) {
+                pth[i] = -1;
+                out[i] = -1;
+                if (p.diag_margin) p.diag_margin[size_t(b) * n + i] = __int_as_float(0x7fc00000);
+            }
+            if (tid == 0) {
+                p.accepted[b] = -1;
+                p.last_node[b] = -1;
+                if (p.diag_gap) p.diag_gap[b] = __int_as_float(0x7fc00000);
             }
         }
-        if (rank == 0 && tid == 0) {
-            pth[depth] = next;
-            out[depth] = y[next];
+        return;
+    }
+    // ---- the walk's outputs, and the extra token (entry `depth`) by the CTA that owns it
+    depth = s_depth;
+    if (rank == 0) {
+        if (tid == 0) {
+            p.accepted[b] = depth;
+            p.last_node[b] = node;
         }
-        ++depth;
-        node = next;
+        for (int i = tid; i < n; i += kTreeThreads) {
+            if (i >= depth) pth[i] = -1;
+            if (i > depth) out[i] = -1;
+        }
     }
-    if (rank == 0 && tid == 0) {
-        if (greedy) out[depth] = s_extra;
-        p.accepted[b] = depth;
-        p.last_node[b] = node;
+    if (warp != 0) return;
+    // the last pass's span masses, a lane per CTA: W, tau = floor(u W) and the owning CTA
+    const unsigned lastbuf = (pass - 1) & 1u;
+    unsigned long long own = 0ull;
+    if (csize == 1) {
+        for (int sb = lane; sb < nsub; sb += 32) own += fix_of(s_sub[sb]);
+        own = warp_sum_u64(own);
     }
-    if (pending) cluster_wait();  // keep this CTA's total readable until every peer is done
+    const unsigned long long tot = lane < csize ? (csize > 1 ? s_totals[lastbuf][lane] : own) : 0ull;
+    const unsigned long long incl = warp_incl_scan_u64(tot);
+    const unsigned long long W = __shfl_sync(0xffffffffu, incl, 31);
+    const unsigned long long tau = fix_scale(s_u[0], W);
+    int owner = 0, mode = 0;  // mode 0: inverse CDF, 1: largest positive entry, 2: argmax p
+    unsigned long long base = 0ull;
+    if (W > 0ull) {
+        const unsigned hit = __ballot_sync(0xffffffffu, lane < csize && incl > tau);
+        if (hit) {
+            owner = __ffs(hit) - 1;
+            base = __shfl_sync(0xffffffffu, incl - tot, owner);
+        } else {
+            mode = 1;
+            owner = 31 - __clz(__ballot_sync(0xffffffffu, lane < csize && tot > 0ull));
+        }
+    } else {
+        mode = 2;
+    }
+    if (rank != owner) return;
+    const int nq = s_q;
+    const float sh = s_shift;
+    const bool use_q = sh > 0.f;
+    const In* trow = target + size_t(node) * V + e0;
+    const In* zrow = draft + size_t(node) * V + e0;
+    int pick = -1;
+    float gap = __int_as_float(0x7fc00000);
+    if (mode == 2) {  // no residual mass: argmax of p over the row, lowest index
+        const In* grow = target + size_t(node) * V;
+        MaxIdx acc{kNegInf, INT_MAX};
+        for (int j = lane; j < V; j += 32) {
+            const float t = E::load(grow + j);
+            if (t > acc.m) { acc.m = t; acc.i = j; }
+        }
+        acc = warp_reduce(acc, [](MaxIdx x, MaxIdx z) { return merge_mi(x, z); });
+        if (lane == 0) pick = (acc.i == INT_MAX) ? 0 : acc.i;
+    } else {
+        // the sub-tile: lane l owns the run [s_lo, s_hi) of sub-tiles
+        const int per = (nsub + 31) / 32;
+        const int s_lo = min(nsub, lane * per), s_hi = min(nsub, s_lo + per);
+        unsigned long long mine = 0ull;
+        for (int sb = s_lo; sb < s_hi; ++sb) mine += fix_of(s_sub[sb]);
+        const unsigned long long excl = base + warp_incl_scan_u64(mine) - mine;
+        int tile = -1;
+        unsigned long long tbase = 0ull;
+        if (mode == 0) {
+            const unsigned h = __ballot_sync(0xffffffffu, excl <= tau && excl + mine > tau);
+            if (h) {
+                const int l = __ffs(h) - 1;
+                if (lane == l) {  // the sums are exact: the run holds tau in one sub-tile
+                    unsigned long long c2 = excl;
+                    for (int sb = s_lo; sb < s_hi; ++sb) {
+                        const unsigned long long v = fix_of(s_sub[sb]);
+                        if (c2 + v > tau) { tile = sb; break; }
+                        c2 += v;
+                    }
+                    tbase = c2;
+                }
+                tile = __shfl_sync(0xffffffffu, tile, l);
+                tbase = __shfl_sync(0xffffffffu, tbase, l);
+            } else {
+                mode = 1;
+            }
+        }
+        if (mode == 1) {
+            int last = -1;
+            for (int sb = s_lo; sb < s_hi; ++sb)
+                if (s_sub[sb] > 0.f) last = sb;
+            for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
+            tile = max(last, 0);
+        }
+        Raw r;
+        load_sub(trow, zrow, use_q, tile, r);
+        float2 w2[kW / 2];
+        weights(r, use_q, sh, s_m[2 * nq], 1.0f / s_s[2 * nq], use_q ? s_m[2 * nq + 1] : 0.f,
+                use_q ? 1.0f / s_s[2 * nq + 1] : 0.f, w2);
+        float wv[kW];
+#pragma unroll
+        for (int e = 0; e < kW / 2; ++e) {
+            wv[2 * e] = w2[e].x;
+            wv[2 * e + 1] = w2[e].y;
+        }
+        const int j0 = e0 + tile * kSub + lane * kW;
+        bool done = false;
+        if (mode == 0) {
+            unsigned long long wsum = 0ull;
+#pragma unroll
+            for (int e = 0; e < kW; ++e) wsum += fix_of(wv[e]);
+            const unsigned long long wex = tbase + warp_incl_scan_u64(wsum) - wsum;
+            const bool hit = wex <= tau && wex + wsum > tau;
+            if (hit) {
+                unsigned long long C = wex;
+                for (int e = 0; e < kW; ++e) {
+                    const unsigned long long Cprev = C;
+                    C += fix_of(wv[e]);
+                    if (C > tau) {
+                        pick = j0 + e;
+                        gap = fminf(fix_to_float(C - tau), fix_to_float(tau - Cprev)) / fix_to_float(W);
+                        break;
+                    }
+                }
+            }
+            done = __any_sync(0xffffffffu, hit);
+        }
+        if (!done) {  // the largest j of the sub-tile with w_j > 0 (rounding fallback)
+            int best = -1;
+            float wbest = 0.f;
+#pragma unroll
+            for (int e = 0; e < kW; ++e)
+                if (wv[e] > 0.f) { best = j0 + e; wbest = wv[e]; }
+            int jb = best;
+            for (int o = 16; o > 0; o >>= 1) jb = max(jb, __shfl_xor_sync(0xffffffffu, jb, o));
+            if (jb >= 0 && best == jb) {
+                pick = jb;
+                const float Wf = fix_to_float(W), tf = fix_to_float(tau);
+                gap = fminf(Wf - tf, tf - (Wf - wbest)) / Wf;
+            } else if (jb < 0 && lane == 0) {
+                pick = e0 + tile * kSub;  // no positive entry: cannot happen when W > 0
+            }
+        }
+    }
+    if (pick >= 0) {
+        out[depth] = pick;
+        if (p.diag_gap) p.diag_gap[b] = gap;
+    }
 }
 
 // ------------------------------------------------------------------ host
-static void tree_shape(int V, int* csize, int* span) {
-    int c = (V + 4095) / 4096;
-    c = c < 1 ? 1 : (c > kTreeMaxCluster ? kTreeMaxCluster : c);
-    int s = (V + c - 1) / c;
-    s = (s + 63) / 64 * 64;
-    c = (V + s - 1) / s;
-    *csize = c;
-    *span = s;
-}
-
 static bool tree_topology(const int32_t* parent, int n, TreeTopo* topo) {
     if (!parent || parent[0] != -1) return false;
     for (int i = 0; i < OSD_TREE_MAX_NODES; ++i) {
@@ -477,42 +617,43 @@ template <typename In>
 static osd_status launch_tree(const TreeParams& base, int B, const void* draft, const void* target,
                               RowStat* stats, cudaStream_t stream) {
     TreeParams tp = base;
-    const bool greedy = (tp.T == 0.f);
     const int n = tp.n, V = tp.V;
-    const long long rows = tree_stat_rows(B, n, greedy);
-    const int slice_len = stats_slice_len(rows);
-    const int n_slices = (V + slice_len - 1) / slice_len;
-    const long long n_draft_rows = greedy ? 0 : (long long)B * n;
-    const long long grid1 = rows * n_slices;
-    if (grid1 > INT_MAX) return OSD_ERR_UNSUPPORTED;
-    cudaError_t e;
-    if (greedy)
-        e = launch(row_stats_kernel<In, true>, dim3(unsigned(grid1)), dim3(kStatThreads), 0, stream, 1,
-                   static_cast<const In*>(draft), static_cast<const In*>(target), n_draft_rows, V, slice_len,
-                   n_slices, tp.c_hi, tp.c_lo, stats);
-    else
-        e = launch(row_stats_kernel<In, false>, dim3(unsigned(grid1)), dim3(kStatThreads), 0, stream, 1,
-                   static_cast<const In*>(draft), static_cast<const In*>(target), n_draft_rows, V, slice_len,
-                   n_slices, tp.c_hi, tp.c_lo, stats);
-    if (e != cudaSuccess) return OSD_ERR_CUDA;
-
-    tp.stats = stats;
-    tp.n_slices = n_slices;
-    tp.n_draft_rows = n_draft_rows;
-    int csize = 1, span = V;
-    if (!greedy) tree_shape(V, &csize, &span);
-    tp.csize = csize;
-    tp.span = span;
-    const bool vec = !greedy && aligned_to(draft, 16) && aligned_to(target, 16) && ((size_t)V * sizeof(In)) % 16 == 0;
-    const int sub = 32 * (vec ? Elem<In>::kVec : 1);
-    const size_t smem = greedy ? 0 : size_t((span + sub - 1) / sub) * sizeof(float);
-    if (smem > size_t(kTreeMaxSub) * sizeof(float)) return OSD_ERR_UNSUPPORTED;
-    const dim3 grid2(unsigned(B) * unsigned(csize));
-    if (vec)
-        e = launch_ex(true, tree_walk_kernel<In, true>, grid2, dim3(kTreeThreads), smem, stream, csize, tp);
-    else
-        e = launch_ex(true, tree_walk_kernel<In, false>, grid2, dim3(kTreeThreads), smem, stream, csize, tp);
-    return from_cuda(e);
+    constexpr size_t es = sizeof(In);
+    if (tp.T == 0.f) {
+        const long long rows = tree_stat_rows(B, n, true);
+        const int slice_len = stats_slice_len(rows);
+        tp.n_slices = (V + slice_len - 1) / slice_len;
+        tp.stats = stats;
+        if (rows * tp.n_slices > INT_MAX) return OSD_ERR_UNSUPPORTED;
+        const cudaError_t e = launch(row_argmax_kernel<In>, dim3(unsigned(rows * tp.n_slices)), dim3(kStatThreads), 0, stream,
+                                     1, static_cast<const In*>(target), V, slice_len, tp.n_slices, stats);
+        if (e != cudaSuccess) return OSD_ERR_CUDA;
+        return from_cuda(launch_ex(true, tree_greedy_kernel, dim3(unsigned(B)), dim3(kGreedyThreads), 0, stream, 1, tp));
+    }
+    // CTAs per sequence: 8, but 4 where 8 would run past one wave (two CTAs an SM) and the
+    // spans stay short (B = 48 and 64 at V = 32000: 31.9 and 38.3 us against 42.5 and 48.4; at
+    // V = 64000, B = 64 the two are level, 59 and 58 us)
+    int c = kSeqMaxCluster;
+    if ((long long)B * c > 2LL * device_sms() && V <= 50000) c /= 2;
+    while (c > 1 && V <= 2048 * c) c /= 2;
+    tp.span = ((V + c - 1) / c + 63) / 64 * 64;
+    tp.csize = (V + tp.span - 1) / tp.span;
+    if ((long long)B * tp.csize > INT_MAX) return OSD_ERR_UNSUPPORTED;
+    // Nodes per round, by the bytes of one node of the batch: a round costs about 3 us beside
+    // them, and first children that the walk does not come to are read for nothing (B = 1,
+    // V = 32000: 4 nodes 15.4 us, 1 node 19.5; B = 32: 26.0, 2 nodes 24.1, 1 node 25.9; B = 64,
+    // V = 128256, 33 MB: 2 nodes 86, 4 nodes 88; B = 64, V = 150016 fp32, 77 MB: 1 node 121, 2 nodes
+    // 142).  A tree without siblings passes them often (B = 32, 9 nodes: 4 nodes 24.3 us, 2 nodes 28.7).
+    const double pos = double(B) * 2 * V * double(es);
+    bool siblings = false;
+    for (int i = 0; i < n; ++i) siblings |= tp.topo.next_sibling[i] >= 0;
+    const int win = pos <= 3e6 || (!siblings && pos <= 40e6) ? kTreeMaxWin : (pos <= 40e6 ? 2 : 1);
+    const dim3 grid(unsigned(B) * unsigned(tp.csize));
+    constexpr int sub = 32 * Elem<In>::kVec;
+    const size_t smem = size_t((tp.span + sub - 1) / sub) * sizeof(float);
+    const bool aligned = aligned_to(draft, 16) && aligned_to(target, 16) && ((size_t)V * es) % 16 == 0;
+    return from_cuda(aligned ? launch(tree_walk_kernel<In, true>, grid, dim3(kTreeThreads), smem, stream, tp.csize, tp, win)
+                             : launch(tree_walk_kernel<In, false>, grid, dim3(kTreeThreads), smem, stream, tp.csize, tp, win));
 }
 
 }  // namespace osd

@@ -17,7 +17,7 @@
 // sub-tile, the span totals meet as exact 64-bit fixed point, and the CTA whose
 // span holds u*W rescans that one sub-tile exactly.
 //
-// T = 0: two launches, row_stats_kernel (the argmax of every target row's slices) and
+// T = 0: two launches, row_argmax_kernel (the argmax of every target row's slices) and
 // verify_greedy_kernel, one warp per sequence: the matches in order, the target
 // argmax at the first mismatch.
 //
@@ -39,9 +39,6 @@
 
 namespace osd {
 
-constexpr int kFinMaxCluster = 8;
-constexpr uint64_t kStageWaitNs = 1000000000ull;  // bound on the wait for staged rows ...
-constexpr uint64_t kPeerWaitNs = 3000000000ull;   // ... and for the peers' statistics and totals
 constexpr int kFinUnroll = 4;     // sub-tiles of loads in flight per warp
 // Where the draw reads the rows from: shared memory, 16-byte-aligned rows in global
 // memory, or rows of any alignment there.
@@ -154,22 +151,6 @@ __device__ __forceinline__ void seq_write_bad(const FinParams& p, int b) {
     }
 }
 
-// One row's statistics from `count` <= 8 partials at x[0], x[stride], ..., merged in
-// that order: the maximum first, then the sums brought to it (all loads in flight together).
-__device__ __forceinline__ MaxSum merge_slots(const MaxSum* x, int stride, int count, float ch, float cl) {
-    MaxSum o[kFinMaxCluster];
-    float m = kNegInf, s = 0.f;
-#pragma unroll
-    for (int i = 0; i < kFinMaxCluster; ++i) {
-        o[i] = (i < count) ? x[i * stride] : MaxSum{kNegInf, 0.f};
-        m = fmaxf(m, o[i].m);
-    }
-#pragma unroll
-    for (int i = 0; i < kFinMaxCluster; ++i)
-        if (o[i].m != kNegInf) s += o[i].s * ex2(mul_c(o[i].m - m, ch, cl));
-    return MaxSum{m, s};
-}
-
 // One round of accept tests, run by warp 0 of every CTA of the cluster alike:
 // positions i0 .. i0 + w - 1, a lane each, the first failing one is a.  Returns
 // a, k when the bonus position is reached without a failure, or -1 when the
@@ -256,7 +237,7 @@ struct DrawSmem {
     unsigned long long tau, W, base;
     int owner, mode, tile;
     // pushed span totals: slot r from CTA r, completing on tbar
-    unsigned long long totals[kFinMaxCluster];
+    unsigned long long totals[kSeqMaxCluster];
     uint64_t tbar;
 };
 
@@ -347,11 +328,9 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
         }
     };
 
-    // pass 1: one fp32 sum per sub-tile, no block barrier.  The kFinUnroll sums of a
-    // step are reduced over the lanes together: each exchange halves the number of
-    // sums a lane carries, 6 shuffles instead of 20, and lane l ends with the sum of
-    // sub-tile l / 8
-    static_assert(kFinUnroll == 4, "the reduction below carries four sums");
+    // pass 1: one fp32 sum per sub-tile, no block barrier; the sums of a step are
+    // reduced over the lanes together
+    static_assert(kFinUnroll == 4, "warp_sum4 carries four sums");
     for (int s0 = warp; s0 < nsub; s0 += kWarps * kFinUnroll) {
         Raw r[kFinUnroll];
 #pragma unroll
@@ -370,13 +349,7 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
                 sum[u] = s2.x + s2.y;
             }
         }
-        const bool hi = lane & 16, mid = lane & 8;
-        float s01 = hi ? sum[2] : sum[0], s23 = hi ? sum[3] : sum[1];
-        s01 += __shfl_xor_sync(0xffffffffu, hi ? sum[0] : sum[2], 16);
-        s23 += __shfl_xor_sync(0xffffffffu, hi ? sum[1] : sum[3], 16);
-        float tot = mid ? s23 : s01;
-        tot += __shfl_xor_sync(0xffffffffu, mid ? s01 : s23, 8);
-        for (int o = 4; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        const float tot = warp_sum4(sum);
         const int s = s0 + (lane >> 3) * kWarps;
         if ((lane & 7) == 0 && s < nsub) s_sub[s] = tot;
     }
@@ -563,104 +536,8 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
 // for their copies.
 constexpr int kLazyMaxWin = 4;               // positions per round ...
 constexpr int kLazyMaxRows = 2 * kLazyMaxWin;  // ... two rows each
-constexpr int kLazyUnroll = 4;               // 16-byte vectors per lane per group (one group in flight ahead)
 constexpr int kLazyThreads = 256;
 constexpr int kStagedThreads = 512;          // with a staged first round: one CTA an SM
-constexpr size_t kStageMaxSmem = 200 * 1024;  // dynamic shared memory per CTA of the staging kernels
-
-// Max and sum of 2^((x - max) c) of chunks [c0, c1) of a staged row, by one warp: the
-// maximum first, then the sum against it.
-template <typename In>
-__device__ __forceinline__ MaxSum staged_stats(const In* row, int c0, int c1, float ch, float cl) {
-    using E = Elem<In>;
-    constexpr int kVec = E::kVec;
-    const int lane = threadIdx.x & 31;
-    float m = kNegInf;
-    for (int c = c0 + lane; c < c1; c += 32) m = fmaxf(m, E::max_raw(lds_v4(row + c * kVec)));
-    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    float2 s2 = f2(0.f);
-    if (m != kNegInf) {
-        for (int c = c0 + lane; c < c1; c += 32) {
-            float2 d[kVec / 2];
-            E::minus(lds_v4(row + c * kVec), m, d);
-#pragma unroll
-            for (int e = 0; e < kVec / 2; ++e) s2 = add2(s2, exp2_pair(d[e], ch, cl));
-        }
-    }
-    float s = s2.x + s2.y;
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    return MaxSum{m, s};
-}
-
-// Max and sum of 2^((x - max) c) of the entries p[0, n), taken by `parts` warps:
-// this one, number `part`, takes every parts-th group of 32 vectors (part 0 also the
-// entries before the first 16-byte boundary, the last part those after the last).
-template <typename In>
-__device__ __forceinline__ MaxSum span_stats(const In* p, int n, int part, int parts, float c_hi, float c_lo) {
-    using E = Elem<In>;
-    constexpr int kVec = E::kVec;
-    const int lane = threadIdx.x & 31;
-    int head = static_cast<int>(((16u - (reinterpret_cast<uintptr_t>(p) & 15u)) & 15u) / sizeof(In));
-    if (head > n) head = n;
-    const int nvec = (n - head) / kVec;
-    const int tail0 = head + nvec * kVec;
-    const In* body = p + head;
-    float m = kNegInf;
-    float2 s2 = f2(0.f);
-    auto raise_max = [&](float cm) {
-        if (cm > m) {
-            s2 = (m == kNegInf) ? f2(0.f) : mul2(s2, f2(ex2(mul_c(m - cm, c_hi, c_lo))));
-            m = cm;
-        }
-    };
-    auto one = [&](float x) {
-        raise_max(x);
-        if (m != kNegInf) s2.x += ex2(mul_c(x - m, c_hi, c_lo));
-    };
-    const int step = 32 * parts;
-    auto load_group = [&](int v, uint4* r) {
-#pragma unroll
-        for (int u = 0; u < kLazyUnroll; ++u) {
-            const int vv = v + u * step;
-            r[u] = (vv < nvec) ? ldg_stream(body + size_t(vv) * kVec) : ninf_raw<In>();
-        }
-    };
-    auto absorb = [&](const uint4* r) {
-        float cm = E::max_raw(r[0]);
-#pragma unroll
-        for (int u = 1; u < kLazyUnroll; ++u) cm = fmaxf(cm, E::max_raw(r[u]));
-        raise_max(cm);
-        if (m != kNegInf) {
-#pragma unroll
-            for (int u = 0; u < kLazyUnroll; ++u) {
-                float2 d[kVec / 2];
-                E::minus(r[u], m, d);  // exact, as is c = c_hi + c_lo
-#pragma unroll
-                for (int e = 0; e < kVec / 2; ++e) s2 = add2(s2, exp2_pair(d[e], c_hi, c_lo));
-            }
-        }
-    };
-    // two groups in turn, the next one's loads out before this one's sums
-    uint4 ra[kLazyUnroll], rb[kLazyUnroll];
-    const int stride = kLazyUnroll * step;
-    int v = part * 32 + lane;
-    if (v < nvec) load_group(v, ra);
-    if (part == 0 && lane < head) one(E::load(p + lane));
-    if (part == parts - 1 && lane < n - tail0) one(E::load(p + tail0 + lane));
-    for (; v < nvec; v += 2 * stride) {
-        if (v + stride < nvec) load_group(v + stride, rb);
-        absorb(ra);
-        if (v + stride >= nvec) break;
-        if (v + 2 * stride < nvec) load_group(v + 2 * stride, ra);
-        absorb(rb);
-    }
-    // warp merge: the maximum first, then one rescale per lane and a plain sum
-    float wm = m;
-    for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
-    float s = (m == kNegInf) ? 0.f : (s2.x + s2.y) * ex2(mul_c(m - wm, c_hi, c_lo));
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return MaxSum{wm, s};
-}
 
 // Byte offset of the sub-tile sums in the kernel's dynamic shared memory: after the
 // staged rows of the first round (none when kStaged is off).
@@ -681,7 +558,7 @@ verify_lazy_kernel(FinParams p, int win, int ahead) {
     __shared__ SeqSmem sh;
     __shared__ DrawSmem ds;
     __shared__ MaxSum s_part[kWarps];
-    __shared__ __align__(8) MaxSum s_recv[2][kFinMaxCluster * kLazyMaxRows];  // [CTA][row], two rounds
+    __shared__ __align__(8) MaxSum s_recv[2][kSeqMaxCluster * kLazyMaxRows];  // [CTA][row], two rounds
     __shared__ __align__(8) uint64_t s_bar[2];
     __shared__ __align__(8) uint64_t s_rbar[kLazyMaxRows];  // staged rows
     __shared__ int s_dec;  // first failing position, k after the bonus row, -1 undecided, -2 a wait gave up
@@ -943,32 +820,6 @@ static int verify_slices(int B, int k, int V) {
 
 static size_t round256(size_t x) { return (x + 255) / 256 * 256; }
 
-// Opt in for `smem` bytes of dynamic shared memory and ask how many CTAs an SM then
-// holds (0 when a query fails).  Kept per device for the last size asked, so repeated
-// calls (and calls under stream capture) make no runtime query.
-template <auto kern, int kThreads>
-static int ctas_per_sm(size_t smem) {
-    static std::mutex mu;
-    static size_t allowed[64] = {};
-    static size_t last_smem[64] = {};
-    static int last_occ[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    std::lock_guard<std::mutex> lock(mu);
-    if (last_smem[dev] == smem && last_occ[dev] > 0) return last_occ[dev];
-    if (allowed[dev] < smem) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
-            cudaSuccess)
-            return 0;
-        allowed[dev] = smem;
-    }
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, smem) != cudaSuccess) return 0;
-    last_smem[dev] = smem;
-    last_occ[dev] = occ;
-    return occ;
-}
-
 // Split V over at most c CTAs in spans of a multiple of 64 entries.
 static void split_vocab(int V, int c, FinParams* fp) {
     int s = (V + c - 1) / c;
@@ -986,7 +837,7 @@ static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
     if (aligned && B <= kFuseMaxB) {
         // every row staged, only in one wave: at B = 32, k = 5, V = 32000 (two CTAs an SM) 12.8 us
         // against 14.7 us on demand; at B = 48, past one wave, it took 34 us (17.8 on demand)
-        split_vocab(V, kFinMaxCluster, &fp);
+        split_vocab(V, kSeqMaxCluster, &fp);
         const size_t smem = fused_recv_offset(2 * k + 1, fp.span, es) + size_t(fp.csize) * (2 * k + 1) * sizeof(MaxSum);
         if (smem <= kStageMaxSmem &&
             (long long)B * fp.csize <= (long long)device_sms() * ctas_per_sm<verify_fused_kernel<In>, kFuseThreads>(smem))
@@ -1006,7 +857,7 @@ static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
     // the first round staged where the batch is at most one CTA an SM, with fewer positions
     // where they do not fit (B = 16, k = 8, V = 128256, 2 positions: 27 us against 39 us streamed)
     if (aligned) {
-        split_vocab(V, kFinMaxCluster, &fp);
+        split_vocab(V, kSeqMaxCluster, &fp);
         for (int w = win; w >= 1 && (long long)B * fp.csize <= device_sms(); w /= 2) {
             const size_t smem = lazy_sub_offset(2 * w, fp.span, es) + sub_bytes();
             if (smem > kStageMaxSmem || ctas_per_sm<verify_lazy_kernel<In, true, true>, kStagedThreads>(smem) < 1) continue;
@@ -1020,7 +871,7 @@ static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
     // 68 KB, so that the rows in flight stay in L2 for the draw (B = 256: V = 32000 2 CTAs a
     // sequence, 37.9 us against 41.1 and 45.9 us with 4 and 8; V = 128256 8 CTAs, 76 us against
     // 85 and 102 us with 4 and 2)
-    int c = kFinMaxCluster;
+    int c = kSeqMaxCluster;
     while (c > 1 && (V <= 2048 * c || ((long long)B * c / 2 >= 3LL * device_sms() && size_t(V / (c / 2)) * 2 * es <= 68 * 1024)))
         c /= 2;
     split_vocab(V, c, &fp);
@@ -1051,9 +902,8 @@ static osd_status launch_verify(const void* draft, const void* target, int B, in
         const long long grid1 = (long long)B * (k + 1) * fp.n_slices;
         if (grid1 > INT_MAX) return OSD_ERR_UNSUPPORTED;
         const cudaError_t e =
-            launch(row_stats_kernel<In, true>, dim3(unsigned(grid1)), dim3(kStatThreads), 0, stream, 1,
-                   static_cast<const In*>(draft), static_cast<const In*>(target), 0LL, V, slice_len, fp.n_slices,
-                   0.f, 0.f, stats);
+            launch(row_argmax_kernel<In>, dim3(unsigned(grid1)), dim3(kStatThreads), 0, stream, 1,
+                   static_cast<const In*>(target), V, slice_len, fp.n_slices, stats);
         if (e != cudaSuccess) return OSD_ERR_CUDA;
         fp.csize = 1;
         fp.span = V;

@@ -190,3 +190,25 @@ def test_invalid_arguments_are_rejected(osd):
     assert ei.value.status == osd.OSD_ERR_INVALID_ARG
     with pytest.raises(ValueError):
         osd.osd_verify_tree(t, t, [-1, 0, 0], y.long(), u, 1.0)
+
+
+# Rounds of nodes read on demand: trees and sizes that end walks in every round, by the
+# nodes per round (4, 2 and 1), alignment and CTAs per sequence.
+COMB = [-1, 0, 0, 1, 1, 3, 3, 5, 5, 7, 7, 9, 9]  # a first-child chain of six with a sibling each
+ROUND_CASES = [  # (parents, B, V, dtype, T, noise)
+    ([-1] + list(range(12)), 12, 4096, torch.bfloat16, 1.0, 0.2),   # a chain of 13: four rounds
+    (COMB, 16, 32001, torch.bfloat16, 1.0, 0.3),                    # unaligned rows
+    (COMB, 9, 128256, torch.float32, 0.7, 0.3),                     # 9 MB a node: rounds of 2
+    ([-1, 0, 0, 1, 3], 40, 128256, torch.float32, 1.0, 0.3),        # 41 MB a node: one node a round
+    (COMB, 48, 9001, torch.float32, 1.0, 0.3),                      # two CTAs a sequence
+    (COMB, 64, 50, torch.bfloat16, 1.3, 0.5),                       # one CTA a sequence
+    ([-1], 5, 33000, torch.bfloat16, 1.0, 0.5),                     # the root alone: a draw from p
+]
+
+
+@pytest.mark.parametrize("parents,B,V,dtype,T,noise", ROUND_CASES)
+def test_rounds_match_oracle(osd, parents, B, V, dtype, T, noise):
+    inp = W.tree_inputs(B, parents, V, dtype, T, seed=B * 1000 + V + 1, target_noise=noise)
+    if len(parents) > 2:  # a token outside [0, V) marks its own sequence only
+        inp["tokens"][1, 2] = V
+    _check(osd, inp, T)
