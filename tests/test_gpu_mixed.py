@@ -183,3 +183,37 @@ def test_invalid_arguments_are_rejected(osd):
     e = torch.zeros(0, 16, device=dev)
     tok, _ = osd.osd_mixed_sample(e, e, torch.zeros(0, device=dev), 0.5)
     assert tok.numel() == 0
+
+
+# Rows off the 16-byte grid: both rows of a pair at the same phase (chunks cut there), or at
+# different ones (chunks shifted into place): `shift` entries between the two.
+@pytest.mark.parametrize("N,V,dtype,shift", [
+    (40, 3, torch.bfloat16, 0), (40, 9, torch.bfloat16, 0), (9, 255, torch.float32, 0), (33, 4099, torch.bfloat16, 0),
+    (9, 32001, torch.bfloat16, 0), (9, 32004, torch.bfloat16, 0), (5, 33003, torch.float32, 0),
+    (40, 9, torch.bfloat16, 3), (9, 1023, torch.float32, 1), (9, 32001, torch.bfloat16, 5), (3, 128257, torch.bfloat16, 1)])
+def test_rows_off_the_16_byte_grid(osd, N, V, dtype, shift):
+    z, t, u = _inputs(N, V, dtype, seed=V + N + shift)
+    u[0], u[N // 2] = 0.0, float(np.nextafter(np.float32(1), np.float32(0)))  # the row's two ends
+    store = torch.zeros(N * V + shift, dtype=dtype, device="cuda")
+    td = store[shift:].view(N, V)
+    td.copy_(t)
+    gap = torch.empty(N, device="cuda")
+    tok, _ = osd.osd_mixed_sample(z.cuda(), td, u.cuda(), 0.4, temperature=0.9, cdf_gap=gap)
+    torch.cuda.synchronize()
+    ref, ref_gap = oracle.mixed_sample(z, t, u, 0.4, float(np.float32(0.9)))
+    ok = ref_gap >= TIE
+    np.testing.assert_array_equal(tok.cpu().numpy()[ok], ref[ok])
+    assert np.all(np.abs(gap.cpu().numpy()[ok] - ref_gap[ok]) <= 2e-6)
+    assert np.all((tok.cpu().numpy() >= 0) & (tok.cpu().numpy() < V))
+
+
+# Few rows: 16 and 32 warps a row, at the row counts and lengths where the choice changes.
+@pytest.mark.parametrize("N,V,dtype", [
+    (1, 6399, torch.bfloat16), (1, 6400, torch.bfloat16), (608, 3200, torch.float32), (609, 3200, torch.float32),
+    (3, 65535, torch.bfloat16), (3, 65792, torch.bfloat16), (2, 32897, torch.float32), (5, 102657, torch.bfloat16)])
+def test_few_rows(osd, N, V, dtype):
+    z, t, u = _inputs(N, V, dtype, seed=3 * V + N)
+    u[0], u[N // 2] = 0.0, float(np.nextafter(np.float32(1), np.float32(0)))
+    z[0, : V // 2] = float("-inf")  # pieces without mass
+    t[0, : V // 2] = float("-inf")
+    _check(osd, z, t, u, 0.4, 0.9)
