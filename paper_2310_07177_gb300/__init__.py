@@ -1,8 +1,10 @@
 """GB300-native hot path of Online Speculative Decoding (Liu et al., ICML 2024).
 
-Thin ctypes binding over ``libosd.so`` (the C ABI in ``include/osd.h``): it
-turns torch tensors into device pointers, sizes and the current CUDA stream,
-allocates outputs with torch, and raises ``OsdError`` on a non-OK status.
+Thin binding over ``libosd.so`` (the C ABI in ``include/osd.h``): it turns torch
+tensors into device pointers, sizes and the current CUDA stream, allocates
+outputs with torch, and raises ``OsdError`` on a non-OK status.  Calls with plain
+CUDA tensors go through native code (``csrc/osd_binding.cpp``); any other call is
+checked here and goes through ctypes.
 Every step of verify and distill runs in the library's CUDA kernels; there is
 no CPU path.  If the library has not been built, calls raise immediately.
 
@@ -15,12 +17,14 @@ from __future__ import annotations
 
 import contextlib
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from typing import NamedTuple, Optional
 
 import torch
 
-from ._build import LIB_PATH, build as build_library  # noqa: F401
+from ._build import BINDING_PATH, LIB_PATH, build as build_library  # noqa: F401
 
 OSD_OK, OSD_ERR_INVALID_ARG, OSD_ERR_UNSUPPORTED, OSD_ERR_CUDA, OSD_ERR_TIMEOUT = range(5)
 OSD_F32, OSD_BF16 = 0, 1
@@ -81,6 +85,30 @@ def load_library():
     lib.osd_mixed_sample.argtypes = [vp, vp, i32, i32, i32, i64, i64, vp, f32, f32, vp, vp, vp, vp]
     _lib = lib
     return lib
+
+
+_binding = None
+
+
+def _load_binding():
+    """The native calls (raises if they have not been built)."""
+    global _binding
+    load_library()
+    if not os.path.exists(BINDING_PATH):
+        raise RuntimeError(f"{BINDING_PATH} not found: build it with paper_2310_07177_gb300.build_library()")
+    loader = importlib.machinery.ExtensionFileLoader("_binding", BINDING_PATH)
+    mod = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_binding", BINDING_PATH, loader=loader))
+    loader.exec_module(mod)
+    mod.setup(VerifyResult, DistillAcceptedResult, TreeResult)
+    _binding = mod
+    return mod
+
+
+def _native(what: str, result):
+    """A native call's result, raising on the status of one that failed."""
+    if type(result) is int:
+        raise OsdError(result, what)
+    return result
 
 
 def osd_status_string(status: int) -> str:
@@ -158,6 +186,10 @@ def osd_verify(draft_logits: torch.Tensor, target_logits: torch.Tensor, draft_to
     may be None.  ``workspace`` (uint8, >= osd_verify_workspace_size bytes) and
     ``out`` may be preallocated to avoid allocations on the hot path.
     """
+    r = (_binding or _load_binding()).verify(draft_logits, target_logits, draft_tokens, uniforms, temperature,
+                                             diagnostics, workspace, out, stream)
+    if r is not None:
+        return _native("osd_verify", r)
     lib = load_library()
     B, k1, V = target_logits.shape
     k = k1 - 1
@@ -237,6 +269,10 @@ def osd_distill(draft_logits: torch.Tensor, target_logits: torch.Tensor, mask: O
     fp32 [..] and fp32 [.., V] contiguous.  Rows with mask 0 get loss 0 and are
     not written in ``dlogits`` (pass a prefilled ``dlogits`` to keep them).
     """
+    r = (_binding or _load_binding()).distill(draft_logits, target_logits, mask, loss_kind, beta, temperature, loss,
+                                              dlogits, status, stream)
+    if r is not None:
+        return _native("osd_distill", r)
     lib = load_library()
     dev = _need_cuda(draft_logits, target_logits, mask, loss, dlogits, status)
     G, P, V, dsg, dsp = _rows_view(draft_logits)
@@ -284,6 +320,10 @@ def osd_distill_accepted(draft_logits: torch.Tensor, target_logits: torch.Tensor
     contributes row (b, accepted[b]) when that is < k; results are compacted on
     the device, active sequences first (see ``DistillAcceptedResult``).
     """
+    r = (_binding or _load_binding()).distill_accepted(draft_logits, target_logits, accepted, loss_kind, beta,
+                                                       temperature, out, status, stream)
+    if r is not None:
+        return _native("osd_distill_accepted", r)
     lib = load_library()
     dev = _need_cuda(draft_logits, target_logits, accepted, status, *(out or ()))
     if draft_logits.dim() != 3 or target_logits.dim() != 3:
@@ -327,6 +367,10 @@ def osd_mixed_sample(draft_logits: torch.Tensor, target_logits: torch.Tensor, un
     (``expand`` of one row is fine); ``uniforms`` [N] fp32 in [0, 1).  Returns
     ``(tokens [N] int32, cdf_gap [N] fp32 or None)``.
     """
+    r = (_binding or _load_binding()).mixed_sample(draft_logits, target_logits, uniforms, beta, temperature, tokens,
+                                                   cdf_gap, status, stream)
+    if r is not None:
+        return _native("osd_mixed_sample", r)
     lib = load_library()
     dev = _need_cuda(draft_logits, target_logits, uniforms, tokens, cdf_gap, status)
     N, V, ds = _rows_2d(draft_logits)
@@ -374,6 +418,10 @@ def osd_verify_tree(draft_logits: Optional[torch.Tensor], target_logits: torch.T
     -1); ``tokens`` [B, n_nodes] int32; ``uniforms`` [B, n_nodes] fp32.  At
     temperature 0 the draft logits and uniforms may be None.
     """
+    r = (_binding or _load_binding()).verify_tree(draft_logits, target_logits, parent, tokens, uniforms, temperature,
+                                                  diagnostics, workspace, out, stream)
+    if r is not None:
+        return _native("osd_verify_tree", r)
     lib = load_library()
     B, n, V = target_logits.shape
     dev = _need_cuda(draft_logits, target_logits, tokens, uniforms, workspace, *(out or ()))
