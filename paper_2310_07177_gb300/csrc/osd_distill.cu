@@ -258,6 +258,7 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
     const int csize = p.csize;
     const float c = p.c, inv_tau = p.inv_tau;
     const int rank = (csize > 1) ? static_cast<int>(cluster_rank()) : 0;
+    grid_dependency_sync();
     long long row = blockIdx.x / csize;  // the launch row; from here on, the output row
     long long g, pp;
     const int V = p.V;
@@ -790,6 +791,7 @@ struct TmShape {
     int n8, n2;
     int run;
     int piece2, piece1;  // rows of the two kinds of tail pieces (2 and 1; 6 and 3 under a mask)
+    int early;           // launched to start before the previous kernel ends
 };
 
 // This thread's chunks of a span held in tensor memory: slot s is chunk
@@ -967,6 +969,9 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
     __shared__ float4 s_slot[kW];  // the warps' values of the exchange in progress
     __shared__ float4 s_res;       // its merged result ...
     __shared__ int s_rerr;         // ... and whether a wait for it gave up
+    // TVD off the 16-byte grid: sign(q - p) = sign((z - gz) - (t - gt) - s_kap)
+    constexpr bool kSign = kTvd && kAnyPhase;
+    [[maybe_unused]] __shared__ float s_kap;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int csize = p.csize;
@@ -1008,6 +1013,7 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
         __syncthreads();
     }
     tm_fence_after_sync();
+    if (tsh.early) grid_dependency_sync();
     const uint32_t tw = s_taddr + (static_cast<uint32_t>(32 * warp) << 16);
 
     uint32_t pph = 0;      // pbar1 and pbar2: one phase per row
@@ -1306,6 +1312,9 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                 },
                 [&](float4 m, bool& bad) {  // -> (gz, gt, cu, cv)
                     bad = m.y < 0.f;
+                    // taken from the logits, the sign is as exact as the sums; from q - p it also has
+                    // the rounding of both log2 E, whose magnitude is 10 and more
+                    if (kSign && lane == 0) s_kap = (logf(m.y / m.w) - kLn2 * (fold_err(m.x) - fold_err(m.z))) / inv_tau;
                     return make_float4(m.x, m.z, -log2_sum(m.w) + fold_err(m.z), -log2_sum(m.y) + fold_err(m.x));
                 }, failed);
             row_err = failed;
@@ -1322,6 +1331,8 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                 continue;
             }
             {
+                if constexpr (kSign) __syncwarp();  // (warp 0 wrote s_kap itself)
+                [[maybe_unused]] const float2 kap2 = f2(kSign ? s_kap : 0.f);
                 // ---- pass 2: divergence terms with the global normalisers.  TVD: A = sum
                 // |q - p|, S = sum q' with q' = q sign(q - p) (kept in tensor memory in
                 // place of the chunk's logits) and Q = sum q; JSD: KL(p||m) and KL(q||m) in bits
@@ -1336,14 +1347,15 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
 #pragma unroll
                             for (int e = 0; e < kCnt; e += 2) {
                                 const bool two = (e + 1 < kCnt);
-                                float2 u, v;
+                                float2 td, zd;
                                 if constexpr (kRaw) {
-                                    u = fma2(bf16x2_minus(tw4[e / 2], gt), f2(c), f2(cu));
-                                    v = fma2(bf16x2_minus(zw[e / 2], gz), f2(c), f2(cv));
+                                    td = bf16x2_minus(tw4[e / 2], gt);
+                                    zd = bf16x2_minus(zw[e / 2], gz);
                                 } else {
-                                    u = fma2(sub2(make_float2(t[e], two ? t[e + 1] : t[e]), f2(gt)), f2(c), f2(cu));
-                                    v = fma2(sub2(make_float2(z[e], two ? z[e + 1] : z[e]), f2(gz)), f2(c), f2(cv));
+                                    td = sub2(make_float2(t[e], two ? t[e + 1] : t[e]), f2(gt));
+                                    zd = sub2(make_float2(z[e], two ? z[e + 1] : z[e]), f2(gz));
                                 }
+                                const float2 u = fma2(td, f2(c), f2(cu)), v = fma2(zd, f2(c), f2(cv));
                                 const float2 pj = make_float2(ex2(u.x), ex2(u.y)), qj = make_float2(ex2(v.x), ex2(v.y));
                                 if constexpr (kJsd) {
                                     // m plus the smallest normal: equal to m above about 2^-102, and
@@ -1356,7 +1368,8 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                                     B2 = fma2(qw, sub2(v, lm), B2);
                                 } else {
                                     const float2 df = sub2(qj, pj);
-                                    const float2 qq = make_float2(copysignf(qj.x, df.x), copysignf(qj.y, df.y));
+                                    const float2 sd = kSign ? sub2(sub2(zd, td), kap2) : df;
+                                    const float2 qq = make_float2(copysignf(qj.x, sd.x), copysignf(qj.y, sd.y));
                                     qs[e] = qq.x;
                                     if (two) qs[e + 1] = qq.y;
                                     A2.x += fabsf(df.x);
@@ -1529,7 +1542,8 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                 [&](const float* z, const float* t, auto tag, int j0, float, float, bool, uint4& zr, uint4& tr) {
                     constexpr int kCnt = decltype(tag)::value;
                     // RKL's bf16 chunks take x - m from the packed words (mixed-precision subtracts)
-                    constexpr bool kRaw = sizeof(In) == 2 && kCnt == 8;
+                    // (FKL with kAnyPhase, which would spill, takes the unpacked ones: 4096 x 32001 183 -> 176 us)
+                    constexpr bool kRaw = sizeof(In) == 2 && kCnt == 8 && !(kFkl && kAnyPhase);
                     const uint32_t zw[4] = {zr.x, zr.y, zr.z, zr.w}, tw4[4] = {tr.x, tr.y, tr.z, tr.w};
                     auto zdiff = [&](int e, float m) {
                         if constexpr (kRaw) return bf16x2_minus(zw[e / 2], m);
@@ -1639,8 +1653,7 @@ static cudaError_t launch_distill_kind(const DistParams& dp, long long rows, siz
             }
         }
     }
-    return launch(kern, dim3(static_cast<unsigned>(rows * dp.csize)), dim3(kT), smem, s,
-                  dp.csize, dp);
+    return launch_ex(true, kern, dim3(static_cast<unsigned>(rows * dp.csize)), dim3(kT), smem, s, dp.csize, dp);
 }
 
 // (TVD, whose extra cluster exchange costs more with wide CTAs, always takes kDistThreads.)
@@ -1705,7 +1718,7 @@ static cudaError_t tm_launch_shape(int span, int csize, TmLaunch* out) {
         std::lock_guard<std::mutex> lock(mu);
         for (int i = 0; i < n_cache; ++i)
             if (cache[i].dev == dev && cache[i].span == span && cache[i].csize == csize) {
-                out->shape = TmShape{slots, t_off, ncols, 0, 0, 0, 0, 0, 2, 1};
+                out->shape = TmShape{slots, t_off, ncols, 0, 0, 0, 0, 0, 2, 1, 0};
                 out->smem = cache[i].smem;
                 out->occ = cache[i].occ;
                 out->clusters = cache[i].clusters;
@@ -1794,7 +1807,7 @@ static cudaError_t tm_launch_shape(int span, int csize, TmLaunch* out) {
         std::lock_guard<std::mutex> lock(mu);
         if (n_cache < 64) cache[n_cache++] = Entry{dev, span, csize, smem, occ, clusters};
     }
-    out->shape = TmShape{slots, t_off, ncols, 0, 0, 0, 0, 0, 2, 1};
+    out->shape = TmShape{slots, t_off, ncols, 0, 0, 0, 0, 0, 2, 1, 0};
     out->smem = smem;
     out->occ = occ;
     out->clusters = clusters;
@@ -1838,7 +1851,11 @@ static cudaError_t launch_distill_tm(const DistParams& dp, long long rows, cudaS
     sh.n2 = static_cast<int>((twos + sh.piece2 - 1) / sh.piece2);
     const long long n1 = (ones + sh.piece1 - 1) / sh.piece1;
     const long long runs = sh.n8 + sh.n2 + n1;
-    return launch(distill_tm_kernel<In, kKind, kAnyPhase>, dim3(static_cast<unsigned>(runs * dp.csize)),
+    // A start before the previous kernel's end (grid_dependency_sync) gains 2 to 7 us a call,
+    // but costs a long flush 0.9 % (65536 x 32000 RKL, one after another: 2517 against 2496 us;
+    // 16384 x 32128 masked 0.2 %; 2048 x 128256, 43 K rows, gains 1.8 %)
+    sh.early = rows < 64 * K;
+    return launch_ex(sh.early != 0, distill_tm_kernel<In, kKind, kAnyPhase>, dim3(static_cast<unsigned>(runs * dp.csize)),
                   dim3(kTmThreads), tl.smem, s, dp.csize, dp, sh);
 }
 template <typename In, bool kAnyPhase>

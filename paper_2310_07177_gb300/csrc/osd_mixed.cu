@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(32 * kWarps, 64 / kWarps) mixed_sample_kernel(
     __shared__ Piece s_piece[kWarps * kPieces];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    grid_dependency_sync();
     const long long row = blockIdx.x;
     const In* zrow = static_cast<const In*>(p.draft) + row * p.dstride;
     const In* trow = static_cast<const In*>(p.target) + row * p.tstride;
@@ -359,9 +360,9 @@ extern "C" osd_status osd_mixed_sample(const void* draft_logits, const void* tar
         const dim3 grid(static_cast<unsigned>(N));
         const int steps = V / (32 * Elem<In>::kVec);
         const int ww = steps > 256 && N <= (steps > 400 ? 16 : 4) * sms ? 32 : (steps > 24 && N <= 4 * sms ? 16 : 4);
-        if (ww == 32) return launch(mixed_sample_kernel<In, kMode, 32>, grid, dim3(1024), 0, s, 1, mp);
-        if (ww == 16) return launch(mixed_sample_kernel<In, kMode, 16>, grid, dim3(512), 0, s, 1, mp);
-        return launch(mixed_sample_kernel<In, kMode, 4>, grid, dim3(128), 0, s, 1, mp);
+        if (ww == 32) return launch_ex(true, mixed_sample_kernel<In, kMode, 32>, grid, dim3(1024), 0, s, 1, mp);
+        if (ww == 16) return launch_ex(true, mixed_sample_kernel<In, kMode, 16>, grid, dim3(512), 0, s, 1, mp);
+        return launch_ex(true, mixed_sample_kernel<In, kMode, 4>, grid, dim3(128), 0, s, 1, mp);
     };
     auto go = [&](auto tag) {
         if (vec) return go_warps(tag, std::integral_constant<int, kMixAligned>());

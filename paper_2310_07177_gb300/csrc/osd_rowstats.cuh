@@ -36,7 +36,7 @@ row_argmax_kernel(const In* __restrict__ target, int V, int slice_len, int n_sli
     constexpr int kVec = E::kVec;
     __shared__ MaxIdx red_mi[kStatThreads / 32];
 
-    allow_dependent_launch();  // the consumer of the statistics waits for them in-kernel
+    grid_dependency_sync();  // (the consumer of the statistics waits for them in-kernel too)
     const long long item = blockIdx.x;
     const long long row = item / n_slices;
     const int slice = static_cast<int>(item - row * n_slices);

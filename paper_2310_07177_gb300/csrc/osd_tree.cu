@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kGreedyThreads) tree_greedy_kernel(TreeParams 
         }
     }
     if (bad) return;
-    grid_dependency_wait();  // the row statistics are complete from here on
+    grid_dependency_sync();  // the row statistics are complete from here on
     for (int nd = tid; nd < n; nd += kGreedyThreads) {
         const RowStat* st = p.stats + (size_t(b) * n + nd) * p.n_slices;
         MaxIdx acc{kNegInf, INT_MAX};
@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p, i
         }
         fence_mbarrier_init();
     }
+    grid_dependency_sync();
     // check the tokens and gather the two logits every child's accept test needs
     int bad = 0;
     for (int i = tid; i < n; i += kTreeThreads) {
@@ -625,7 +626,7 @@ static osd_status launch_tree(const TreeParams& base, int B, const void* draft, 
         tp.n_slices = (V + slice_len - 1) / slice_len;
         tp.stats = stats;
         if (rows * tp.n_slices > INT_MAX) return OSD_ERR_UNSUPPORTED;
-        const cudaError_t e = launch(row_argmax_kernel<In>, dim3(unsigned(rows * tp.n_slices)), dim3(kStatThreads), 0, stream,
+        const cudaError_t e = launch_ex(true, row_argmax_kernel<In>, dim3(unsigned(rows * tp.n_slices)), dim3(kStatThreads), 0, stream,
                                      1, static_cast<const In*>(target), V, slice_len, tp.n_slices, stats);
         if (e != cudaSuccess) return OSD_ERR_CUDA;
         return from_cuda(launch_ex(true, tree_greedy_kernel, dim3(unsigned(B)), dim3(kGreedyThreads), 0, stream, 1, tp));
@@ -652,8 +653,8 @@ static osd_status launch_tree(const TreeParams& base, int B, const void* draft, 
     constexpr int sub = 32 * Elem<In>::kVec;
     const size_t smem = size_t((tp.span + sub - 1) / sub) * sizeof(float);
     const bool aligned = aligned_to(draft, 16) && aligned_to(target, 16) && ((size_t)V * es) % 16 == 0;
-    return from_cuda(aligned ? launch(tree_walk_kernel<In, true>, grid, dim3(kTreeThreads), smem, stream, tp.csize, tp, win)
-                             : launch(tree_walk_kernel<In, false>, grid, dim3(kTreeThreads), smem, stream, tp.csize, tp, win));
+    return from_cuda(aligned ? launch_ex(true, tree_walk_kernel<In, true>, grid, dim3(kTreeThreads), smem, stream, tp.csize, tp, win)
+                             : launch_ex(true, tree_walk_kernel<In, false>, grid, dim3(kTreeThreads), smem, stream, tp.csize, tp, win));
 }
 
 }  // namespace osd

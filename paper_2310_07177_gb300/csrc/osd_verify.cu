@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kGreedyWarps * 32) verify_greedy_kernel(FinPar
         yv[c] = (i < k) ? y[i] : 0;
         bad |= (i < k) && (yv[c] < 0 || yv[c] >= V);
     }
-    grid_dependency_wait();  // the row statistics are complete from here on
+    grid_dependency_sync();  // the row statistics are complete from here on
     // row i <= k of the sequence: its target argmax, lowest index on ties, merged
     // from the slices by the lane that owns the row
     int idx[kC];
@@ -591,7 +591,10 @@ verify_lazy_kernel(FinParams p, int win, int ahead) {
         if constexpr (kStaged)
             for (int q = 0; q < kLazyMaxRows; ++q) mbar_init_only(&s_rbar[q], 1);
         fence_mbarrier_init();
-        if constexpr (kStaged) {
+    }
+    grid_dependency_sync();
+    if constexpr (kStaged) {
+        if (tid == 0) {
             const uint32_t bytes = static_cast<uint32_t>(n * sizeof(In));  // a multiple of 16 on this path
             for (int q = 0; q < rows_of(0, w0); ++q) {
                 mbar_arrive_expect_tx(&s_rbar[q], bytes);
@@ -741,6 +744,9 @@ __global__ void __launch_bounds__(kFuseThreads) verify_fused_kernel(FinParams p)
         mbar_init_only(&s_bar, 1);
         mbar_init_only(&ds.tbar, 1);
         fence_mbarrier_init();
+    }
+    grid_dependency_sync();
+    if (tid == 0) {
         for (int q = 0; q < nrows; ++q) {
             mbar_arrive_expect_tx(&rbar[q], bytes);
             bulk_g2s(rows + size_t(q) * p.span,
@@ -841,7 +847,7 @@ static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
         const size_t smem = fused_recv_offset(2 * k + 1, fp.span, es) + size_t(fp.csize) * (2 * k + 1) * sizeof(MaxSum);
         if (smem <= kStageMaxSmem &&
             (long long)B * fp.csize <= (long long)device_sms() * ctas_per_sm<verify_fused_kernel<In>, kFuseThreads>(smem))
-            return from_cuda(launch(verify_fused_kernel<In>, dim3(unsigned(B) * unsigned(fp.csize)), dim3(kFuseThreads),
+            return from_cuda(launch_ex(true, verify_fused_kernel<In>, dim3(unsigned(B) * unsigned(fp.csize)), dim3(kFuseThreads),
                                     smem, stream, fp.csize, fp));
     }
     // Rows on demand.  A round costs about 2 us beside its bytes, and positions past the
@@ -863,7 +869,7 @@ static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
             if (smem > kStageMaxSmem || ctas_per_sm<verify_lazy_kernel<In, true, true>, kStagedThreads>(smem) < 1) continue;
             // so small a second round that its bytes cost nothing if the first one rejects
             const int ahead = pos * std::min(2 * w, kLazyMaxWin) <= 9e6;
-            return from_cuda(launch(verify_lazy_kernel<In, true, true>, dim3(unsigned(B) * unsigned(fp.csize)),
+            return from_cuda(launch_ex(true, verify_lazy_kernel<In, true, true>, dim3(unsigned(B) * unsigned(fp.csize)),
                                     dim3(kStagedThreads), smem, stream, fp.csize, fp, w, ahead));
         }
     }
@@ -877,9 +883,9 @@ static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
     split_vocab(V, c, &fp);
     if ((long long)B * fp.csize > INT_MAX) return OSD_ERR_UNSUPPORTED;
     const dim3 grid(unsigned(B) * unsigned(fp.csize));
-    return from_cuda(aligned ? launch(verify_lazy_kernel<In, false, true>, grid, dim3(kLazyThreads), sub_bytes(), stream,
+    return from_cuda(aligned ? launch_ex(true, verify_lazy_kernel<In, false, true>, grid, dim3(kLazyThreads), sub_bytes(), stream,
                                       fp.csize, fp, win, 0)
-                             : launch(verify_lazy_kernel<In, false, false>, grid, dim3(kLazyThreads), sub_bytes(), stream,
+                             : launch_ex(true, verify_lazy_kernel<In, false, false>, grid, dim3(kLazyThreads), sub_bytes(), stream,
                                       fp.csize, fp, win, 0));
 }
 
@@ -902,7 +908,7 @@ static osd_status launch_verify(const void* draft, const void* target, int B, in
         const long long grid1 = (long long)B * (k + 1) * fp.n_slices;
         if (grid1 > INT_MAX) return OSD_ERR_UNSUPPORTED;
         const cudaError_t e =
-            launch(row_argmax_kernel<In>, dim3(unsigned(grid1)), dim3(kStatThreads), 0, stream, 1,
+            launch_ex(true, row_argmax_kernel<In>, dim3(unsigned(grid1)), dim3(kStatThreads), 0, stream, 1,
                    static_cast<const In*>(target), V, slice_len, fp.n_slices, stats);
         if (e != cudaSuccess) return OSD_ERR_CUDA;
         fp.csize = 1;

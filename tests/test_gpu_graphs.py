@@ -81,3 +81,78 @@ def test_graph_replay_matches_eager(osd):
     assert torch.equal(tok, etok)
     for f in ("accepted", "path", "out_tokens", "last_node"):
         assert torch.equal(getattr(gt, f), getattr(et, f)), f
+
+
+def _chain(osd, z, t, y, u, sync):
+    """Calls back to back that read what the one before wrote (gradients as logits, accepted
+    counts) and write over what it read, small enough that each starts as the last one ends."""
+    g = [torch.zeros_like(z, dtype=torch.float32) for _ in range(2)]
+    t32, w = t.float(), t.clone()
+    rej = osd.DistillAcceptedResult(torch.zeros(3, device="cuda"), torch.zeros(3, z.shape[2], device="cuda"),
+                                    torch.zeros(3, dtype=torch.int32, device="cuda"),
+                                    torch.zeros(1, dtype=torch.int32, device="cuda"))
+    out = []
+    for i in range(12):
+        kind = ("fkl", "rkl", "jsd", "tvd", "ce")[i % 5]
+        osd.osd_distill(z, w[:, :-1], loss_kind=kind, dlogits=g[0])
+        sync()
+        osd.osd_distill(g[0], t32[:, :-1], loss_kind=kind, temperature=0.01, dlogits=g[1])  # reads g0 ...
+        sync()
+        osd.osd_distill(z, w[:, :-1], loss_kind="ce", dlogits=g[0])                            # ... and writes it
+        sync()
+        r = osd.osd_verify(z, w, y, u, 1.0, diagnostics=False)
+        sync()
+        osd.osd_distill_accepted(z, w, r.accepted, kind, out=rej)
+        sync()
+        tok, _ = osd.osd_mixed_sample(g[0][:, 0], g[1][:, 0], u[:, 0].contiguous(), 0.5, temperature=0.01)
+        sync()
+        r0 = osd.osd_verify(None, w, y, None, 0.0, diagnostics=False)
+        sync()
+        w.copy_(t).mul_(1.0 - 0.05 * i)  # other kernels write the logits between
+        out += [g[0].clone(), g[1].clone(), r.out_tokens, rej.dlogits.clone(), rej.count.clone(), tok, r0.out_tokens]
+    torch.cuda.synchronize()
+    return out
+
+
+def test_dependent_calls_back_to_back(osd):
+    inp = W.verify_inputs(W.VerifySpec(3, 2, 2048, torch.bfloat16, 2.0, 1.0, 0.8, 1.0), seed=5)
+    z, t, y, u = (inp[k].cuda() for k in ("draft", "target", "tokens", "uniforms"))
+    a = _chain(osd, z, t, y, u, lambda: None)
+    b = _chain(osd, z, t, y, u, torch.cuda.synchronize)
+    assert len(a) == len(b)
+    for i, (p, q) in enumerate(zip(a, b)):
+        assert torch.equal(p, q), i
+
+
+def test_capture_with_forked_streams_and_status(osd):
+    """Captured calls that follow a memset (the status), an event of another stream, or a
+    join of two streams: a graph's edges are then not between two kernels alone."""
+    inp = W.verify_inputs(W.VerifySpec(3, 2, 4096, torch.bfloat16, 2.0, 1.0, 0.8, 1.0), seed=6)
+    z, t, y, u = (inp[k].cuda() for k in ("draft", "target", "tokens", "uniforms"))
+    st = torch.full((1,), 7, dtype=torch.int32, device="cuda")
+    ga, gb = torch.zeros(3, 2, 4096, device="cuda"), torch.zeros(3, 2, 4096, device="cuda")
+    other = torch.cuda.Stream()
+
+    def step():
+        main = torch.cuda.current_stream()
+        other.wait_stream(main)
+        with torch.cuda.stream(other):
+            osd.osd_distill(z, t[:, :2], loss_kind="jsd", dlogits=gb)
+            r0 = osd.osd_verify(None, t, y, None, 0.0)
+        osd.osd_distill(z, t[:, :2], loss_kind="rkl", dlogits=ga, status=st)
+        main.wait_stream(other)
+        l, g = osd.osd_distill(gb, ga, loss_kind="fkl", temperature=0.01)
+        return r0, osd.osd_verify(z, t, y, u, 1.0), l, g
+    e0, e1, el, eg = step()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        c0, c1, cl, cg = step()
+    for x in (ga, gb):
+        x.zero_()
+    st.fill_(7)
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert int(st) == 0 and torch.equal(el, cl) and torch.equal(eg, cg)
+    assert torch.equal(e0.out_tokens, c0.out_tokens) and torch.equal(e1.out_tokens, c1.out_tokens)
