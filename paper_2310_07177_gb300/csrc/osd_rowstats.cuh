@@ -9,6 +9,7 @@
 #include <cstdint>
 
 #include "osd_device.cuh"
+#include "osd_host.hpp"
 
 namespace osd {
 
@@ -222,6 +223,191 @@ __device__ __forceinline__ float warp_sum4(const float (&sum)[4]) {
     tot += __shfl_xor_sync(0xffffffffu, mid ? s01 : s23, 8);
     for (int o = 4; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
     return tot;
+}
+
+// ------------------------------------------------------------------ T = 0, rows on demand
+// A greedy walk reads a target row only to compare its argmax with the tokens that may
+// follow; large batches therefore walk as the samplers do, one cluster per sequence,
+// in rounds of a node and the next ones down the walk's likeliest way, four times as
+// many after each round.  `Walk` (a kernel parameter) is the chain of a
+// draft or a token tree:
+//   node_ok(b)          (every thread, strided) whether sequence b's tokens all lie in [0, V)
+//   row(b, node)        the node's row among the target rows
+//   next(node)          the likeliest child, -1 at a leaf
+//   child(b, node, x)   the child whose token is x, -1 if none
+//   step(b, depth, child), finish(b, depth, node, x), bad(b): the outputs (one CTA; the
+//                       last two by every thread of it)
+constexpr int kWalkThreads = 256;
+constexpr int kWalkMaxWin = 8;  // nodes per round, a warp or more each
+
+// First argmax of the entries p[0, n) (entry 0 has index j0), shared out as in span_stats.
+template <typename In>
+__device__ __forceinline__ MaxIdx span_argmax(const In* p, int n, int j0, int part, int parts) {
+    using E = Elem<In>;
+    constexpr int kVec = E::kVec;
+    const int lane = threadIdx.x & 31;
+    int head = static_cast<int>(((16u - (reinterpret_cast<uintptr_t>(p) & 15u)) & 15u) / sizeof(In));
+    if (head > n) head = n;
+    const int nvec = (n - head) / kVec;
+    const int tail0 = head + nvec * kVec;
+    const In* body = p + head;
+    MaxIdx acc{kNegInf, INT_MAX};
+    auto take = [&](float x, int j) {
+        if (x > acc.m) acc = MaxIdx{x, j};
+    };
+    const int step = 32 * parts;
+    auto load_group = [&](int v, uint4* r) {
+#pragma unroll
+        for (int u = 0; u < kSpanUnroll; ++u) {
+            const int vv = v + u * step;
+            r[u] = (vv < nvec) ? ldg_stream(body + size_t(vv) * kVec) : ninf_raw<In>();
+        }
+    };
+    auto absorb = [&](int v, const uint4* r) {
+        float cm = E::max_raw(r[0]);
+#pragma unroll
+        for (int u = 1; u < kSpanUnroll; ++u) cm = fmaxf(cm, E::max_raw(r[u]));
+        if (cm > acc.m) {  // rare: find the first entry equal to the group maximum
+#pragma unroll
+            for (int u = 0; u < kSpanUnroll; ++u) {
+                float x[kVec];
+                E::unpack(r[u], x);
+#pragma unroll
+                for (int e = 0; e < kVec; ++e) take(x[e], j0 + head + (v + u * step) * kVec + e);
+            }
+        }
+    };
+    if (part == 0 && lane < head) take(E::load(p + lane), j0 + lane);
+    uint4 ra[kSpanUnroll], rb[kSpanUnroll];
+    const int stride = kSpanUnroll * step;
+    int v = part * 32 + lane;
+    if (v < nvec) load_group(v, ra);
+    for (; v < nvec; v += 2 * stride) {
+        if (v + stride < nvec) load_group(v + stride, rb);
+        absorb(v, ra);
+        if (v + stride >= nvec) break;
+        if (v + 2 * stride < nvec) load_group(v + 2 * stride, ra);
+        absorb(v + stride, rb);
+    }
+    if (part == parts - 1 && lane < n - tail0) take(E::load(p + tail0 + lane), j0 + tail0 + lane);
+    return warp_reduce(acc, [](MaxIdx a, MaxIdx b) { return merge_mi(a, b); });
+}
+
+template <typename In, typename Walk>
+__global__ void __launch_bounds__(kWalkThreads, 4)
+greedy_walk_kernel(Walk wk, const In* target, int V, int csize, int span, int win) {
+    constexpr int kWarps = kWalkThreads / 32;
+    __shared__ MaxIdx s_part[kWarps];
+    __shared__ __align__(8) MaxIdx s_recv[2][kSeqMaxCluster * kWalkMaxWin];  // [CTA][node], two rounds
+    __shared__ __align__(8) uint64_t s_bar[2];
+    __shared__ int s_best[kWalkMaxWin];
+    __shared__ int s_node, s_depth, s_state;  // state: 0 another round, 1 done, 2 a wait gave up
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = (csize > 1) ? static_cast<int>(cluster_rank()) : 0;
+    const int b = blockIdx.x / csize;
+    const int e0 = rank * span, n = min(span, V - e0);
+    if (tid == 0) {
+        mbar_init_only(&s_bar[0], 1);
+        mbar_init_only(&s_bar[1], 1);
+        fence_mbarrier_init();
+        s_node = 0;
+        s_depth = 0;
+    }
+    grid_dependency_sync();
+    const int bad = wk.node_ok(b) ? 0 : 1;
+    if (__syncthreads_or(bad)) {  // uniform over the cluster, before any push to a peer
+        if (rank == 0) wk.bad(b);
+        return;
+    }
+    // the barriers are initialised before any peer pushes to them: arrive now, wait before the first push
+    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    for (unsigned round = 0;; ++round) {
+        const int node = s_node;
+        int w = 1;
+        for (int nd = wk.next(node); nd >= 0 && w < win; nd = wk.next(nd)) ++w;
+        const int parts = kWarps / w;
+        const int q = warp / parts;
+        if (q < w) {
+            int nd = node;
+            for (int i = 0; i < q; ++i) nd = wk.next(nd);
+            const MaxIdx mine = span_argmax<In>(target + wk.row(b, nd) * V + e0, n, e0, warp - q * parts, parts);
+            if (lane == 0) s_part[warp] = mine;
+        }
+        __syncthreads();
+        if (round == 0 && csize > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (warp == 0) {
+            const unsigned buf = round & 1u;
+            MaxIdx* recv = s_recv[buf];
+            bool gone = false;
+            MaxIdx acc{kNegInf, INT_MAX};
+            if (lane < w) {
+                for (int x = 0; x < parts; ++x) acc = merge_mi(acc, s_part[lane * parts + x]);
+                for (int c = 0; c < csize && csize > 1; ++c)
+                    st_async_v2(map_rank(&recv[rank * kWalkMaxWin + lane], static_cast<uint32_t>(c)),
+                                make_float2(acc.m, __int_as_float(acc.i)), map_rank(&s_bar[buf], static_cast<uint32_t>(c)));
+            }
+            if (csize > 1) {
+                if (lane == 0) mbar_arrive_expect_tx(&s_bar[buf], static_cast<uint32_t>(csize * w) * 8u);
+                gone = !mbar_wait_cluster_bounded(&s_bar[buf], (round >> 1) & 1u, kPeerWaitNs);
+                acc = MaxIdx{kNegInf, INT_MAX};
+                if (!gone && lane < w)
+                    for (int c = 0; c < csize; ++c) acc = merge_mi(acc, recv[c * kWalkMaxWin + lane]);
+            }
+            if (lane < w) s_best[lane] = acc.i == INT_MAX ? 0 : acc.i;
+            gone = __any_sync(0xffffffffu, gone);
+            __syncwarp();
+            if (lane == 0) {
+                int nd = node, depth = s_depth, state = gone ? 2 : 1;
+                for (int i = 0; i < w && state == 1; ++i) {
+                    const int ch = wk.child(b, nd, s_best[i]);
+                    if (ch < 0) {
+                        s_best[0] = s_best[i];  // the walk ends at nd, with its argmax as the extra token
+                        break;
+                    }
+                    if (rank == 0) wk.step(b, depth, ch);
+                    ++depth;
+                    if (i + 1 == w || ch != wk.next(nd)) state = 0;
+                    nd = ch;
+                }
+                s_node = nd;
+                s_depth = depth;
+                s_state = state;
+            }
+        }
+        __syncthreads();
+        if (s_state) {
+            if (s_state == 2 && csize > 1 && tid == 0)
+                mbar_wait_cluster_bounded(&s_bar[round & 1u], (round >> 1) & 1u, kPeerWaitNs);
+            break;
+        }
+        win = min(4 * win, kWalkMaxWin);
+    }
+    if (rank != 0) return;
+    if (s_state == 2) wk.bad(b);  // the peers' argmaxes did not arrive in time: reported as bad
+    else wk.finish(b, s_depth, s_node, s_best[0]);
+}
+
+// Launch a greedy walk over B sequences of `rows` rows each, at most `depth` of them on any
+// walk, or return false where the pass over every row does better: that one reads at the copy
+// bandwidth, a walk pays about 2.5 us a round.  Trees, of which a walk sees the smaller part,
+// from 20 MB and a CTA an SM on (27 nodes: 16 x 32000 9.0 -> 5.6 us, 64 x 100000 58.5 -> 17,
+// 48 x 128256 fp32 96 -> 21; 2 x 135808 fp32 10.2 against 12.4); chains only where one position is 40 MB (256 x 9 x 128256: 90.5 us, on demand 32 with
+// 0.15 accepted, 59 with 1.7 and 98 with 6.4; 32 x 9 x 128256, 8 MB: 16.6 against 16 and 23).
+template <typename In, typename Walk>
+static bool launch_greedy_walk(const Walk& wk, const In* target, int B, int rows, int depth, int V, cudaStream_t stream,
+                               osd_status* st) {
+    const double pos = double(B) * V * double(sizeof(In));  // bytes of one node of the batch
+    if (pos < 40e6 && (B < 8 || rows < 2 * depth || pos * rows < 20e6)) return false;
+    const int win = pos <= 4e6 ? 4 : (pos <= 16e6 ? 2 : 1);
+    int c = kSeqMaxCluster;
+    while (c > 1 && (V <= 2048 * c || ((long long)B * c / 2 >= 3LL * device_sms() && size_t(V / (c / 2)) * sizeof(In) <= 68 * 1024)))
+        c /= 2;
+    const int span = ((V + c - 1) / c + 63) / 64 * 64;
+    const int csize = (V + span - 1) / span;
+    if ((long long)B * csize > INT_MAX) return false;
+    *st = from_cuda(launch_ex(true, greedy_walk_kernel<In, Walk>, dim3(unsigned(B) * unsigned(csize)), dim3(kWalkThreads), 0,
+                              stream, csize, wk, target, V, csize, span, win));
+    return true;
 }
 
 }  // namespace osd

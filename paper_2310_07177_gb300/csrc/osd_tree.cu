@@ -13,8 +13,10 @@
 // sub-tile sums of the last pass, as the verifier draws its residual token (masses
 // summed in exact 64-bit fixed point).  Only the rows the walk comes to are read.
 //
-// T = 0: two launches, row_argmax_kernel (osd_rowstats.cuh) over every target row's
-// slices and tree_greedy_kernel, which follows the matching children.
+// T = 0: greedy_walk_kernel (osd_rowstats.cuh), which reads the target rows of the
+// matching children on its way; where the tree is small or little more than a
+// chain, two launches, row_argmax_kernel over every target row's slices and
+// tree_greedy_kernel, which follows the matching children.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -111,6 +113,46 @@ __global__ void __launch_bounds__(kGreedyThreads) tree_greedy_kernel(TreeParams 
     p.accepted[b] = depth;
     p.last_node[b] = node;
 }
+
+// The same walk on demand (osd_rowstats.cuh).
+struct GreedyTree {
+    TreeParams p;
+    __device__ bool node_ok(int b) const {
+        bool ok = true;
+        for (int i = 1 + threadIdx.x; i < p.n; i += kWalkThreads) {
+            const int y = p.tokens[size_t(b) * p.n + i];
+            ok = ok && y >= 0 && y < p.V;
+        }
+        return ok;
+    }
+    __device__ size_t row(int b, int nd) const { return size_t(b) * p.n + nd; }
+    __device__ int next(int nd) const { return p.topo.first_child[nd]; }
+    __device__ int child(int b, int nd, int x) const {
+        for (int c = p.topo.first_child[nd]; c >= 0; c = p.topo.next_sibling[c])
+            if (p.tokens[size_t(b) * p.n + c] == x) return c;
+        return -1;
+    }
+    __device__ void step(int b, int depth, int c) const {
+        p.path[size_t(b) * p.n + depth] = c;
+        p.out_tokens[size_t(b) * p.n + depth] = p.tokens[size_t(b) * p.n + c];
+    }
+    __device__ void finish(int b, int depth, int nd, int x) const {
+        for (int i = threadIdx.x; i < p.n; i += kWalkThreads) {
+            if (i >= depth) p.path[size_t(b) * p.n + i] = -1;
+            if (i >= depth) p.out_tokens[size_t(b) * p.n + i] = i == depth ? x : -1;
+            if (p.diag_margin) p.diag_margin[size_t(b) * p.n + i] = __int_as_float(0x7fc00000);
+        }
+        if (threadIdx.x == 0) {
+            p.accepted[b] = depth;
+            p.last_node[b] = nd;
+            if (p.diag_gap) p.diag_gap[b] = __int_as_float(0x7fc00000);
+        }
+    }
+    __device__ void bad(int b) const {
+        finish(b, 0, -1, -1);
+        if (threadIdx.x == 0) p.accepted[b] = -1;
+    }
+};
 
 // T > 0.  Each CTA owns a span of the vocabulary.  A round takes the rows of a node and of
 // the `win` - 1 next ones down its first children (the likeliest way on).  The span
@@ -621,6 +663,10 @@ static osd_status launch_tree(const TreeParams& base, int B, const void* draft, 
     const int n = tp.n, V = tp.V;
     constexpr size_t es = sizeof(In);
     if (tp.T == 0.f) {
+        osd_status st = OSD_OK;
+        int level[OSD_TREE_MAX_NODES] = {1}, depth = 1;  // rows of the longest walk
+        for (int i = 1; i < n; ++i) depth = std::max(depth, level[i] = level[tp.topo.parent[i]] + 1);
+        if (launch_greedy_walk<In>(GreedyTree{tp}, static_cast<const In*>(target), B, n, depth, V, stream, &st)) return st;
         const long long rows = tree_stat_rows(B, n, true);
         const int slice_len = stats_slice_len(rows);
         tp.n_slices = (V + slice_len - 1) / slice_len;

@@ -19,7 +19,7 @@
 //
 // T = 0: two launches, row_argmax_kernel (the argmax of every target row's slices) and
 // verify_greedy_kernel, one warp per sequence: the matches in order, the target
-// argmax at the first mismatch.
+// argmax at the first mismatch; large batches walk on demand (greedy_walk_kernel).
 //
 // The log-ratio of the accept test is formed from differences of raw logits and
 // maxima, (t_y - m_t) - (z_y - m_z), and the ratio of the two sums, so no
@@ -127,6 +127,36 @@ __global__ void __launch_bounds__(kGreedyWarps * 32) verify_greedy_kernel(FinPar
     }
 }
 
+// The same walk on demand (osd_rowstats.cuh): position i follows position i - 1 by draft token i - 1.
+struct GreedyChain {
+    FinParams p;
+    __device__ bool node_ok(int b) const {
+        bool ok = true;
+        for (int i = threadIdx.x; i < p.k; i += kWalkThreads) {
+            const int y = p.tokens[size_t(b) * p.k + i];
+            ok = ok && y >= 0 && y < p.V;
+        }
+        return ok;
+    }
+    __device__ size_t row(int b, int i) const { return size_t(b) * (p.k + 1) + i; }
+    __device__ int next(int i) const { return i < p.k ? i + 1 : -1; }
+    __device__ int child(int b, int i, int x) const { return i < p.k && p.tokens[size_t(b) * p.k + i] == x ? i + 1 : -1; }
+    __device__ void step(int, int, int) const {}
+    __device__ void finish(int b, int a, int, int x) const {
+        if (threadIdx.x == 0) {
+            p.accepted[b] = a;
+            if (p.diag_gap) p.diag_gap[b] = __int_as_float(0x7fc00000);
+        }
+        for (int i = threadIdx.x; i <= p.k; i += kWalkThreads)
+            p.out_tokens[size_t(b) * (p.k + 1) + i] = i < a ? p.tokens[size_t(b) * p.k + i] : (i == a ? x : -1);
+        for (int i = threadIdx.x; i < p.k; i += kWalkThreads) {
+            p.mask[size_t(b) * p.k + i] = i == a ? 1 : 0;
+            if (p.diag_margin) p.diag_margin[size_t(b) * p.k + i] = __int_as_float(0x7fc00000);
+        }
+    }
+    __device__ void bad(int b) const;
+};
+
 // Shared memory of one sequence's decision: the merged statistics of its 2k+1
 // rows (local row r <= k is target row r, r > k is draft row r-k-1), the draft
 // tokens, the two logits each accept test needs, the uniforms, and a.
@@ -150,6 +180,7 @@ __device__ __forceinline__ void seq_write_bad(const FinParams& p, int b) {
         if (p.diag_margin) p.diag_margin[size_t(b) * k + i] = __int_as_float(0x7fc00000);
     }
 }
+__device__ void GreedyChain::bad(int b) const { seq_write_bad<kWalkThreads>(p, b); }
 
 // One round of accept tests, run by warp 0 of every CTA of the cluster alike:
 // positions i0 .. i0 + w - 1, a lane each, the first failing one is a.  Returns
@@ -902,6 +933,8 @@ static osd_status launch_verify(const void* draft, const void* target, int B, in
     fp.accepted = accepted; fp.out_tokens = out_tokens; fp.mask = mask;
     fp.diag_margin = diag_margin; fp.diag_gap = diag_gap;
     if (greedy) {
+        osd_status st = OSD_OK;
+        if (launch_greedy_walk<In>(GreedyChain{fp}, static_cast<const In*>(target), B, k + 1, k + 1, V, stream, &st)) return st;
         const int slice_len = verify_slice_len(B, k);
         fp.n_slices = verify_slices(B, k, V);
         fp.stats = stats;

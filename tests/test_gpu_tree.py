@@ -203,6 +203,10 @@ ROUND_CASES = [  # (parents, B, V, dtype, T, noise)
     (COMB, 48, 9001, torch.float32, 1.0, 0.3),                      # two CTAs a sequence
     (COMB, 64, 50, torch.bfloat16, 1.3, 0.5),                       # one CTA a sequence
     ([-1], 5, 33000, torch.bfloat16, 1.0, 0.5),                     # the root alone: a draw from p
+    # T = 0, on demand from 20 MB of rows on: rounds of 4, of 2, of 1 and then of 4 and 8 nodes
+    (W.MEDUSA_TREE, 12, 33001, torch.bfloat16, 0.0, 0.02),
+    (W.MEDUSA_TREE, 9, 128256, torch.float32, 0.0, 0.02),
+    ([-1] + list(range(12)), 160, 128256, torch.bfloat16, 0.0, 0.02),
 ]
 
 

@@ -345,3 +345,37 @@ def test_unaligned_largest_vocabulary_past_128_sequences(osd):
     assert ((acc >= 0) & (acc <= 1)).all()
     out = res.out_tokens.cpu()
     assert ((out[torch.arange(130), acc.long()] >= 0) & (out[torch.arange(130), acc.long()] < V)).all()
+
+
+# T = 0 on demand: batches of which one position is 40 MB; drafts that pass none, some or all
+# positions, so that walks end in the first round, the second, the third or at the bonus row.
+@pytest.mark.parametrize("B,k,V,dtype", [(64, 9, 160001, torch.float32), (250, 3, 82001, torch.bfloat16),
+                                         (1024, 1, 20480, torch.bfloat16)])
+def test_greedy_on_demand_matches_oracle(osd, B, k, V, dtype):
+    g = torch.Generator(device="cuda").manual_seed(B + V)
+    t = torch.randn(B, k + 1, V, generator=g, device="cuda").mul_(2).round_().div_(2).to(dtype)  # ties everywhere
+    best = torch.where(t == t.amax(-1, keepdim=True), torch.arange(V, device="cuda"), V).amin(-1)
+    y = best[:, :k].to(torch.int32).clone()
+    stop = torch.randint(0, k + 1, (B,), generator=g, device="cuda")
+    for b in range(B):
+        s = int(stop[b])
+        if s < k:
+            y[b, s] = (int(best[b, s]) + 1) % V
+    y[1, k - 1] = V
+    y[2, 0] = -1
+    res = osd.osd_verify(None, t, y, None, 0.0)
+    torch.cuda.synchronize()
+    acc, tok = res.accepted.cpu(), res.out_tokens.cpu()
+    for b in range(B):
+        if b in (1, 2):
+            assert acc[b] == -1 and (tok[b] == -1).all()
+            continue
+        s = int(stop[b])
+        want = [int(x) for x in best[b, :s + 1]] + [-1] * (k - s)
+        assert int(acc[b]) == s and tok[b].tolist() == want, b
+    assert torch.isnan(res.diag_margin).all() and torch.isnan(res.diag_cdf_gap).all()
+    mask = torch.zeros(B, k, dtype=torch.uint8)
+    for b in range(B):
+        if b not in (1, 2) and int(stop[b]) < k:
+            mask[b, int(stop[b])] = 1
+    assert torch.equal(res.mismatch_mask.cpu(), mask)
