@@ -72,6 +72,37 @@ static int ctas_per_sm(size_t smem) {
     return occ;
 }
 
+// The largest cluster size of 1 .. `most` of which `clusters` run at the same time when each
+// CTA takes `smem` bytes of dynamic shared memory (a fixed figure per kern), 0 if none: the
+// SMs of a cluster lie in one GPC, so fewer fit than the SMs' own count says.  `spare`: of
+// sizes above 2, with a 32nd of the slots to spare.  Kept per device.
+template <auto kern, int kThreads>
+static int widest_cluster(long long clusters, int most, size_t smem, bool spare) {
+    constexpr int kMost = 8;
+    static std::atomic<int> fit[64][kMost + 1];  // clusters of a size that run at once, plus 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    for (int c = most < kMost ? most : kMost; c >= 1; --c) {
+        int n = fit[dev][c].load(std::memory_order_relaxed) - 1;
+        if (n < 0) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(static_cast<unsigned>(c));
+            cfg.blockDim = dim3(kThreads);
+            cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr = {};
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = static_cast<unsigned>(c);
+            attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            if (ctas_per_sm<kern, kThreads>(smem) < 1 || cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) return 0;
+            fit[dev][c].store(n + 1, std::memory_order_relaxed);
+        }
+        if (clusters + (spare && c > 2 ? clusters / 31 : 0) <= n) return c;
+    }
+    return 0;
+}
+
 // Launch `kernel` with an optional thread-block cluster of `cluster` CTAs
 // along x (cluster == 1 launches without the attribute); launch_ex can also
 // mark it a programmatic dependent of the previous kernel on the stream.

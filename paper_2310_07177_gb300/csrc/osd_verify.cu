@@ -565,7 +565,7 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
 // CTAs: 84 us); staging the first position in shared memory at these sizes, three CTAs an
 // SM, gave 70 us with the poor draft and 257 us with the good one, whose rounds then wait
 // for their copies.
-constexpr int kLazyMaxWin = 4;               // positions per round ...
+constexpr int kLazyMaxWin = 8;                 // positions per round ...
 constexpr int kLazyMaxRows = 2 * kLazyMaxWin;  // ... two rows each
 constexpr int kLazyThreads = 256;
 constexpr int kStagedThreads = 512;          // with a staged first round: one CTA an SM
@@ -588,7 +588,7 @@ verify_lazy_kernel(FinParams p, int win, int ahead) {
     constexpr int kThreads = kStaged ? kStagedThreads : kLazyThreads, kWarps = kThreads / 32;
     __shared__ SeqSmem sh;
     __shared__ DrawSmem ds;
-    __shared__ MaxSum s_part[kWarps];
+    __shared__ MaxSum s_part[kWarps > kLazyMaxRows ? kWarps : kLazyMaxRows];
     __shared__ __align__(8) MaxSum s_recv[2][kSeqMaxCluster * kLazyMaxRows];  // [CTA][row], two rounds
     __shared__ __align__(8) uint64_t s_bar[2];
     __shared__ __align__(8) uint64_t s_rbar[kLazyMaxRows];  // staged rows
@@ -606,7 +606,7 @@ verify_lazy_kernel(FinParams p, int win, int ahead) {
     const In* target = static_cast<const In*>(p.target) + size_t(b) * (k + 1) * V;
     const float ch = p.c_hi, cl = p.c_lo;
     In* staged = reinterpret_cast<In*>(lsm);
-    float* s_sub = reinterpret_cast<float*>(lsm + (kStaged ? lazy_sub_offset(2 * win, p.span, sizeof(In)) : 0));
+    float* s_sub = reinterpret_cast<float*>(lsm + (kStaged ? lazy_sub_offset(min(2 * win, 2 * p.k + 1), p.span, sizeof(In)) : 0));
     const int w0 = min(win, k + 1);  // positions of the first round
     // row q of the round of w positions from i0: the target rows first, then the draft rows
     // (the bonus position k has none)
@@ -872,45 +872,61 @@ static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
     constexpr size_t es = sizeof(In);
     const bool aligned = aligned_to(fp.target, 16) && aligned_to(fp.draft, 16) && ((size_t)V * es) % 16 == 0;
     if (aligned && B <= kFuseMaxB) {
-        // every row staged, only in one wave: at B = 32, k = 5, V = 32000 (two CTAs an SM) 12.8 us
-        // against 14.7 us on demand; at B = 48, past one wave, it took 34 us (17.8 on demand)
+        // every row staged, only in one wave and with slots to spare, since a grid that just
+        // fits finds them scattered over the GPCs: at B = 32, k = 5, V = 32000 (two CTAs an SM, 256
+        // of 304 slots) 12.8 us against 14.4 us on demand; at B = 36, V = 20224 (288) 16.6 against 10.1
         split_vocab(V, kSeqMaxCluster, &fp);
         const size_t smem = fused_recv_offset(2 * k + 1, fp.span, es) + size_t(fp.csize) * (2 * k + 1) * sizeof(MaxSum);
         if (smem <= kStageMaxSmem &&
-            (long long)B * fp.csize <= (long long)device_sms() * ctas_per_sm<verify_fused_kernel<In>, kFuseThreads>(smem))
+            (long long)B * fp.csize * 8 <= (long long)device_sms() * ctas_per_sm<verify_fused_kernel<In>, kFuseThreads>(smem) * 7)
             return from_cuda(launch_ex(true, verify_fused_kernel<In>, dim3(unsigned(B) * unsigned(fp.csize)), dim3(kFuseThreads),
                                     smem, stream, fp.csize, fp));
     }
     // Rows on demand.  A round costs about 2 us beside its bytes, and positions past the
-    // first failure are read for nothing: the first round takes as many positions as
-    // 200 MB hold, at most 4 (B = 256, V = 128256, 131 MB a position: 1, 76 us with a poor
-    // draft against 93 and 135 us with 2 and 4; B = 64, V = 32000, 8 MB: 4, 17.0 us against 18.0
-    // and 19.0 us with 2 and 1).
+    // first failure are read for nothing: the first round takes 1 position from 40 MB a position
+    // of the batch on (B = 233, V = 27472 fp32, 51 MB: 36.8 us against 41.6 and 46.7 with 2 and 4),
+    // 2 from 10 MB (B = 204, V = 14144 fp32, 23 MB: 38.7 against 43.4 with 4), 4 from 2 MB
+    // (B = 100, V = 23488, 9 MB: 16.6 against 18.6 and 21.0 with 2 and 1), else 8 (B = 51, V = 10944:
+    // 14.4 against 15.4 with 4).
     constexpr int sub = 32 * Elem<In>::kVec;
     auto sub_bytes = [&]() { return size_t((fp.span + sub - 1) / sub) * sizeof(float); };
     const double pos = double(B) * 2 * V * double(es);  // bytes of one position of the batch
-    int win = 1;
-    while (win < kLazyMaxWin && win <= k && pos * win < 100e6) win *= 2;
-    // the first round staged where the batch is at most one CTA an SM, with fewer positions
-    // where they do not fit (B = 16, k = 8, V = 128256, 2 positions: 27 us against 39 us streamed)
-    if (aligned) {
-        split_vocab(V, kSeqMaxCluster, &fp);
-        for (int w = win; w >= 1 && (long long)B * fp.csize <= device_sms(); w /= 2) {
-            const size_t smem = lazy_sub_offset(2 * w, fp.span, es) + sub_bytes();
-            if (smem > kStageMaxSmem || ctas_per_sm<verify_lazy_kernel<In, true, true>, kStagedThreads>(smem) < 1) continue;
-            // so small a second round that its bytes cost nothing if the first one rejects
-            const int ahead = pos * std::min(2 * w, kLazyMaxWin) <= 9e6;
-            return from_cuda(launch_ex(true, verify_lazy_kernel<In, true, true>, dim3(unsigned(B) * unsigned(fp.csize)),
-                                    dim3(kStagedThreads), smem, stream, fp.csize, fp, w, ahead));
+    const int win = pos > 40e6 ? 1 : (pos > 10e6 ? 2 : (pos > 2e6 ? 4 : kLazyMaxWin));
+    const int most = std::max(1, std::min<int>(kSeqMaxCluster, int(size_t(V) * es / 2048)));  // spans of 2 KB or more
+    if (aligned && B <= device_sms() / 2) {
+        // the first round staged where the batch runs at one CTA an SM, with fewer positions
+        // where they do not fit (B = 16, k = 8, V = 128256, 2 positions: 27 us against 39 us streamed;
+        // B = 36, k = 6, V = 20224: 10.1 us against 11.3), in pairs of SMs: with clusters of 3 or 5 a batch
+        // that just fits was slower (B = 28, V = 8704, 5 CTAs: 13.9 us, 4: 9.8)
+        const int c = widest_cluster<verify_lazy_kernel<In, true, true>, kStagedThreads>(B, most, kStageMaxSmem, false) & ~1;
+        if (c >= 2) split_vocab(V, c, &fp);
+        for (int w = win; w >= 1 && c >= 2; w /= 2) {
+            const size_t smem = lazy_sub_offset(std::min(2 * w, 2 * k + 1), fp.span, es) + sub_bytes();
+            if (smem <= kStageMaxSmem && ctas_per_sm<verify_lazy_kernel<In, true, true>, kStagedThreads>(smem) >= 1) {
+                // so small a second round that its bytes cost nothing if the first one rejects
+                const int ahead = pos * std::min(2 * w, kLazyMaxWin) <= 9e6;
+                return from_cuda(launch_ex(true, verify_lazy_kernel<In, true, true>, dim3(unsigned(B) * unsigned(fp.csize)),
+                                        dim3(kStagedThreads), smem, stream, fp.csize, fp, w, ahead));
+            }
+            if (c == 2) break;  // long spans: streamed at four CTAs an SM instead
         }
     }
-    // fewer, longer spans while three CTAs an SM remain and a position's span stays within
-    // 68 KB, so that the rows in flight stay in L2 for the draw (B = 256: V = 32000 2 CTAs a
-    // sequence, 37.9 us against 41.1 and 45.9 us with 4 and 8; V = 128256 8 CTAs, 76 us against
-    // 85 and 102 us with 4 and 2)
-    int c = kSeqMaxCluster;
-    while (c > 1 && (V <= 2048 * c || ((long long)B * c / 2 >= 3LL * device_sms() && size_t(V / (c / 2)) * 2 * es <= 68 * 1024)))
-        c /= 2;
+    // one wave of the widest clusters, not quite full, since a grid that just fits waits for its last
+    // slots (B = 192, V = 11200 with 3 CTAs a sequence, of which 194 fit: 27.0 us, with 2 25.1; B = 84,
+    // V = 38180 fp32, 6 CTAs: 21.0 us, with 8, of which 74 fit, 31.9; B = 186, V = 24576, 3: 20.5, with
+    // 4 27.0), as long as L2 holds a position for the draw; past that the fewest CTAs whose
+    // spans stay within 68 KB, so that the rows in flight do (B = 256, V = 128256 8 CTAs, 76 us
+    // against 85 and 102 us with 4 and 2)
+    int c = most;
+    if (pos <= 100e6) {
+        // (batches past one wave: B = 340, 2 CTAs against 1: V = 32000 54 and 64 us, V = 8192 27 and 24)
+        const int c1 = size_t(V) * es >= 48 * 1024 ? 2 : 1;
+        constexpr size_t kSubs = 4096;  // more than any span within 100 MB takes
+        c = std::max(c1, aligned ? widest_cluster<verify_lazy_kernel<In, false, true>, kLazyThreads>(B, most, kSubs, true)
+                                : widest_cluster<verify_lazy_kernel<In, false, false>, kLazyThreads>(B, most, kSubs, true));
+    } else {
+        while (c > 1 && size_t(V / (c / 2)) * 2 * es <= 68 * 1024) c /= 2;
+    }
     split_vocab(V, c, &fp);
     if ((long long)B * fp.csize > INT_MAX) return OSD_ERR_UNSUPPORTED;
     const dim3 grid(unsigned(B) * unsigned(fp.csize));

@@ -94,6 +94,12 @@ ROUND_CASES = [  # (B, k, V, dtype, T, noise)
     (256, 3, 4104, torch.bfloat16, 1.3, 0.3),    # two CTAs a sequence
     (300, 2, 63, torch.bfloat16, 1.0, 0.3),      # one, and no whole warp step
     (9, 1, 32008, torch.bfloat16, 1.0, 0.3),
+    (51, 12, 10944, torch.bfloat16, 1.0, 0.1),   # 8 positions staged by clusters of 2, the rest streamed
+    (50, 20, 4101, torch.bfloat16, 1.0, 0.1),    # 16 rows a round on 8 warps: 8, 8 and 5 positions
+    (90, 10, 2048, torch.float32, 1.0, 0.1),     # the same on aligned rows
+    (36, 6, 20224, torch.bfloat16, 1.0, 0.3),    # staged by clusters of 4
+    (186, 2, 24576, torch.bfloat16, 1.0, 0.3),   # streamed by clusters of 3
+    (310, 1, 24600, torch.bfloat16, 1.0, 0.3),   # past one wave
 ]
 
 
