@@ -159,11 +159,19 @@ __device__ __forceinline__ void stage_shifted(In* zs, In* ts, const In* zrow, co
         for (int e = 0; e < kVec; ++e) v[e] = E::load(row + j + e);
         return pack_raw<In, kVec>(v);
     };
+    if constexpr (sizeof(In) == 4) {
+#pragma unroll 4
+        for (int r = tid; r < r0; r += kT) {
+            copy_raw(zs + r, zrow + m.jb + r);
+            copy_raw(ts + r, trow + m.jb + r);
+        }
+    } else {
 #pragma unroll 2
-    for (int v = tid; v < m.nv; v += kT) {
-        const uint4 z = chunk(zrow, m.jb + v * kVec), t = chunk(trow, m.jb + v * kVec);
-        *reinterpret_cast<uint4*>(zs + v * kVec) = z;
-        *reinterpret_cast<uint4*>(ts + v * kVec) = t;
+        for (int v = tid; v < m.nv; v += kT) {
+            const uint4 z = chunk(zrow, m.jb + v * kVec), t = chunk(trow, m.jb + v * kVec);
+            *reinterpret_cast<uint4*>(zs + v * kVec) = z;
+            *reinterpret_cast<uint4*>(ts + v * kVec) = t;
+        }
     }
     if (tid < m.rag) {
         const int j = span_entry<In>(m, r0 + tid);
