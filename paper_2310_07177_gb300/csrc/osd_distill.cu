@@ -1834,11 +1834,12 @@ static cudaError_t launch_distill_tm(const DistParams& dp, long long rows, cudaS
     const long long K = tl.clusters;
     TmShape sh = tl.shape;
     sh.run = rows >= 16 * K ? kTmRows : (rows >= 8 * K ? 4 : 2);
-    if (dp.mask) {
+    if (dp.mask && rows >= 4 * K) {
         // a mask leaves only part of each piece active: runs twice as long and tail
         // pieces of 6 and 3 rows instead of 2 and 1 carry about as much work at 40 %
         // (6554 of 16384 rows of 32128, JSD: 353 against 356 us; runs of 20 and pieces
-        // of 5 and 3: 352 us)
+        // of 5 and 3: 352 us); with few rows they would only queue behind each other (7 rows of
+        // 4797 fp32 RKL: 13.3 us in pieces of 3, 6.7 singly)
         sh.run *= 2;
         sh.piece2 = 6;
         sh.piece1 = 3;
