@@ -1635,7 +1635,7 @@ static cudaError_t launch_distill_kind(const DistParams& dp, long long rows, siz
         const cudaError_t e = allow_wide_clusters<distill_kernel<In, kKind, kAligned, kT>>();
         if (e != cudaSuccess) return e;
     }
-    if (smem > 48 * 1024) {
+    if (smem > 47 * 1024) {  // 48 KB without an opt-in, of which the kernel's static arrays take some
         // the opt-in is per device and kernel; set it once, so that later calls
         // (including ones under stream capture) make no attribute call
         static std::atomic<int> allowed[64];

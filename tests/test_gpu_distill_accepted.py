@@ -58,6 +58,7 @@ CASES = [  # (B, k, V, dtype)
     (9, 4, 33001, torch.bfloat16),
     (64, 8, 4097, torch.float32),
     (5, 2, 128256, torch.bfloat16),
+    (1, 3, 48936, torch.float32),   # 48 KB of dynamic shared memory to the byte
 ]
 
 
