@@ -308,9 +308,10 @@ __device__ __forceinline__ double warp_incl_scan_f64(double v) {
 }
 
 // ---------------------------------------------------------------- programmatic dependent launch
-// Every kernel here is launched with programmatic stream serialisation: it may start
-// while the kernel before it on the stream ends, and calls grid_dependency_sync before
-// its first access of global memory.  That waits for the kernels before it to be
+// Kernels here are launched with programmatic stream serialisation (distillation and mixed
+// sampling only where a call leaves SMs free): they may start while the kernel before
+// them on the stream ends, and call grid_dependency_sync before their first access of global
+// memory.  That waits for the kernels before it to be
 // complete and visible, then lets the next one start as this one ends.  What comes
 // before it (scheduling, barrier and tensor-memory set-up) overlaps the previous
 // kernel: back to back, a distill call on 16 x 32000 takes 5.0 us instead of 8.2, greedy

@@ -225,6 +225,11 @@ __device__ __forceinline__ void tvd_gradient(const In* zs, const In* ts, int n, 
     }
 }
 
+// (CE's wide CTAs always start after the previous kernel's end: with the wait in it they took 47
+// registers instead of 40 and 12606 x 101056 CE 1869 us instead of 1801)
+template <int kKind, int kT>
+constexpr bool kEarlyStart = !(kKind == OSD_CE && kT == kDistThreadsWide);
+
 template <typename In, int kKind, bool kAligned, int kT>
 __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
     // JSD clamps both rows to -1e30: a zero probability then stays exactly 0 and
@@ -258,7 +263,7 @@ __global__ void __launch_bounds__(kT) distill_kernel(DistParams p) {
     const int csize = p.csize;
     const float c = p.c, inv_tau = p.inv_tau;
     const int rank = (csize > 1) ? static_cast<int>(cluster_rank()) : 0;
-    grid_dependency_sync();
+    if constexpr (kEarlyStart<kKind, kT>) grid_dependency_sync();
     long long row = blockIdx.x / csize;  // the launch row; from here on, the output row
     long long g, pp;
     const int V = p.V;
@@ -1628,6 +1633,12 @@ static cudaError_t allow_wide_clusters() {
     return cudaSuccess;
 }
 
+// Whether a grid starts before the previous kernel's end (grid_dependency_sync), which gains 2
+// to 3 us a call of few rows (16 x 32000: 8.2 -> 5.0 us).  Where a call fills the SMs, the next
+// one's CTAs then pile up on those that become free first: 146 sequences of 3 x 29952
+// accepted JSD 15.6 us against 13.2 without.
+static bool start_early(long long ctas) { return ctas <= 2LL * device_sms(); }
+
 template <typename In, int kKind, bool kAligned, int kT>
 static cudaError_t launch_distill_kind(const DistParams& dp, long long rows, size_t smem, cudaStream_t s) {
     auto kern = distill_kernel<In, kKind, kAligned, kT>;
@@ -1653,7 +1664,8 @@ static cudaError_t launch_distill_kind(const DistParams& dp, long long rows, siz
             }
         }
     }
-    return launch_ex(true, kern, dim3(static_cast<unsigned>(rows * dp.csize)), dim3(kT), smem, s, dp.csize, dp);
+    return launch_ex(kEarlyStart<kKind, kT> && start_early(rows * dp.csize), kern, dim3(static_cast<unsigned>(rows * dp.csize)), dim3(kT), smem, s,
+                     dp.csize, dp);
 }
 
 // (TVD, whose extra cluster exchange costs more with wide CTAs, always takes kDistThreads.)
@@ -1852,10 +1864,9 @@ static cudaError_t launch_distill_tm(const DistParams& dp, long long rows, cudaS
     sh.n2 = static_cast<int>((twos + sh.piece2 - 1) / sh.piece2);
     const long long n1 = (ones + sh.piece1 - 1) / sh.piece1;
     const long long runs = sh.n8 + sh.n2 + n1;
-    // A start before the previous kernel's end (grid_dependency_sync) gains 2 to 7 us a call,
-    // but costs a long flush 0.9 % (65536 x 32000 RKL, one after another: 2517 against 2496 us;
-    // 16384 x 32128 masked 0.2 %; 2048 x 128256, 43 K rows, gains 1.8 %)
-    sh.early = rows < 64 * K;
+    // (582 x 47424 RKL 48.8 us with an early start against 47.1, 65536 x 32000 2517 against 2496;
+    // 16-CTA clusters over many waves, 2048 x 128256, gain 1.8 %)
+    sh.early = start_early(runs * dp.csize) || (dp.csize > 8 && rows >= 8 * K && rows < 64 * K);
     return launch_ex(sh.early != 0, distill_tm_kernel<In, kKind, kAnyPhase>, dim3(static_cast<unsigned>(runs * dp.csize)),
                   dim3(kTmThreads), tl.smem, s, dp.csize, dp, sh);
 }

@@ -359,10 +359,13 @@ extern "C" osd_status osd_mixed_sample(const void* draft_logits, const void* tar
         constexpr int kMode = decltype(mode)::value;
         const dim3 grid(static_cast<unsigned>(N));
         const int steps = V / (32 * Elem<In>::kVec);
-        const int ww = steps > 256 && N <= (steps > 400 ? 16 : 4) * sms ? 32 : (steps > 24 && N <= 4 * sms ? 16 : 4);
-        if (ww == 32) return launch_ex(true, mixed_sample_kernel<In, kMode, 32>, grid, dim3(1024), 0, s, 1, mp);
-        if (ww == 16) return launch_ex(true, mixed_sample_kernel<In, kMode, 16>, grid, dim3(512), 0, s, 1, mp);
-        return launch_ex(true, mixed_sample_kernel<In, kMode, 4>, grid, dim3(128), 0, s, 1, mp);
+        const int ww = steps > 256 && N <= (steps > 400 ? 16 : 4) * sms ? 32 : (steps > 24 && N <= (steps > 64 ? 4 : 2) * sms ? 16 : 4);
+        // a start before the previous kernel's end packs a call that fills the SMs onto those that
+        // become free first (1761 x 16256: 36.7 us against 34.0 without; 50 x 32000: 10.1 against 12.3)
+        const bool early = N <= sms;
+        if (ww == 32) return launch_ex(early, mixed_sample_kernel<In, kMode, 32>, grid, dim3(1024), 0, s, 1, mp);
+        if (ww == 16) return launch_ex(early, mixed_sample_kernel<In, kMode, 16>, grid, dim3(512), 0, s, 1, mp);
+        return launch_ex(early, mixed_sample_kernel<In, kMode, 4>, grid, dim3(128), 0, s, 1, mp);
     };
     auto go = [&](auto tag) {
         if (vec) return go_warps(tag, std::integral_constant<int, kMixAligned>());
