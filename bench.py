@@ -208,6 +208,12 @@ def _bytes_verify(B, k, V, s_in, greedy):
     return (B * (k + 1) * V * s_in) if greedy else ((B * k + B * (k + 1)) * V * s_in)
 
 
+def _bytes_verify_needed(accepted, k, V, s_in):
+    """What a sampled pass cannot do without: the tests run in order, so both rows of every
+    position up to the first rejection, and the bonus row where all k pass."""
+    return sum(2 * (a + 1) if a < k else 2 * k + 1 for a in accepted if a >= 0) * V * s_in
+
+
 # ----------------------------------------------------------------------------- our arm
 def run_ours(args):
     import torch
@@ -314,14 +320,14 @@ def run_ours(args):
     if wl == "serving-32k":
         ver_pos = 2 * sv.B * sv.k
         positions = ver_pos + dist_pos + n_rej
-        launches = 2 * 2 + 1 + len(kinds)
-        bytes_v = _bytes_verify(sv.B, sv.k, sv.V, s_in, False)
+        launches = 1 + 2 + 1 + len(kinds)  # sampled and greedy verify, the rejected rows, the flushes
+        bytes_v = _bytes_verify_needed(vout.accepted.tolist(), sv.k, sv.V, s_in)
         bytes_g = _bytes_verify(sv.B, sv.k, sv.V, s_in, True)
     else:
         ver_pos = sv.B * sv.k
         positions = ver_pos + n_rej
-        launches = 2 + 1
-        bytes_v = _bytes_verify(sv.B, sv.k, sv.V, s_in, False)
+        launches = 1 + 1
+        bytes_v = _bytes_verify_needed(vout.accepted.tolist(), sv.k, sv.V, s_in)
     value = job_throughput(positions, world, ms_step)
     peak, peak_src = _peak_hbm()
     avg_ver = statistics.mean(verify_ms)
@@ -351,7 +357,7 @@ def run_ours(args):
         kernels["distill_jsd_masked"] = _time_jsd_flush(osd, dev, l2_flush, stream, reps=max(5, args.steps))
     for kv in kernels.values():
         kv["frac_of_peak"] = kv["gbs"] / peak
-    # the dominant kernel: distill on the default step, verify's row statistics at 128k
+    # the dominant kernel: distill on the default step, verify at 128k
     top = "distill" if wl == "serving-32k" else "verify"
     achieved = kernels[top]["gbs"]
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
@@ -361,7 +367,7 @@ def run_ours(args):
                             if top == "distill" else _traffic("verify", VERIFY_SOURCES)),
                 "kernel": (" + ".join(("distill_tm_kernel " if k in ("rkl", "tvd", "jsd") else "distill_kernel ")
                                       + k.upper() for k in kinds) if top == "distill"
-                           else "row_stats_kernel + verify_finalize_kernel"),
+                           else "verify_lazy_kernel"),
                 "peak_source": peak_src}
 
     e2e = None
@@ -453,7 +459,7 @@ def _time_large_vocab(osd, dev, l2_flush, stream, reps):
                                         workspace=ws, out=out), l2_flush, stream, reps)
     t_d = _timed(lambda: osd.osd_distill_accepted(v["draft"], v["target"], out.accepted, "fkl", 0.5, out=rej),
                  l2_flush, stream, reps)
-    bv = _bytes_verify(sv.B, sv.k, sv.V, 2, False)
+    bv = _bytes_verify_needed(out.accepted.tolist(), sv.k, sv.V, 2)
     bd = n_rej * sv.V * (2 * 2 + 4) + sv.B * 4
     res = {
         "verify_large_vocab": {"us_per_call": t_v * 1e3, "alg_bytes": bv, "gbs": bv / (t_v / 1e3) / 1e9,
@@ -511,8 +517,8 @@ def _time_tree_verify(osd, dev, l2_flush, stream, reps):
         if i >= 2:
             ms.append(a.elapsed_time(b))
     avg = statistics.mean(ms)
-    alg = 2 * B * n * V * 2  # every node's draft and target row, read once by the statistics pass
     acc = res.accepted.float().mean().item()
+    alg = int(B * (acc + 1)) * 2 * V * 2  # the draft and target rows of the nodes on the walks
     return {"us_per_call": avg * 1e3, "alg_bytes": alg, "gbs": alg / (avg / 1e3) / 1e9,
             "positions_per_s": B * (acc + 1) / (avg / 1e3), "mean_accepted": round(acc, 3),
             "nodes": n, "in_step": False}

@@ -239,11 +239,6 @@ struct MaxSum {
     float m;
     float s;
 };
-__device__ __forceinline__ MaxSum merge_ms(MaxSum a, MaxSum b, float c_hi, float c_lo) {
-    if (b.m > a.m) { MaxSum t = a; a = b; b = t; }
-    if (b.m != kNegInf) a.s += b.s * ex2(mul_c(b.m - a.m, c_hi, c_lo));
-    return a;
-}
 // Argmax with the lowest index on ties.
 struct MaxIdx {
     float m;
@@ -366,11 +361,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
     return ok != 0;
 }
-// Arrive on a barrier of this CTA (release at CTA scope: this thread's earlier
-// shared-memory writes are visible to the threads that then see the phase end).
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_addr(bar)) : "memory");
-}
 // The phase test with acquire at cluster scope: for barriers completed by
 // st.async writes from other CTAs of the cluster.
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
@@ -448,22 +438,6 @@ __device__ __forceinline__ uint32_t map_rank(const void* p, uint32_t rank) {
 __device__ __forceinline__ float ld_dsmem_f32(uint32_t addr) {
     float v;
     asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ unsigned long long ld_dsmem_u64(uint32_t addr) {
-    unsigned long long v;
-    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ float4 ld_dsmem_v4f32(uint32_t addr) {  // 16-byte aligned
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ float2 ld_dsmem_v2f32(uint32_t addr) {  // 8-byte aligned
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
     return v;
 }
 __device__ __forceinline__ int ld_dsmem_s32(uint32_t addr) {
