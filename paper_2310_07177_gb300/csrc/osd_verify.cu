@@ -637,7 +637,11 @@ verify_lazy_kernel(FinParams p, int win, int ahead) {
             }
         }
     }
-    // the draft tokens, the two logits each accept test needs, and the uniforms
+    __syncthreads();  // the barriers are initialised before anyone waits on them
+    // ... and before any peer pushes to them: arrive now, wait before the first push
+    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    // the draft tokens, the two logits each accept test needs, and the uniforms: two dependent
+    // loads of one warp, which the others do not wait for before they start on the rows
     int bad = 0;
     if (warp == kWarps - 1) {
         const int32_t* y = p.tokens + size_t(b) * k;
@@ -654,9 +658,6 @@ verify_lazy_kernel(FinParams p, int win, int ahead) {
     }
     if (warp == kWarps - 2)
         for (int i = lane; i <= k; i += 32) sh.u[i] = p.uniforms[size_t(b) * (k + 1) + i];
-    __syncthreads();  // the barriers are initialised before anyone waits on them
-    // ... and before any peer pushes to them: arrive now, wait before the first push
-    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 
     int a = -1, i0 = 0, w = w0;
     unsigned round = 0;
@@ -784,6 +785,9 @@ __global__ void __launch_bounds__(kFuseThreads) verify_fused_kernel(FinParams p)
                      ((q <= k) ? target + size_t(q) * V : draft + size_t(q - k - 1) * V) + e0, bytes, &rbar[q]);
         }
     }
+    __syncthreads();  // the barriers are initialised before anyone waits on them
+    // ... and before any peer pushes to them: arrive now, wait before the first push
+    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     // meanwhile the draft tokens, the two logits each accept test needs, and the uniforms
     int bad = 0;
     if (warp == kWarps - 1) {
@@ -801,9 +805,6 @@ __global__ void __launch_bounds__(kFuseThreads) verify_fused_kernel(FinParams p)
     }
     if (warp == kWarps - 2)
         for (int i = lane; i <= k; i += 32) sh.u[i] = p.uniforms[size_t(b) * (k + 1) + i];
-    __syncthreads();  // the barriers are initialised before anyone waits on them
-    // ... and before any peer pushes to them: arrive now, wait before the first push
-    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 
     // span statistics of every row: warp items (row, part)
     const int nch = n / kVec;
