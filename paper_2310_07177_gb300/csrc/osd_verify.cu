@@ -728,9 +728,11 @@ verify_lazy_kernel(FinParams p, int win, int ahead) {
 // turn out not to be needed: each CTA of the sequence's cluster bulk-copies its
 // vocabulary span of all 2k + 1 rows (all the copies in flight at once, a barrier
 // per row, so that a row's statistics start as soon as it has landed), and one
-// exchange decides all the positions.  It runs only when its grid fits in one wave.
-// At B = 32, k = 5, V = 32000 it measured 23.9 us in the bench step with 512 threads
-// (256 threads 26.7 us; 16-CTA clusters 38 us).
+// exchange decides all the positions.  It runs only when its grid fits in one wave with
+// slots to spare (see launch_sampling).  At B = 32, k = 5, V = 32000 (22 MB, 3.3 us at the copy
+// bandwidth) it takes 12.0 us back to back, 19.7 us alone with a cold L2: a chain of copy,
+// statistics, exchange, tests and draw, barrier stalls first (6.7 warps an issue).  512
+// threads (256 threads 12 % more; 16-CTA clusters 60 % more).
 constexpr int kFuseThreads = 512;
 constexpr int kFuseParts = 4;           // warp items per row for the span statistics
 constexpr int kFuseMaxB = 64;           // at most this many sequences, and the grid in one wave
