@@ -195,18 +195,21 @@ __device__ __forceinline__ MaxSum span_stats(const In* p, int n, int part, int p
     return MaxSum{wm, s};
 }
 
-// One row's statistics from `count` <= 8 partials at x[0], x[stride], ..., merged in
+// One row's statistics from `count` <= kMost partials at x[0], x[stride], ..., merged in
 // that order: the maximum first, then the sums brought to it (all loads in flight together).
+// The caller's bound on its partials is kMost: one that is too low drops part of the row.  (A
+// loop over groups of 8 for any count cost the streaming verifier 3 to 6 %, by its spills.)
+template <int kMost>
 __device__ __forceinline__ MaxSum merge_slots(const MaxSum* x, int stride, int count, float ch, float cl) {
-    MaxSum o[kSeqMaxCluster];
+    MaxSum o[kMost];
     float m = kNegInf, s = 0.f;
 #pragma unroll
-    for (int i = 0; i < kSeqMaxCluster; ++i) {
+    for (int i = 0; i < kMost; ++i) {
         o[i] = (i < count) ? x[i * stride] : MaxSum{kNegInf, 0.f};
         m = fmaxf(m, o[i].m);
     }
 #pragma unroll
-    for (int i = 0; i < kSeqMaxCluster; ++i)
+    for (int i = 0; i < kMost; ++i)
         if (o[i].m != kNegInf) s += o[i].s * ex2(mul_c(o[i].m - m, ch, cl));
     return MaxSum{m, s};
 }

@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p, i
                 MaxSum* recv = s_recv[buf];
                 bool gone = false;
                 if (lane < nr) {
-                    const MaxSum acc = merge_slots(s_part + lane * parts, 1, parts, ch, cl);
+                    const MaxSum acc = merge_slots<kTreeWarps>(s_part + lane * parts, 1, parts, ch, cl);
                     if (csize > 1) {
                         for (int d = 0; d < csize; ++d)
                             st_async_v2(map_rank(&recv[rank * kTreeMaxRows + lane], static_cast<uint32_t>(d)),
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p, i
                 }
                 __syncwarp();
                 if (!gone && lane < nr) {
-                    const MaxSum o = merge_slots(recv + lane, kTreeMaxRows, csize, ch, cl);
+                    const MaxSum o = merge_slots<kSeqMaxCluster>(recv + lane, kTreeMaxRows, csize, ch, cl);
                     s_m[lane] = o.m;
                     s_s[lane] = o.s;
                 }

@@ -206,18 +206,19 @@ __device__ __forceinline__ int seq_test(const FinParams& p, int b, const SeqSmem
     return i0 + w == k + 1 ? k : -1;
 }
 
-// Warp 0, after a round's span statistics (nr rows, `parts` partials each): merge
+// Warp 0, after a round's span statistics (nr rows, `parts` <= kMostParts partials each): merge
 // them, push the span's to every CTA of the cluster (slot [rank][row] of recv,
 // completing on bar), merge the cluster's and run the tests.  Every CTA merges the
 // same slots in the same order, so all decide alike.  Returns seq_test's answer,
 // or -2 when a CTA's copies (`stuck`, sent as a negative sum) or the wait gave up.
+template <int kMostParts>
 __device__ __forceinline__ int seq_round(const FinParams& p, int b, SeqSmem& sh, const MaxSum* part, int parts,
                                          MaxSum* recv, int stride, uint64_t* bar, uint32_t parity, int rank, int i0,
                                          int w, int nr, bool stuck) {
     const int lane = threadIdx.x & 31, csize = p.csize, k = p.k;
     const float ch = p.c_hi, cl = p.c_lo;
     for (int r = lane; r < nr; r += 32) {
-        MaxSum acc = merge_slots(part + r * parts, 1, parts, ch, cl);
+        MaxSum acc = merge_slots<kMostParts>(part + r * parts, 1, parts, ch, cl);
         if (stuck) acc.s = -1.f;
         if (csize > 1) {
             for (int d = 0; d < csize; ++d)
@@ -236,7 +237,7 @@ __device__ __forceinline__ int seq_round(const FinParams& p, int b, SeqSmem& sh,
     if (!gone) {
         for (int r = lane; r < nr; r += 32) {
             for (int c = 0; c < csize; ++c) gone |= recv[c * stride + r].s < 0.f;
-            const MaxSum o = merge_slots(recv + r, stride, csize, ch, cl);
+            const MaxSum o = merge_slots<kSeqMaxCluster>(recv + r, stride, csize, ch, cl);
             const int at = (r < w) ? i0 + r : k + 1 + i0 + r - w;
             sh.m[at] = o.m;
             sh.s[at] = o.s;
@@ -664,7 +665,7 @@ verify_lazy_kernel(FinParams p, int win, int ahead) {
     bool stuck = false;  // a staging copy gave up in this CTA
     for (;;) {
         const int nr = rows_of(i0, w);
-        const int parts = max(1, kWarps / nr);  // warps per row
+        const int parts = max(1, kWarps / nr);  // warps per row: all kWarps on a lone bonus row
         int timed_out = 0;
         for (int it = warp; it < nr * parts; it += kWarps) {
             const int q = it / parts, part = it - q * parts;
@@ -693,8 +694,8 @@ verify_lazy_kernel(FinParams p, int win, int ahead) {
             __syncthreads();
         }
         if (warp == 0) {
-            const int dec = seq_round(p, b, sh, s_part, parts, s_recv[round & 1u], kLazyMaxRows, &s_bar[round & 1u],
-                                      (round >> 1) & 1u, rank, i0, w, nr, stuck);
+            const int dec = seq_round<kWarps>(p, b, sh, s_part, parts, s_recv[round & 1u], kLazyMaxRows, &s_bar[round & 1u],
+                                              (round >> 1) & 1u, rank, i0, w, nr, stuck);
             if (lane == 0) s_dec = dec;
         }
         __syncthreads();
@@ -830,7 +831,8 @@ __global__ void __launch_bounds__(kFuseThreads) verify_fused_kernel(FinParams p)
     }
     if (csize > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (warp == 0) {
-        const int dec = seq_round(p, b, sh, s_part, kFuseParts, recv, nrows, &s_bar, 0, rank, 0, k + 1, nrows, stuck);
+        const int dec =
+            seq_round<kFuseParts>(p, b, sh, s_part, kFuseParts, recv, nrows, &s_bar, 0, rank, 0, k + 1, nrows, stuck);
         if (lane == 0) s_dec = dec;
     }
     __syncthreads();

@@ -117,6 +117,41 @@ def test_rounds_match_oracle(osd, B, k, V, dtype, T, noise):
     np.testing.assert_array_equal(res.accepted.cpu().numpy() < 0, bad)
 
 
+# A last round of the bonus row alone, every warp of a staged kernel's CTA on it: the row's
+# peak (or its only finite entries) at each 16-byte-vector group of a warp in turn, so
+# that a partial left out of the merge shows in the token or in the CDF.
+LONE_BONUS_CASES = [(1, 6, 128256), (32, 3, 128256), (36, 4, 32000), (50, 4, 24000), (48, 4, 16384), (16, 6, 128256)]
+
+
+@pytest.mark.parametrize("rest", ["normal", "-inf"])
+@pytest.mark.parametrize("B,k,V", LONE_BONUS_CASES)
+def test_peak_of_a_lone_bonus_row(osd, B, k, V, rest):
+    g = torch.Generator().manual_seed(V + k)
+    n = max(B, 34)  # peaks: 33 groups of 32 vectors of 8 entries, then the row's last entry
+    n_calls = (n + B - 1) // B
+    z = (torch.randn(B, k, V, generator=g) * 2.5).to(torch.bfloat16)
+    for call in range(n_calls):
+        bonus = torch.randn(B, V, generator=g) * 2.5 if rest == "normal" else torch.full((B, V), float("-inf"))
+        for b in range(B):
+            i = (call * B + b) % 34
+            at = V - 1 if i == 33 else (i * 256 + 5 * i % 256) % V
+            if rest == "normal":
+                bonus[b, at] = 20.0
+            else:  # two entries of one vector share the mass
+                bonus[b, at] = 1.0
+                bonus[b, at ^ 1] = 0.0
+        t = torch.cat([z, bonus.to(torch.bfloat16)[:, None]], dim=1).contiguous()
+        y = torch.randint(0, V, (B, k), generator=g, dtype=torch.int32)
+        u = torch.rand(B, k + 1, generator=g)
+        inp = {"draft": z, "target": t, "tokens": y, "uniforms": u}
+        res, ref = _run(osd, inp, 1.0)
+        assert (res.accepted.cpu() == k).all()  # equal rows accept every draft token
+        check_verify(res, ref, k, V)
+        # the edges of the CDF are as exact as the accept ratios (check_margins)
+        gap, gap_ref = res.diag_cdf_gap.cpu().numpy(), ref["cdf_gap"]
+        assert np.abs(gap - gap_ref).max() <= 2e-6, np.abs(gap - gap_ref).max()
+
+
 GREEDY_CASES = [
     (16, 3, 1, torch.float32), (32, 4, 1001, torch.bfloat16), (9, 2, 40000, torch.float32),
     (12, 5, 32000, torch.bfloat16), (38, 7, 32768, torch.bfloat16), (7, 3, 4096, torch.bfloat16),
