@@ -305,10 +305,14 @@ __device__ __forceinline__ double warp_incl_scan_f64(double v) {
 // ---------------------------------------------------------------- programmatic dependent launch
 // Kernels here are launched with programmatic stream serialisation (distillation and mixed
 // sampling only where a call leaves SMs free): they may start while the kernel before
-// them on the stream ends, and call grid_dependency_sync before their first access of global
-// memory.  That waits for the kernels before it to be
-// complete and visible, then lets the next one start as this one ends.  What comes
-// before it (scheduling, barrier and tensor-memory set-up) overlaps the previous
+// them on the stream ends.  Every CTA of a kernel calls grid_dependency_sync, whatever it
+// does afterwards: it waits for the kernel before to be complete and visible, and a grid
+// whose CTAs all left without it could end before that one, which the kernel after, waiting
+// for this grid alone, would then overtake.  It comes before the first access of global
+// memory, but for the greedy walks' second kernels, which read their tokens (and fill
+// outputs that the first one does not touch) ahead of it: the first kernel lets them start only
+// once it has waited itself.  After the wait the next kernel may start as this one ends.  What
+// comes before it (scheduling, barrier and tensor-memory set-up) overlaps the previous
 // kernel: back to back, a distill call on 16 x 32000 takes 5.0 us instead of 8.2, greedy
 // verification of 32 x 5 x 32000 6.0 instead of 8.2, verification of 4 x 4 x 32000 9.7 instead of 12.3.
 // Both instructions are no-ops without the attribute.

@@ -85,8 +85,11 @@ __global__ void __launch_bounds__(kGreedyThreads) tree_greedy_kernel(TreeParams 
             p.last_node[b] = -1;
         }
     }
+    // the row statistics are complete from here on.  A bad sequence waits for them too: the grid
+    // must not end before row_argmax_kernel has, since the next call on the stream waits for this
+    // grid alone before it writes the workspace again (or the logits, which that kernel reads).
+    grid_dependency_sync();
     if (bad) return;
-    grid_dependency_sync();  // the row statistics are complete from here on
     for (int nd = tid; nd < n; nd += kGreedyThreads) {
         const RowStat* st = p.stats + (size_t(b) * n + nd) * p.n_slices;
         MaxIdx acc{kNegInf, INT_MAX};

@@ -177,6 +177,28 @@ def test_bad_tokens(osd):
     assert torch.all(res.last_node[1:] == -1)
 
 
+def test_greedy_call_after_one_with_only_bad_tokens(osd):
+    """A greedy call whose only sequence has a bad token ends with its statistics pass all the
+    same: the next call may write the workspace and the logits that pass uses."""
+    n, V = 16, 1 << 19
+    inp = W.tree_inputs(1, [-1] + list(range(n - 1)), V, torch.float32, 0.0, seed=3)
+    dev = torch.device("cuda")
+    t, y, par = inp["target"].to(dev), inp["tokens"].to(dev), inp["parent"]
+    bad = y.clone()
+    bad[0, 1] = V
+    other = t.flip(-1).contiguous()
+    ws = torch.empty(osd.osd_verify_tree_workspace_size(1, n, V), dtype=torch.uint8, device=dev)
+    want = osd.osd_verify_tree(None, other, par, y, None, 0.0)
+    torch.cuda.synchronize()
+    for _ in range(20):
+        r = osd.osd_verify_tree(None, t, par, bad, None, 0.0, workspace=ws)
+        got = osd.osd_verify_tree(None, other, par, y, None, 0.0, workspace=ws)
+        torch.cuda.synchronize()
+        assert r.accepted.item() == -1 and r.last_node.item() == -1 and (r.out_tokens == -1).all()
+        for f in ("accepted", "path", "out_tokens", "last_node"):
+            assert torch.equal(getattr(got, f), getattr(want, f)), f
+
+
 def test_invalid_arguments_are_rejected(osd):
     dev = torch.device("cuda")
     t = torch.zeros(2, 3, 16, device=dev)
