@@ -934,6 +934,18 @@ __device__ __forceinline__ float log2_sum(float x) {
     const uint32_t b = __float_as_uint(x);
     return static_cast<float>(static_cast<int>(b >> 23) - 127) + lg2(__uint_as_float((b & 0x007fffffu) | 0x3f800000u));
 }
+// fe - log2 x of such a sum, and in `del` by how much rounding it raises the powers of 2
+// that have it in their exponent: 2^result = 2^(fe - log2 x) (1 + del).
+__device__ __forceinline__ float minus_log2(float x, float fe, float* del) {
+    *del = 0.f;
+    if (!(x >= 1.f && x <= 3.0e38f)) return fe - lg2(x);
+    const uint32_t b = __float_as_uint(x);
+    const float e = static_cast<float>(static_cast<int>(b >> 23) - 127);
+    const float l = log2f(__uint_as_float((b & 0x007fffffu) | 0x3f800000u));
+    const float L = e + l, r = fe - L;
+    *del = kLn2 * ((l - (L - e)) - (fe - (r + L)));  // the two roundings' errors, exact
+    return r;
+}
 constexpr uint64_t kTmPartWaitNs = 3000000000ull;  // partials: peers may first wait out their copies
 // Named barriers 1 and 2 of the CTA (0 is __syncthreads): `arrive` marks the
 // warp's arrival without waiting (release), `sync` waits for all kTmThreads (acquire).
@@ -974,9 +986,16 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
     __shared__ float4 s_slot[kW];  // the warps' values of the exchange in progress
     __shared__ float4 s_res;       // its merged result ...
     __shared__ int s_rerr;         // ... and whether a wait for it gave up
-    // TVD off the 16-byte grid: sign(q - p) = sign((z - gz) - (t - gt) - s_kap)
-    constexpr bool kSign = kTvd && kAnyPhase;
+    // TVD off the 16-byte grid: sign(q - p) = sign((z - gz) - (t - gt) - s_kap), the gradient
+    // from Q+ and Q- (sums of q where q >= p and elsewhere) as tvd_gradient has it, and what
+    // all q and all p of a row are off by in common (the rounding of cv and cu, which the
+    // first chunks' references make large on peaked rows) taken out of both results.  Errors
+    // of 1.5e-7 to 2e-7 of the gradient's norm, 3e-8 to 2.3e-7 in the loss, for 2 % of the time (4096 x
+    // 32001 bf16 201 us).  The aligned runs form the gradient from sums over all entries,
+    // which leaves it 2^-24 of the largest q, in absolute terms.
+    constexpr bool kApart = kTvd && kAnyPhase;
     [[maybe_unused]] __shared__ float s_kap;
+    [[maybe_unused]] __shared__ float2 s_del;  // kApart: what rounding cv and cu multiplies every q and p by, less 1
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int csize = p.csize;
@@ -1317,9 +1336,17 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                 },
                 [&](float4 m, bool& bad) {  // -> (gz, gt, cu, cv)
                     bad = m.y < 0.f;
-                    // taken from the logits, the sign is as exact as the sums; from q - p it also has
-                    // the rounding of both log2 E, whose magnitude is 10 and more
-                    if (kSign && lane == 0) s_kap = (logf(m.y / m.w) - kLn2 * (fold_err(m.x) - fold_err(m.z))) / inv_tau;
+                    if constexpr (kApart) {
+                        float dq, dp;
+                        const float cq = minus_log2(m.y, fold_err(m.x), &dq), cp = minus_log2(m.w, fold_err(m.z), &dp);
+                        if (lane == 0) {
+                            s_del = make_float2(dq, dp);
+                            // taken from the logits, the sign is as exact as the sums; from q - p it also
+                            // has the rounding of both log2 E, whose magnitude is 10 and more
+                            s_kap = (kLn2 * (cp - cq) - (dp - dq)) / inv_tau;
+                        }
+                        return make_float4(m.x, m.z, cp, cq);
+                    }
                     return make_float4(m.x, m.z, -log2_sum(m.w) + fold_err(m.z), -log2_sum(m.y) + fold_err(m.x));
                 }, failed);
             row_err = failed;
@@ -1336,11 +1363,12 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                 continue;
             }
             {
-                if constexpr (kSign) __syncwarp();  // (warp 0 wrote s_kap itself)
-                [[maybe_unused]] const float2 kap2 = f2(kSign ? s_kap : 0.f);
+                if constexpr (kApart) __syncwarp();  // (warp 0 wrote s_kap itself)
+                [[maybe_unused]] const float2 kap2 = f2(kApart ? s_kap : 0.f);
                 // ---- pass 2: divergence terms with the global normalisers.  TVD: A = sum
                 // |q - p|, S = sum q' with q' = q sign(q - p) (kept in tensor memory in
-                // place of the chunk's logits) and Q = sum q; JSD: KL(p||m) and KL(q||m) in bits
+                // place of the chunk's logits) and Q = sum q, or 2 Q+ and 2 Q- (kApart);
+                // JSD: KL(p||m) and KL(q||m) in bits
                 float2 A2 = f2(0.f), B2 = f2(0.f), C2 = f2(0.f);
                 if (!jsd_trivial) {
                     sweep_tm<In, false, false, false, false, kTvd, kJsd ? kTmJsdG : kTmG>(tw, tsh, nv, tail, rj, tz, tt,
@@ -1373,14 +1401,21 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                                     B2 = fma2(qw, sub2(v, lm), B2);
                                 } else {
                                     const float2 df = sub2(qj, pj);
-                                    const float2 sd = kSign ? sub2(sub2(zd, td), kap2) : df;
+                                    const float2 sd = kApart ? sub2(sub2(zd, td), kap2) : df;
                                     const float2 qq = make_float2(copysignf(qj.x, sd.x), copysignf(qj.y, sd.y));
                                     qs[e] = qq.x;
                                     if (two) qs[e + 1] = qq.y;
                                     A2.x += fabsf(df.x);
                                     if (two) A2.y += fabsf(df.y);
-                                    B2 = add2(B2, two ? qq : make_float2(qq.x, 0.f));
-                                    C2 = add2(C2, two ? qj : make_float2(qj.x, 0.f));
+                                    const float2 qs2 = two ? qq : make_float2(qq.x, 0.f);
+                                    const float2 qz = two ? qj : make_float2(qj.x, 0.f);
+                                    if constexpr (kApart) {  // q + q' is 2 q where q >= p, else 0
+                                        C2 = add2(C2, sub2(qz, qs2));
+                                        B2 = add2(B2, add2(qz, qs2));
+                                    } else {
+                                        B2 = add2(B2, qs2);
+                                        C2 = add2(C2, qz);
+                                    }
                                 }
                             }
                             if constexpr (kTvd) {
@@ -1392,7 +1427,8 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                 // ---- exchange 2: the sums of pass 2
                 const float4 v2 = make_float4(warp_sum(A2.x + A2.y), warp_sum(B2.x + B2.y),
                                               kJsd ? 0.f : warp_sum(C2.x + C2.y), 0.f);
-                // -> TVD (loss, k1, k2) with the gradient k1 q' + k2 |q'| below; JSD (loss, S)
+                // -> TVD (loss, k1, k2) with the gradient k1 q' + k2 |q'| below, or (loss, Q- / tau,
+                // Q+ / tau) (kApart); JSD (loss, S)
                 const float4 r2v = exchange(v2, make_float4(0.f, 0.f, 0.f, 0.f), &pbar2, recv2,
                     [&](float4 x) {
                         return make_float4(warp_sum(x.x), warp_sum(x.y), kJsd ? 0.f : warp_sum(x.z), 0.f);
@@ -1400,7 +1436,14 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                     [&](float4 m, bool&) {
                         if constexpr (kJsd)
                             return make_float4(jsd_trivial ? 0.f : kLn2 * (beta * m.x + (1.f - beta) * m.y), m.y, 0.f, 0.f);
-                        else
+                        else if constexpr (kApart) {
+                            // the common factors taken out: of the loss to first order, by what they are known
+                            // to be, with Q+ - Q- and P+ - P-; of the gradient by Q, which is 1
+                            __syncwarp();  // (warp 0 wrote s_del itself)
+                            const float Q = 0.5f * (m.y + m.z), dq = 0.5f * (m.y - m.z), dp = dq - m.x;
+                            const float k = inv_tau * (1.5f - Q);  // (1 / (2 Q^2) near Q = 1)
+                            return make_float4(0.5f * (m.x - s_del.x * dq + s_del.y * dp), m.z * k, m.y * k, 0.f);
+                        } else
                             return make_float4(0.5f * m.x, 0.5f * m.z * inv_tau, -0.5f * m.y * inv_tau, 0.f);
                     }, failed);
                 row_err = failed;
@@ -1521,8 +1564,16 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
         if constexpr (kTvd) {
             // d TVD / d z = q (s Q - S) / (2 tau) with s = sign(q - p), S = sum q s
             // and Q = sum q (1 up to rounding; summed, it cancels S exactly where
-            // every s is the same): k1 q' + k2 |q'| with k1 = Q / (2 tau), k2 = -S / (2 tau)
+            // every s is the same): k1 q' + k2 |q'| with k1 = Q / (2 tau), k2 = -S / (2 tau).
+            // kApart: q' Q- / tau, or q' Q+ / tau where q' < 0, both products of positive sums,
+            // where s Q - S cancels to 2 Q- of rows whose smaller side holds little mass
             const float k1 = sa, k2 = sb;
+            const uint32_t fpos = __float_as_uint(sa), fdiff = fpos ^ __float_as_uint(sb);
+            auto factor = [&](float q) {
+                const uint32_t neg = static_cast<uint32_t>(__float_as_int(q) >> 31);
+                return __uint_as_float(fpos ^ (neg & fdiff));
+            };
+            auto grad = [&](float q) { return kApart ? q * factor(q) : fmaf(k2, fabsf(q), k1 * q); };
             sweep_tm<In, false, false, false, false, false>(tw, tsh, nv, 0, rj, tz, tt,
                 [&](const float*, const float*, auto tag, int j0, float, float, bool, uint4& zr, uint4& tr) {
                     constexpr int kCnt = decltype(tag)::value;
@@ -1530,12 +1581,21 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                         float q[kVec], gr[kVec];
                         unpack_q<In>(zr, tr, q);
 #pragma unroll
-                        for (int e = 0; e < kVec; ++e) gr[e] = fmaf(k2, fabsf(q[e]), k1 * q[e]);
+                        for (int e = 0; e < kVec; e += 2) {
+                            if constexpr (kApart) {
+                                const float2 r = mul2(make_float2(q[e], q[e + 1]), make_float2(factor(q[e]), factor(q[e + 1])));
+                                gr[e] = r.x;
+                                gr[e + 1] = r.y;
+                            } else {
+                                gr[e] = grad(q[e]);
+                                gr[e + 1] = grad(q[e + 1]);
+                            }
+                        }
 #pragma unroll
                         for (int e = 0; e < kVec; e += 4) stg_v4(orow + j0 + e, gr[e], gr[e + 1], gr[e + 2], gr[e + 3]);
                     }
                 });
-            if (tid < tail) orow[kAnyPhase ? rj() : tail0 + tid] = fmaf(k2, fabsf(tq), k1 * tq);
+            if (tid < tail) orow[kAnyPhase ? rj() : tail0 + tid] = grad(tq);
         } else {
             // JSD: q (log2(q/m) - S), every probability carrying the gradient's factor,
             // which cancels in log2(q/m); RKL: q ((z - gz) - (t - tp) - X / E) / tau^2,

@@ -416,3 +416,40 @@ def test_rows_off_the_16_byte_grid(osd, kind, N, V, dtype, shift):
     lr, gr = _oracle(z, t, mask, kind, 0.3)
     check_distill(loss.cpu().numpy(), g.cpu().numpy(), lr, gr, mask.numpy() == 1,
                   _tvd_ambiguous(z, t) if kind == "tvd" else None)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V", [32001, 2053])
+@pytest.mark.parametrize("side", ["above", "below"])
+def test_tvd_with_little_mass_on_one_side(osd, side, V, dtype):
+    """Rows off the 16-byte grid whose q lies above p (or below) at one entry alone, with 1, 0.1
+    and 0.01 % of q's mass there: the gradient of every other entry carries that mass as a
+    factor, and that entry's is the row's largest.  Its relative error, at an exponent of up
+    to 13.3: 3.3e-7 from rounding that to 2^-21, 1.2e-7 from log2(e)'s to 1.3e-8, 1.7e-7 from
+    the normaliser's logarithm (2^-22), 2.4e-7 from ex2.approx (2^-22) and 1.2e-7 from the
+    sum and the product: below 1e-6.  The loss sums |q - p| of numbers that add up to 1 each
+    and are good to 2^-21: 5e-7, absolute."""
+    eps = [1e-2, 1e-3, 1e-4]
+    g = torch.Generator().manual_seed(V)
+    z = torch.randn(16 * len(eps), V, generator=g) * 2.0
+    z[:, 7] = 14.0  # most of the mass
+    at = torch.randint(8, V, (z.shape[0],), generator=g)
+    r = torch.arange(z.shape[0])
+    e = torch.tensor(eps, dtype=torch.float64).repeat_interleave(16)
+    z = z.to(dtype)
+    z[r, at] = -200.0
+    rest = torch.logsumexp(z.double(), -1)
+    t = z.clone()
+    z[r, at] = (rest + torch.log(e / (1 - e))).to(dtype)                       # q = e there
+    other = e / 8 if side == "above" else torch.full_like(e, 0.5)
+    t[r, at] = (rest + torch.log(other / (1 - other))).to(dtype)               # p = e / 8, or 1 / 2
+    q, p = torch.softmax(z.double(), -1), torch.softmax(t.double(), -1)
+    up = q > p
+    qa, qb = (q * up).sum(-1, keepdim=True), (q * ~up).sum(-1, keepdim=True)
+    assert ((qa if side == "above" else qb) < 0.02).all()
+    ref = torch.where(up, q * qb, -q * qa).numpy()
+    loss, grad = _run(osd, z, t, None, "tvd", 0.5)
+    np.testing.assert_allclose(loss, (0.5 * (q - p).abs().sum(-1)).numpy(), rtol=0, atol=5e-7)
+    err = np.abs(grad - ref).max(-1) / np.abs(ref).max(-1)
+    print(side, V, dtype, err.reshape(len(eps), -1).max(-1))
+    assert err.max() <= 1e-6, err.reshape(len(eps), -1).max(-1)
