@@ -315,46 +315,47 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
     };
     const float mt = sh.m[a], inv_st = 1.0f / sh.s[a];
     const float mz = bonus ? 0.f : sh.m[k + 1 + a];
-    const float inv_sz = bonus ? 0.f : 1.0f / sh.s[k + 1 + a];
+    const float st_sz = bonus ? 0.f : sh.s[a] / sh.s[k + 1 + a];
     const float ch = p.c_hi, cl = p.c_lo;
     const int nsub = (n + kSub - 1) / kSub;  // sub-tiles: one warp step of 32 x kW entries
     // raw entries of this lane in sub-tile s (slots past the span read as -inf: weight 0)
     struct Raw {
         uint4 t, z;
     };
-    auto load_sub = [&](int s, Raw& r) {
+    auto load_sub = [&](auto has_q, int s, Raw& r) {
+        constexpr bool kQ = decltype(has_q)::value;
         const int j0 = e0 + s * kSub + lane * kW;
         const int cnt = min(kW, e0 + n - j0);
-        if (cnt == kW && inside(trow, j0) && (bonus || inside(zrow, j0))) {
+        if (cnt == kW && inside(trow, j0) && (!kQ || inside(zrow, j0))) {
             r.t = ldv(trow, j0);
-            r.z = bonus ? r.t : ldv(zrow, j0);
+            if constexpr (kQ) r.z = ldv(zrow, j0);
         } else {
             float tv[kW], zv[kW];
 #pragma unroll
             for (int e = 0; e < kW; ++e) {
                 tv[e] = (e < cnt) ? ld1(trow, j0 + e) : kNegInf;
-                zv[e] = (e < cnt && !bonus) ? ld1(zrow, j0 + e) : kNegInf;
+                zv[e] = (e < cnt && kQ) ? ld1(zrow, j0 + e) : kNegInf;
             }
             r.t = pack_raw<In, kW>(tv);
-            r.z = pack_raw<In, kW>(zv);
+            if constexpr (kQ) r.z = pack_raw<In, kW>(zv);
         }
     };
-    // residual weights of one sub-tile slot, in pairs (both passes take them here, so
-    // they round identically)
-    auto sub_weights = [&](const Raw& r, float2* w) {
+    // residual weights of one sub-tile slot times st, the target row's sum, in pairs:
+    // e_t, or max(0, e_t - e_z st / sz) with one rounding, so that entries of equal
+    // probability weigh exactly 0 where the two sums are equal.  (The difference of two
+    // rounded products does not: ptxas fuses a packed product into it.)  has_q (a
+    // std::true_type) unless a = k: with a branch on `bonus` among the loads and sums instead, B =
+    // 256, k = 8, V = 128256 took 78.8 us where it takes 69.9 (0.13 accepted), k = 1 71.1 for 63.9.
+    auto sub_weights = [&](auto has_q, const Raw& r, float2* w) {
         float2 d[kW / 2];
         E::minus(r.t, mt, d);
 #pragma unroll
         for (int e = 0; e < kW / 2; ++e) w[e] = exp2_pair(d[e], ch, cl);
-        if (bonus) {
-#pragma unroll
-            for (int e = 0; e < kW / 2; ++e) w[e] = mul2(w[e], f2(inv_st));
-        } else {
+        if constexpr (decltype(has_q)::value) {
             E::minus(r.z, mz, d);
 #pragma unroll
             for (int e = 0; e < kW / 2; ++e) {
-                const float2 q = mul2(exp2_pair(d[e], ch, cl), f2(-inv_sz));
-                const float2 df = fma2(w[e], f2(inv_st), q);
+                const float2 df = fma2(exp2_pair(d[e], ch, cl), f2(-st_sz), w[e]);
                 w[e] = make_float2(fmaxf(df.x, 0.f), fmaxf(df.y, 0.f));
             }
         }
@@ -363,28 +364,32 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
     // pass 1: one fp32 sum per sub-tile, no block barrier; the sums of a step are
     // reduced over the lanes together
     static_assert(kFinUnroll == 4, "warp_sum4 carries four sums");
-    for (int s0 = warp; s0 < nsub; s0 += kWarps * kFinUnroll) {
-        Raw r[kFinUnroll];
+    auto pass1 = [&](auto has_q) {
+        for (int s0 = warp; s0 < nsub; s0 += kWarps * kFinUnroll) {
+            Raw r[kFinUnroll];
 #pragma unroll
-        for (int u = 0; u < kFinUnroll; ++u)
-            if (s0 + u * kWarps < nsub) load_sub(s0 + u * kWarps, r[u]);
-        float sum[kFinUnroll];
+            for (int u = 0; u < kFinUnroll; ++u)
+                if (s0 + u * kWarps < nsub) load_sub(has_q, s0 + u * kWarps, r[u]);
+            float sum[kFinUnroll];
 #pragma unroll
-        for (int u = 0; u < kFinUnroll; ++u) {
-            sum[u] = 0.f;
-            if (s0 + u * kWarps < nsub) {
-                float2 w[kW / 2];
-                sub_weights(r[u], w);
-                float2 s2 = w[0];
+            for (int u = 0; u < kFinUnroll; ++u) {
+                sum[u] = 0.f;
+                if (s0 + u * kWarps < nsub) {
+                    float2 w[kW / 2];
+                    sub_weights(has_q, r[u], w);
+                    float2 s2 = w[0];
 #pragma unroll
-                for (int e = 1; e < kW / 2; ++e) s2 = add2(s2, w[e]);
-                sum[u] = s2.x + s2.y;
+                    for (int e = 1; e < kW / 2; ++e) s2 = add2(s2, w[e]);
+                    sum[u] = s2.x + s2.y;
+                }
             }
+            const float tot = warp_sum4(sum);
+            const int s = s0 + (lane >> 3) * kWarps;
+            if ((lane & 7) == 0 && s < nsub) s_sub[s] = tot * inv_st;
         }
-        const float tot = warp_sum4(sum);
-        const int s = s0 + (lane >> 3) * kWarps;
-        if ((lane & 7) == 0 && s < nsub) s_sub[s] = tot;
-    }
+    };
+    if (bonus) pass1(std::false_type());
+    else pass1(std::true_type());
     __syncthreads();
     // span total, exact, reduced across warp 0
     bool got = true;
@@ -475,15 +480,19 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
         if (mode == 0 || mode == 1) {
             float w[kW];
             {
-                Raw r;
-                if (s >= 0) load_sub(s, r);
-                else { r.t = ninf_raw<In>(); r.z = r.t; }
                 float2 w2[kW / 2];
-                sub_weights(r, w2);
+                auto at_tile = [&](auto has_q) {
+                    Raw r;
+                    if (s >= 0) load_sub(has_q, s, r);
+                    else { r.t = ninf_raw<In>(); r.z = r.t; }
+                    sub_weights(has_q, r, w2);
+                };
+                if (bonus) at_tile(std::false_type());
+                else at_tile(std::true_type());
 #pragma unroll
                 for (int e = 0; e < kW / 2; ++e) {
-                    w[2 * e] = w2[e].x;
-                    w[2 * e + 1] = w2[e].y;
+                    w[2 * e] = w2[e].x * inv_st;
+                    w[2 * e + 1] = w2[e].y * inv_st;
                 }
             }
             const int j0 = e0 + max(s, 0) * kSub + lane * kW;

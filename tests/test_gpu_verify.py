@@ -152,6 +152,28 @@ def test_peak_of_a_lone_bonus_row(osd, B, k, V, rest):
         assert np.abs(gap - gap_ref).max() <= 2e-6, np.abs(gap - gap_ref).max()
 
 
+@pytest.mark.parametrize("B,k,V", [(32, 2, 4096), (150, 2, 8192), (16, 3, 128256), (1, 1, 32000)])
+def test_entries_of_equal_probability_have_no_residual_weight(osd, B, k, V):
+    """p and q differ at two entries alone, which trade places: the residual max(0, p - q) is all
+    at one of them, 1e-7 or so of p, less than the rounding errors of the other entries."""
+    g = torch.Generator().manual_seed(V)
+    z = torch.randn(B, k, V, generator=g) * 2.0
+    z[..., 5] = 9.0
+    i = 2 * torch.randint(64, (V - 8) // 2, (B,), generator=g)
+    i = i // 8 * 8 + 1  # entries 1 and 3 of a 16-byte vector: every sum takes them alike
+    r = torch.arange(B)
+    z[r, 0, i], z[r, 0, i + 2] = -26.0, -6.0
+    t = torch.cat([z, torch.randn(B, 1, V, generator=g)], dim=1)
+    t[r, 0, i], t[r, 0, i + 2] = -6.0, -26.0
+    y = torch.randint(0, V, (B, k), generator=g, dtype=torch.int32)
+    y[:, 0] = (i + 2).to(torch.int32)  # p / q = e^-20: always rejected
+    inp = {"draft": z.to(torch.bfloat16), "target": t.to(torch.bfloat16), "tokens": y,
+           "uniforms": torch.rand(B, k + 1, generator=g).clamp_(min=1e-3)}
+    res, ref = _run(osd, inp, 1.0)
+    assert (res.accepted.cpu() == 0).all() and (ref["accepted"] == 0).all()
+    np.testing.assert_array_equal(res.out_tokens[:, 0].cpu().numpy(), i.numpy())
+
+
 GREEDY_CASES = [
     (16, 3, 1, torch.float32), (32, 4, 1001, torch.bfloat16), (9, 2, 40000, torch.float32),
     (12, 5, 32000, torch.bfloat16), (38, 7, 32768, torch.bfloat16), (7, 3, 4096, torch.bfloat16),
