@@ -414,8 +414,11 @@ __device__ __forceinline__ uint32_t cluster_rank() {
     return r;
 }
 // The .aligned forms need a converged warp, hence the __syncwarp() first.
-// Arrive without ordering: used once this CTA has consumed every value it read
-// from its peers' shared memory, to tell them they may exit.
+// Arrive without ordering: once this CTA has consumed every value it read
+// from its peers' shared memory, to tell them they may exit; and after a thread's
+// fence_mbarrier_init, which is all that peers need to push to its barriers (a release by
+// every thread, 2.6 us while the rows' copies fill the memory queue, made verification of 32
+// x 5 x 32000 with a cold L2 21.5 us instead of 19.0, of 4 x 4 x 32000 17.2 instead of 15.6).
 __device__ __forceinline__ void cluster_arrive_relaxed() {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");

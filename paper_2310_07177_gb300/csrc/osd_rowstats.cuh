@@ -323,7 +323,7 @@ greedy_walk_kernel(Walk wk, const In* target, int V, int csize, int span, int wi
         return;
     }
     // the barriers are initialised before any peer pushes to them: arrive now, wait before the first push
-    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (csize > 1) cluster_arrive_relaxed();
     for (unsigned round = 0;; ++round) {
         const int node = s_node;
         int w = 1;

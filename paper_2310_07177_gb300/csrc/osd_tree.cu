@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p, i
         for (int i = tid; i < n; i += kTreeThreads) p.diag_margin[size_t(b) * n + i] = __int_as_float(0x7fc00000);
     __syncthreads();  // the barriers are initialised before anyone waits on them
     // ... and before any peer pushes to them: arrive now, wait before the first push
-    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (csize > 1) cluster_arrive_relaxed();
 
     constexpr int kRound = 0, kMass = 1, kDraw = 2, kGone = 3, kBad = 4;  // what comes next
     int act = kRound, node = 0;  // node: the round's first

@@ -649,7 +649,7 @@ verify_lazy_kernel(FinParams p, int win, int ahead) {
     }
     __syncthreads();  // the barriers are initialised before anyone waits on them
     // ... and before any peer pushes to them: arrive now, wait before the first push
-    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (csize > 1) cluster_arrive_relaxed();
     // the draft tokens, the two logits each accept test needs, and the uniforms: two dependent
     // loads of one warp, which the others do not wait for before they start on the rows
     int bad = 0;
@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(kFuseThreads) verify_fused_kernel(FinParams p)
     }
     __syncthreads();  // the barriers are initialised before anyone waits on them
     // ... and before any peer pushes to them: arrive now, wait before the first push
-    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (csize > 1) cluster_arrive_relaxed();
     // meanwhile the draft tokens, the two logits each accept test needs, and the uniforms
     int bad = 0;
     if (warp == kWarps - 1) {
