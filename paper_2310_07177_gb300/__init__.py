@@ -3,8 +3,8 @@
 Thin binding over ``libosd.so`` (the C ABI in ``include/osd.h``): it turns torch
 tensors into device pointers, sizes and the current CUDA stream, allocates
 outputs with torch, and raises ``OsdError`` on a non-OK status.  Calls with plain
-CUDA tensors go through native code (``csrc/osd_binding.cpp``); any other call is
-checked here and goes through ctypes.
+CUDA tensors go through native code (``csrc/osd_binding.cpp``) where that is built for
+this torch and Python; any other call is checked here and goes through ctypes.
 Every step of verify and distill runs in the library's CUDA kernels; there is
 no CPU path.  If the library has not been built, calls raise immediately.
 
@@ -20,6 +20,7 @@ import ctypes
 import importlib.machinery
 import importlib.util
 import os
+import warnings
 from typing import NamedTuple, Optional
 
 import torch
@@ -90,12 +91,26 @@ def load_library():
 _binding = None
 
 
+class _NoBinding:
+    """Stands in for the native calls: takes none, so that every call goes through ctypes."""
+
+    @staticmethod
+    def _none(*args):
+        return None
+
+    verify = distill = distill_accepted = mixed_sample = verify_tree = _none
+
+
 def _load_binding():
-    """The native calls (raises if they have not been built)."""
+    """The native calls, or _NoBinding (with a warning) where they have not been built for
+    this torch and Python: ctypes makes the same calls."""
     global _binding
     load_library()
     if not os.path.exists(BINDING_PATH):
-        raise RuntimeError(f"{BINDING_PATH} not found: build it with paper_2310_07177_gb300.build_library()")
+        warnings.warn(f"{BINDING_PATH} not found: calls go through ctypes, 10 to 20 us slower; build it with "
+                      "paper_2310_07177_gb300.build_library()", RuntimeWarning, 3)
+        _binding = _NoBinding
+        return _binding
     loader = importlib.machinery.ExtensionFileLoader("_binding", BINDING_PATH)
     mod = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_binding", BINDING_PATH, loader=loader))
     loader.exec_module(mod)

@@ -1,5 +1,5 @@
 """Build libosd.so (the CUDA kernels behind include/osd.h) in-tree with nvcc,
-and _binding.so, the Python calls in native code over it, with g++.
+and the binding, the Python calls in native code over it, with g++.
 
 One translation unit per source file, compiled in parallel (the kernels for
 sm_103a only), then linked into ``paper_2310_07177_gb300/libosd.so`` against the
@@ -15,6 +15,8 @@ import shutil
 import subprocess
 import sysconfig
 
+import torch
+
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
@@ -22,7 +24,9 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD_DIR = os.path.join(PKG, "_build")
 LIB_PATH = os.path.join(PKG, "libosd.so")
 BINDING_SRC = os.path.join(CSRC, "osd_binding.cpp")
-BINDING_PATH = os.path.join(PKG, "_binding.so")
+# compiled against torch's C++ and Python's C interface, of which its name says the versions:
+# one of another torch or Python is neither taken for current nor loaded
+BINDING_PATH = os.path.join(PKG, f"_binding-{torch.__version__}-{sysconfig.get_config_var('SOABI')}.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
@@ -52,7 +56,7 @@ def up_to_date() -> bool:
 
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) -> str:
-    """Compile every .cu under csrc/ and the binding, link libosd.so and _binding.so;
+    """Compile every .cu under csrc/ and the binding, link libosd.so and the binding;
     returns the path of the former."""
     if not force and up_to_date():
         return LIB_PATH
@@ -69,8 +73,6 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
         if verbose or ptxas_info:
             print(r.stdout + r.stderr)
         return obj
-
-    import torch  # for its headers and libraries
 
     tdir = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(exe)))
@@ -100,7 +102,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
            "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10_cuda", "-lc10"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
-        raise RuntimeError(f"link of _binding.so failed:\n{r.stdout}\n{r.stderr}")
+        raise RuntimeError(f"link of the binding failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, BINDING_PATH)
     return LIB_PATH
 

@@ -135,3 +135,23 @@ def test_product_path_fails_loudly_without_library(tmp_path, monkeypatch):
     monkeypatch.setattr(osd, "_lib", None)
     with pytest.raises(RuntimeError, match="missing"):
         osd.load_library()
+
+
+def test_binding_of_another_torch_is_not_used(lib, monkeypatch, tmp_path):
+    """The binding's name says which torch and Python it was built for: for another one a build is
+    due, and until then the calls go through ctypes, with a warning."""
+    import torch
+
+    import paper_2310_07177_gb300 as osd
+    from paper_2310_07177_gb300 import _build
+    assert torch.__version__ in os.path.basename(_build.BINDING_PATH) and _build.up_to_date()
+    other = str(tmp_path / "_binding-0.0-other.so")
+    monkeypatch.setattr(_build, "BINDING_PATH", other)
+    assert not _build.up_to_date()
+    monkeypatch.setattr(osd, "BINDING_PATH", other)
+    monkeypatch.setattr(osd, "_binding", None)
+    with pytest.warns(RuntimeWarning, match="ctypes"):
+        binding = osd._load_binding()
+    assert binding.verify(*[None] * 9) is None and binding.verify_tree(*[None] * 10) is None
+    with pytest.raises(ValueError, match="CUDA tensors only"):  # the Python code's own checks
+        osd.osd_mixed_sample(torch.zeros(2, 3), torch.zeros(2, 3), torch.zeros(2), 0.5)
