@@ -1693,11 +1693,15 @@ static cudaError_t allow_wide_clusters() {
     return cudaSuccess;
 }
 
-// Whether a grid starts before the previous kernel's end (grid_dependency_sync), which gains 2
+// Whether a grid starts before the previous kernel's end (grid_dependency_sync), which gains 1
 // to 3 us a call of few rows (16 x 32000: 8.2 -> 5.0 us).  Where a call fills the SMs, the next
 // one's CTAs then pile up on those that become free first: 146 sequences of 3 x 29952
-// accepted JSD 15.6 us against 13.2 without.
-static bool start_early(long long ctas) { return ctas <= 2LL * device_sms(); }
+// accepted JSD 15.6 us against 13.2 without, and where long spans leave room for two CTAs an
+// SM, `per_sm`, from 8/5 of the SMs on: accepted rows of 83336 fp32, 36 of 5, RKL 15.4 against 12.1
+// (FKL, 90 % accepted, 8.9 against 9.3), 38 of 5 x 89620 TVD 18.5 against 16.2, 30 of them level.
+static bool start_early(long long ctas, long long per_sm = 0) {
+    return ctas <= 2LL * device_sms() && !(per_sm == 2 && ctas * 5 > 8LL * device_sms());
+}
 
 template <typename In, int kKind, bool kAligned, int kT>
 static cudaError_t launch_distill_kind(const DistParams& dp, long long rows, size_t smem, cudaStream_t s) {
@@ -1724,8 +1728,9 @@ static cudaError_t launch_distill_kind(const DistParams& dp, long long rows, siz
             }
         }
     }
-    return launch_ex(kEarlyStart<kKind, kT> && start_early(rows * dp.csize), kern, dim3(static_cast<unsigned>(rows * dp.csize)), dim3(kT), smem, s,
-                     dp.csize, dp);
+    const long long per_sm = 227 * 1024 / (static_cast<long long>(smem) + 2048);  // (1 KB reserved, 1 KB static)
+    return launch_ex(kEarlyStart<kKind, kT> && start_early(rows * dp.csize, per_sm), kern,
+                     dim3(static_cast<unsigned>(rows * dp.csize)), dim3(kT), smem, s, dp.csize, dp);
 }
 
 // (TVD, whose extra cluster exchange costs more with wide CTAs, always takes kDistThreads.)
