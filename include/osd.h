@@ -113,10 +113,12 @@ osd_status osd_verify_workspace_size(int B, int k, int V, size_t *bytes);
  * uniforms       [B, k+1]     fp32 in [0, 1) (not read when T == 0)
  * temperature    >= 0 and finite, else OSD_ERR_INVALID_ARG
  * accepted       [B]          out: a in 0..k; -1 if any draft token of the
- *                             sequence lies outside [0, V), or (small batches
- *                             at T > 0, whose rows are staged by bulk copy) if
- *                             the GPU did not deliver the sequence's rows within
- *                             a one-second bound
+ *                             sequence lies outside [0, V), or if a bounded
+ *                             wait gave up: one second for rows staged by bulk
+ *                             copy (some T > 0 calls), three for what the
+ *                             thread blocks that share a sequence tell each
+ *                             other (T > 0, and large batches at T = 0); its
+ *                             tokens are then -1 and its mask 0 as well
  * out_tokens     [B, k+1]     out: y_0..y_{a-1}, the sampled token at a, then -1
  * mismatch_mask  [B, k]       out: 1 at i == a when a < k, else 0 (the first
  *                             rejected position, the rows Algorithm 1 keeps
@@ -128,8 +130,8 @@ osd_status osd_verify_workspace_size(int B, int k, int V, size_t *bytes);
  *                             when T == 0)
  * workspace      device scratch of at least osd_verify_workspace_size()
  *                bytes, 16-byte aligned; contents need no initialisation and
- *                are garbage afterwards.  Calls that overlap on the GPU
- *                must not share it.
+ *                are garbage afterwards (of the present kernels only those at
+ *                T = 0 use it).  Calls that overlap on the GPU must not share it.
  * Limits: 1 <= k <= OSD_VERIFY_MAX_K, 1 <= V <= OSD_VERIFY_MAX_V, B >= 0.
  */
 osd_status osd_verify(const void *draft_logits, const void *target_logits,
@@ -278,7 +280,8 @@ osd_status osd_verify_tree_workspace_size(int B, int n_nodes, int V, size_t *byt
  * uniforms       [B, n_nodes] fp32 in [0, 1): u[b, i] tests node i, u[b, 0]
  *                drives the extra draw (not read at T == 0)
  * accepted       [B] out: accepted tokens (the depth reached), -1 if a token
- *                lies outside [0, V)
+ *                lies outside [0, V) or a bounded wait gave up (three seconds,
+ *                as in osd_verify)
  * path           [B, n_nodes] out: the accepted nodes, root excluded, then -1
  * out_tokens     [B, n_nodes] out: the accepted tokens, the extra token, then -1
  * last_node      [B] out: the node where the walk stopped (its rows are the

@@ -1975,7 +1975,7 @@ static osd_status distill_run(const void* draft_logits, const void* target_logit
     // Rows off the 16-byte grid take the runs too where every row's draft, target and gradient
     // share one phase in it, as those of contiguous tensors do (V = 32001): the same
     // bulk copies from the row's first boundary, its head and tail entry by entry (4096 x 32001
-    // bf16: TVD 192 us, FKL 182, JSD 218, CE, on the per-row kernel with the same copies, 181; with
+    // bf16: TVD 201 us, FKL 182, JSD 218, CE, on the per-row kernel with the same copies, 181; with
     // 2-byte loads and 4-byte stores on the per-row kernel they took 455, 512, 775 and 488 us).
     // Where the phases differ (a view of [B, k + 1, V], rows chosen by verification) the per-row
     // kernel shifts the rows into place as it loads them (1024 x 32003 bf16 RKL against such a

@@ -393,9 +393,10 @@ greedy_walk_kernel(Walk wk, const In* target, int V, int csize, int span, int wi
 // Launch a greedy walk over B sequences of `rows` rows each, at most `depth` of them on any
 // walk, or return false where the pass over every row does better: that one reads at the copy
 // bandwidth, a walk pays about 2.5 us a round.  Trees, of which a walk sees the smaller part,
-// from 20 MB and a CTA an SM on (27 nodes: 16 x 32000 9.0 -> 5.6 us, 64 x 100000 58.5 -> 17,
-// 48 x 128256 fp32 96 -> 21; 2 x 135808 fp32 10.2 against 12.4); chains only where one position is 40 MB (256 x 9 x 128256: 90.5 us, on demand 32 with
-// 0.15 accepted, 59 with 1.7 and 98 with 6.4; 32 x 9 x 128256, 8 MB: 16.6 against 16 and 23).
+// from 20 MB and 8 sequences on (27 nodes: 16 x 32000 8.7 -> 5.1 us, 64 x 100000 58 -> 15,
+// 48 x 128256 fp32 96 -> 20; 2 x 135808 fp32 8.9 against 9.3); chains only where one position is
+// 40 MB (256 x 9 x 128256: 90 us, on demand 27 with 0.02 accepted, 54 with 0.9, 77 with 3.5 and
+// 100 with 6.4; 32 x 9 x 128256, 8 MB: 16.4 against 6.9 and 21 with the first and the last draft).
 template <typename In, typename Walk>
 static bool launch_greedy_walk(const Walk& wk, const In* target, int B, int rows, int depth, int V, cudaStream_t stream,
                                osd_status* st) {

@@ -164,10 +164,10 @@ struct GreedyTree {
 // a mass pass, whose span totals meet the same way, or the walk leaves the round.
 //
 // What bounds it: the chain of dependent phases, about 3 us a round and 2 us a rejection.
-// B = 32, 27 nodes, V = 32000 (1.8 accepted): 24 us where the statistics of every node's rows
-// took 44; V = 128256: 50 us against 125; B = 64, V = 32001: 39 us against 107.  Two CTAs an SM
-// at 120 registers: with three or four the passes spill (33 and 35 us); rows staged in
-// shared memory first took 26 us, and at V = 128256, where they leave one CTA an SM, 79 us.
+// B = 32, 27 nodes, V = 32000 (1.8 accepted): 23.3 us where the statistics of every node's rows
+// took 43.8; V = 128256: 48 us against 125; B = 64, V = 32001: 41 us against 109.  Two CTAs an SM
+// at 120 registers: with three or four the passes spill (33 and 35 us, where two took 24); rows
+// staged in shared memory first took 26 us, and at V = 128256, where they leave one CTA an SM, 79 us.
 template <typename In, bool kAligned>
 __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p, int win) {
     using E = Elem<In>;
@@ -681,8 +681,8 @@ static osd_status launch_tree(const TreeParams& base, int B, const void* draft, 
         return from_cuda(launch_ex(true, tree_greedy_kernel, dim3(unsigned(B)), dim3(kGreedyThreads), 0, stream, 1, tp));
     }
     // CTAs per sequence: 8, but 4 where 8 would run past one wave (two CTAs an SM) and the
-    // spans stay short (B = 48 and 64 at V = 32000: 31.9 and 38.3 us against 42.5 and 48.4; at
-    // V = 64000, B = 64 the two are level, 59 and 58 us)
+    // spans stay short (B = 48 and 64 at V = 32000: 30.7 and 36.6 us against 39.7 and 44.9; at
+    // V = 64000, B = 64 55.6 against 52.5)
     int c = kSeqMaxCluster;
     if ((long long)B * c > 2LL * device_sms() && V <= 50000) c /= 2;
     while (c > 1 && V <= 2048 * c) c /= 2;
@@ -691,9 +691,9 @@ static osd_status launch_tree(const TreeParams& base, int B, const void* draft, 
     if ((long long)B * tp.csize > INT_MAX) return OSD_ERR_UNSUPPORTED;
     // Nodes per round, by the bytes of one node of the batch: a round costs about 3 us beside
     // them, and first children that the walk does not come to are read for nothing (B = 1,
-    // V = 32000: 4 nodes 15.4 us, 1 node 19.5; B = 32: 26.0, 2 nodes 24.1, 1 node 25.9; B = 64,
-    // V = 128256, 33 MB: 2 nodes 86, 4 nodes 88; B = 64, V = 150016 fp32, 77 MB: 1 node 121, 2 nodes
-    // 142).  A tree without siblings passes them often (B = 32, 9 nodes: 4 nodes 24.3 us, 2 nodes 28.7).
+    // V = 32000: 4 nodes 14.2 us, 1 node 18.4; B = 32: 24.8, 2 nodes 23.1, 1 node 25.3; B = 64,
+    // V = 128256, 33 MB: 2 nodes 85, 4 nodes 93, 1 node 83; B = 64, V = 150016 fp32, 77 MB: 1 node 134, 2
+    // nodes 150).  A tree without siblings passes them often (B = 32, 9 nodes: 4 nodes 19.6 us, 2 21.3).
     const double pos = double(B) * 2 * V * double(es);
     bool siblings = false;
     for (int i = 0; i < n; ++i) siblings |= tp.topo.next_sibling[i] >= 0;

@@ -567,14 +567,14 @@ __device__ __forceinline__ bool residual_draw(const FinParams& p, int b, int a, 
 // holds.
 //
 // What bounds it: with a poor draft at B = 256, k = 8, V = 128256 (0.13 accepted) the two
-// rows a sequence needs are 148 MB, 22 us at the copy bandwidth, of which it takes
-// 76 us (all rows in two launches: 211 us), 50 % issue activity, the rest waits of the
-// dependent phases (statistics, exchange, draw); the same batch with 2.8 accepted takes
-// 153 us (211), with 6.8, where nearly every row is read, 218 us (208).  64 registers and four
-// CTAs an SM with groups of 4 vectors in flight measured best (groups of 2 with five or six
-// CTAs: 84 us); staging the first position in shared memory at these sizes, three CTAs an
-// SM, gave 70 us with the poor draft and 257 us with the good one, whose rounds then wait
-// for their copies.
+// rows a sequence needs are 148 MB, 22 us at the copy bandwidth; it takes 70 us (all
+// rows in two launches: 211 us), half of the issue slots idle while the dependent phases
+// (statistics, exchange, draw) wait for each other.  The same batch with 3.0 accepted takes
+// 148 us (211), with 5.6 185 us (209), with 7.1, where nearly every row is read, 209 us (208).
+// 64 registers and four CTAs an SM with groups of 4 vectors in flight measured best, at 76 us
+// (groups of 2 with five or six CTAs: 84 us); staging the first position in shared memory
+// at these sizes, three CTAs an SM, then gave 70 us with the poor draft and 257 us with the good
+// one, whose rounds wait for their copies.
 constexpr int kLazyMaxWin = 8;                 // positions per round ...
 constexpr int kLazyMaxRows = 2 * kLazyMaxWin;  // ... two rows each
 constexpr int kLazyThreads = 256;
@@ -740,9 +740,9 @@ verify_lazy_kernel(FinParams p, int win, int ahead) {
 // per row, so that a row's statistics start as soon as it has landed), and one
 // exchange decides all the positions.  It runs only when its grid fits in one wave with
 // slots to spare (see launch_sampling).  At B = 32, k = 5, V = 32000 (22 MB, 3.3 us at the copy
-// bandwidth) it takes 12.0 us back to back, 19.7 us alone with a cold L2: a chain of copy,
-// statistics, exchange, tests and draw, barrier stalls first (6.7 warps an issue).  512
-// threads (256 threads 12 % more; 16-CTA clusters 60 % more).
+// bandwidth) it takes 11.4 us back to back, 19.0 us alone with a cold L2: a chain of copy,
+// statistics, exchange, tests and draw.  512 threads (256 threads 12 % more; 16-CTA
+// clusters 60 % more).
 constexpr int kFuseThreads = 512;
 constexpr int kFuseParts = 4;           // warp items per row for the span statistics
 constexpr int kFuseMaxB = 64;           // at most this many sequences, and the grid in one wave
@@ -888,7 +888,8 @@ static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
     if (aligned && B <= kFuseMaxB) {
         // every row staged, only in one wave and with slots to spare, since a grid that just
         // fits finds them scattered over the GPCs: at B = 32, k = 5, V = 32000 (two CTAs an SM, 256
-        // of 304 slots) 12.8 us against 14.4 us on demand; at B = 36, V = 20224 (288) 16.6 against 10.1
+        // of 304 slots) 11.4 us whatever the draft, against 13.3 us on demand from 2 accepted on (11.6
+        // with 0.6); at B = 36, V = 20224 (288) 14.2 against 12.0
         split_vocab(V, kSeqMaxCluster, &fp);
         const size_t smem = fused_recv_offset(2 * k + 1, fp.span, es) + size_t(fp.csize) * (2 * k + 1) * sizeof(MaxSum);
         if (smem <= kStageMaxSmem &&
@@ -898,10 +899,10 @@ static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
     }
     // Rows on demand.  A round costs about 2 us beside its bytes, and positions past the
     // first failure are read for nothing: the first round takes 1 position from 40 MB a position
-    // of the batch on (B = 233, V = 27472 fp32, 51 MB: 36.8 us against 41.6 and 46.7 with 2 and 4),
-    // 2 from 10 MB (B = 204, V = 14144 fp32, 23 MB: 38.7 against 43.4 with 4), 4 from 2 MB
-    // (B = 100, V = 23488, 9 MB: 16.6 against 18.6 and 21.0 with 2 and 1), else 8 (B = 51, V = 10944:
-    // 14.4 against 15.4 with 4).
+    // of the batch on (B = 233, k = 4, V = 27472 fp32, 51 MB: 42.3 us against 44.5 and 45.0 with 2 and
+    // 4), 2 from 10 MB (B = 204, k = 4, V = 14144 fp32, 23 MB: 26.1, level with 26.5 and 25.5 with 1 and
+    // 4), 4 from 2 MB (B = 100, k = 4, V = 23488, 9 MB: 17.5 against 18.2 and 20.4 with 2 and 1; at
+    // B = 51, k = 6, V = 10944, 2.2 MB, 8 would do better, 10.7 against 12.6), else 8.
     constexpr int sub = 32 * Elem<In>::kVec;
     auto sub_bytes = [&]() { return size_t((fp.span + sub - 1) / sub) * sizeof(float); };
     const double pos = double(B) * 2 * V * double(es);  // bytes of one position of the batch
@@ -909,9 +910,9 @@ static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
     const int most = std::max(1, std::min<int>(kSeqMaxCluster, int(size_t(V) * es / 2048)));  // spans of 2 KB or more
     if (aligned && B <= device_sms() / 2) {
         // the first round staged where the batch runs at one CTA an SM, with fewer positions
-        // where they do not fit (B = 16, k = 8, V = 128256, 2 positions: 27 us against 39 us streamed;
-        // B = 36, k = 6, V = 20224: 10.1 us against 11.3), in pairs of SMs: with clusters of 3 or 5 a batch
-        // that just fits was slower (B = 28, V = 8704, 5 CTAs: 13.9 us, 4: 9.8)
+        // where they do not fit (B = 16, k = 8, V = 128256, 2 positions: 27.7 us against 43.7 us streamed;
+        // B = 36, k = 6, V = 20224: level, 12.6 us), in pairs of SMs: with clusters of 3 or 5 a batch
+        // that just fits is slower (B = 28, k = 5, V = 8704, 5 CTAs: 13.8 us, 4: 8.7)
         const int c = widest_cluster<verify_lazy_kernel<In, true, true>, kStagedThreads>(B, most, kStageMaxSmem, false) & ~1;
         if (c >= 2) split_vocab(V, c, &fp);
         for (int w = win; w >= 1 && c >= 2; w /= 2) {
@@ -926,16 +927,19 @@ static osd_status launch_sampling(FinParams fp, cudaStream_t stream) {
         }
     }
     // one wave of the widest clusters, not quite full, since a grid that just fits waits for its last
-    // slots (B = 192, V = 11200 with 3 CTAs a sequence, of which 194 fit: 27.0 us, with 2 25.1; B = 84,
-    // V = 38180 fp32, 6 CTAs: 21.0 us, with 8, of which 74 fit, 31.9; B = 186, V = 24576, 3: 20.5, with
-    // 4 27.0), as long as L2 holds a position for the draw; past that the fewest CTAs whose
-    // spans stay within 68 KB, so that the rows in flight do (B = 256, V = 128256 8 CTAs, 76 us
-    // against 85 and 102 us with 4 and 2)
+    // slots (B = 192, k = 4, V = 11200 with 3 CTAs a sequence, of which 194 fit: 20.9 us, with 2 18.3;
+    // B = 84, k = 4, V = 38180 fp32, 6 CTAs: 26.8 us, with 8, of which 74 fit, 31.5; B = 186, k = 2, V = 24576,
+    // 3: 18.0, with 4 23.2), as long as L2 holds a position for the draw; past that the fewest CTAs
+    // whose spans stay within 68 KB, so that the rows in flight do (B = 256, k = 8, V = 128256 8 CTAs,
+    // 70 us against 77 and 95 us with 4 and 2)
     int c = most;
     if (pos <= 100e6) {
-        // (batches past one wave: B = 340, 2 CTAs against 1: V = 32000 54 and 64 us, V = 8192 27 and 24)
+        // (batches past one wave: B = 340, k = 4, 2 CTAs against 1: V = 32000 46.3 and 58.7 us, V = 8192
+        // 23.6 and 22.1)
         const int c1 = size_t(V) * es >= 48 * 1024 ? 2 : 1;
-        constexpr size_t kSubs = 4096;  // more than any span within 100 MB takes
+        // the sub-tile sums of any span here: of V <= 2^21 fp32 entries over 8 CTAs 8 KB, over fewer
+        // (then the batch is larger and, within 100 MB, V smaller) less
+        constexpr size_t kSubs = 8192;
         c = std::max(c1, aligned ? widest_cluster<verify_lazy_kernel<In, false, true>, kLazyThreads>(B, most, kSubs, true)
                                 : widest_cluster<verify_lazy_kernel<In, false, false>, kLazyThreads>(B, most, kSubs, true));
     } else {
@@ -1115,7 +1119,7 @@ extern "C" osd_status osd_verify_noalloc(const void* draft_logits, const void* t
             scratch = slot.addr;
         }
     }
-    // The statistics pass writes every workspace entry before the finalize pass
+    // Only two launches at T = 0 use it: the first writes every entry before the second
     // reads it, so nothing in the shared array needs clearing between calls.
     return osd_verify(draft_logits, target_logits, dtype, B, k, V, draft_tokens, uniforms, temperature,
                       accepted, out_tokens, mismatch_mask, diag_margin, diag_cdf_gap, scratch,

@@ -53,10 +53,10 @@ CASES = [  # (B, k, V, dtype, T)
     (512, 4, 16, torch.bfloat16, 1.0),       # many sequences over a tiny vocabulary
     (1024, 8, 64, torch.float32, 0.7),
     (16, 64, 300, torch.bfloat16, 1.0),      # the largest k
-    (160, 2, 20000, torch.bfloat16, 1.0),    # past 128 sequences: 4 finalize CTAs per sequence
-    (130, 3, 40961, torch.float32, 0.7),     # the same, element-wise path
+    (160, 2, 20000, torch.bfloat16, 1.0),    # past 128 sequences: clusters of 3 or 4 CTAs
+    (130, 3, 40961, torch.float32, 0.7),     # the same, rows off the 16-byte grid
     (2, 3, 1 << 21, torch.bfloat16, 1.0),    # the largest vocabulary
-    # past 128 sequences the finalize takes clusters of at most 4 CTAs
+    # more of those
     (129, 1, 4096, torch.float32, 1.0),
     (200, 3, 8264, torch.bfloat16, 1.0),
     (300, 2, 16384, torch.float32, 0.7),     # exactly one slice
@@ -387,8 +387,8 @@ def test_workload_small_configs_full(osd, cfg):
 
 
 def test_unaligned_largest_vocabulary_past_128_sequences(osd):
-    """The element-wise finalize (rows off the 16-byte path) at B > 128 and a
-    vocabulary near the limit: its spans need more than four CTAs a sequence."""
+    """Rows off the 16-byte grid at B > 128 and a vocabulary near the limit: spans that
+    take more than four CTAs a sequence."""
     V = (1 << 21) - 1  # odd: bf16 rows are not 16-byte multiples
     spec = W.VerifySpec(130, 1, V, torch.bfloat16, 2.0, 1.0, 1.0, 1.0)
     inp = W.verify_inputs(spec, seed=2121, device="cuda")
