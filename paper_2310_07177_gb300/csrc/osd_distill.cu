@@ -990,8 +990,8 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
     // from Q+ and Q- (sums of q where q >= p and elsewhere) as tvd_gradient has it, and what
     // all q and all p of a row are off by in common (the rounding of cv and cu, which the
     // first chunks' references make large on peaked rows) taken out of both results.  Errors
-    // of 1.5e-7 to 2e-7 of the gradient's norm, 3e-8 to 2.3e-7 in the loss, for 2 % of the time (4096 x
-    // 32001 bf16 201 us).  The aligned runs form the gradient from sums over all entries,
+    // of 1.5e-7 to 2e-7 of the gradient's norm, 3e-8 to 2.3e-7 in the loss, for 1 % of the time (4096 x
+    // 32001 bf16 200 us).  The aligned runs form the gradient from sums over all entries,
     // which leaves it 2^-24 of the largest q, in absolute terms.
     constexpr bool kApart = kTvd && kAnyPhase;
     [[maybe_unused]] __shared__ float s_kap;
@@ -1405,14 +1405,15 @@ __global__ void __launch_bounds__(kTmThreads, 7) distill_tm_kernel(DistParams p,
                                     const float2 qq = make_float2(copysignf(qj.x, sd.x), copysignf(qj.y, sd.y));
                                     qs[e] = qq.x;
                                     if (two) qs[e + 1] = qq.y;
-                                    A2.x += fabsf(df.x);
-                                    if (two) A2.y += fabsf(df.y);
                                     const float2 qs2 = two ? qq : make_float2(qq.x, 0.f);
                                     const float2 qz = two ? qj : make_float2(qj.x, 0.f);
                                     if constexpr (kApart) {  // q + q' is 2 q where q >= p, else 0
+                                        A2 = add2(A2, make_float2(fabsf(df.x), two ? fabsf(df.y) : 0.f));
                                         C2 = add2(C2, sub2(qz, qs2));
                                         B2 = add2(B2, add2(qz, qs2));
                                     } else {
+                                        A2.x += fabsf(df.x);
+                                        if (two) A2.y += fabsf(df.y);
                                         B2 = add2(B2, qs2);
                                         C2 = add2(C2, qz);
                                     }
@@ -1975,7 +1976,7 @@ static osd_status distill_run(const void* draft_logits, const void* target_logit
     // Rows off the 16-byte grid take the runs too where every row's draft, target and gradient
     // share one phase in it, as those of contiguous tensors do (V = 32001): the same
     // bulk copies from the row's first boundary, its head and tail entry by entry (4096 x 32001
-    // bf16: TVD 201 us, FKL 182, JSD 218, CE, on the per-row kernel with the same copies, 181; with
+    // bf16: TVD 200 us, FKL 182, JSD 218, CE, on the per-row kernel with the same copies, 181; with
     // 2-byte loads and 4-byte stores on the per-row kernel they took 455, 512, 775 and 488 us).
     // Where the phases differ (a view of [B, k + 1, V], rows chosen by verification) the per-row
     // kernel shifts the rows into place as it loads them (1024 x 32003 bf16 RKL against such a
